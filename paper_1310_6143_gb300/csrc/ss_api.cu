@@ -969,7 +969,8 @@ ss_status build_tiles(ss_system *h) {
     h->ntiles = (int64_t)tiles.size();
     SS_CUDA(h, dalloc(h, (void **)&h->tiles, tiles.size() * sizeof(TileDesc)));
     SS_CUDA(h, dalloc(h, (void **)&h->sys_tiles, st.size() * sizeof(int32_t)));
-    SS_CUDA(h, dalloc(h, (void **)&h->partials, tiles.size() * kPartComps * sizeof(double)));
+    // (the alternative integrators cut a tile into up to kAltSub parts with a partial each)
+    SS_CUDA(h, dalloc(h, (void **)&h->partials, tiles.size() * kAltSub * kPartComps * sizeof(double)));
     SS_CUDA(h, cudaMemcpyAsync(h->tiles, tiles.data(), tiles.size() * sizeof(TileDesc), cudaMemcpyHostToDevice,
                                h->stream));
     SS_CUDA(h, cudaMemcpyAsync(h->sys_tiles, st.data(), st.size() * sizeof(int32_t), cudaMemcpyHostToDevice,
@@ -1772,12 +1773,6 @@ ss_status mc_upload_params(ss_system *h) {
     return SS_OK;
 }
 
-// The kernel variant the alternative integrators launch for these arguments.
-template <typename R>
-int alt_mode(const KArgs<R> &a) {
-    return a.ex ? 2 : (a.J_tensor || a.any_cubic) ? 1 : 0;  // rows, general, plain (as step_mode)
-}
-
 // A grid-stride grid capped at one wave of `per_sm` resident blocks on every SM: more blocks
 // than fit would leave a partial second wave running at low occupancy.
 int one_wave(const ss_system *h, int grid, int per_sm) {
@@ -1785,22 +1780,36 @@ int one_wave(const ss_system *h, int grid, int per_sm) {
     return per_sm > 0 && wave < grid ? (int)wave : grid;
 }
 
-// Midpoint steps: per step the midpoint launches (the first of which leaves the tile partials
-// of the record of the state at the start of the step, finalised into the ring at the
-// device's step) and the step counter.
+// Grids of the alternative integrators' launches (which = 0: midpoint iterations, 1: the
+// semi-implicit corrector).  The first pass takes the tiles whole when they give every resident
+// block six or more rounds, else in up to kAltSub parts of at least one block's spins: a
+// 512 x 512 x 16 film has 1,024 tiles of 4,096 spins, 1.7 rounds of the 608 resident blocks
+// (the second 68 % full); in quarters it runs 6.7.
+template <typename R>
+AltGrids alt_grids(const ss_system *h, int which) {
+    const int mode = step_mode(h);
+    AltGrids g{};
+    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((h->n + 255) / 256, (int64_t)h->sm_count * 8));
+    const int64_t wave = (int64_t)h->sm_count * std::max(1, alt_pass_blocks_per_sm<R>(2, mode));
+    g.sub = 1;
+    while (g.sub < kAltSub && h->ntiles * g.sub < 6 * wave && h->tile / (2 * g.sub) >= 256) g.sub *= 2;
+    g.len = (h->tile + g.sub - 1) / g.sub;
+    g.first = (int)std::max<int64_t>(1, std::min<int64_t>(h->ntiles * g.sub, wave));
+    g.second = one_wave(h, grid, alt_pass_blocks_per_sm<R>(which, mode));
+    g.nfin = h->nfin;
+    g.rows = h->rows ? rows_grid(h) : 0;
+    return g;
+}
+
+// Midpoint steps.
 template <typename R>
 cudaError_t enqueue_midpoint(ss_system *h, int64_t nsteps, int iterations) {
     KArgs<R> a = make_args<R>(h);
     use_rows(h, a);  // long rows: bare exchange sums from the row passes
     a.rows_bare = 1;
-    const int rgrid = h->rows ? rows_grid(h) : 0;
-    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((h->n + 255) / 256, (int64_t)h->sm_count * 8));
-    const int igrid = one_wave(h, grid, alt_pass_blocks_per_sm<R>(0, alt_mode(a)));
+    const AltGrids g = alt_grids<R>(h, 0);
     cudaError_t e = cudaSuccess;
-    for (int64_t k = 0; k < nsteps && e == cudaSuccess; ++k) {
-        e = launch_midpoint<R>(a, iterations, grid, igrid, rgrid, h->stream);
-        if (e == cudaSuccess) e = launch_advance_step(a.step, h->stream);
-    }
+    for (int64_t k = 0; k < nsteps && e == cudaSuccess; ++k) e = launch_midpoint<R>(a, iterations, g, h->stream);
     return e;
 }
 
@@ -1867,21 +1876,15 @@ ss_status integrate_with_demag(ss_system *h, int64_t n, int key, F enqueue, cons
     return SS_OK;
 }
 
-// Semi-implicit predictor-corrector steps: predictor (with the record's tile partials),
-// record, corrector, step counter.
+// Semi-implicit predictor-corrector steps.
 template <typename R>
 cudaError_t enqueue_sib(ss_system *h, int64_t nsteps) {
     KArgs<R> a = make_args<R>(h);
     use_rows(h, a);  // long rows: bare exchange sums from the row passes
     a.rows_bare = 1;
-    const int rgrid = h->rows ? rows_grid(h) : 0;
-    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((h->n + 255) / 256, (int64_t)h->sm_count * 8));
-    const int cgrid = one_wave(h, grid, alt_pass_blocks_per_sm<R>(1, alt_mode(a)));
+    const AltGrids g = alt_grids<R>(h, 1);
     cudaError_t e = cudaSuccess;
-    for (int64_t k = 0; k < nsteps && e == cudaSuccess; ++k) {
-        e = launch_sib<R>(a, grid, cgrid, rgrid, h->stream);
-        if (e == cudaSuccess) e = launch_advance_step(a.step, h->stream);
-    }
+    for (int64_t k = 0; k < nsteps && e == cudaSuccess; ++k) e = launch_sib<R>(a, g, h->stream);
     return e;
 }
 

@@ -239,18 +239,21 @@ template <typename R> cudaError_t launch_mc_colour(const KArgs<R> &a, const McAr
 template <typename R> int mc_blocks_per_sm(int block, int mode);  // mode: kPlain or kGeneral
 cudaError_t launch_advance_step(unsigned long long *step, cudaStream_t s);
 template <typename R> cudaError_t launch_demag(const KArgs<R> &a, const DemagArgs &d, cudaStream_t s);
-// One midpoint step's launches after its record: Euler predictor, `iters` fixed-point
-// iterations, copy back (the step counter is advanced separately).
-// (rgrid: grid of the long-row passes, used when a.ex is set)
-// (igrid: grid of the fixed-point iterations, at most one resident wave)
-template <typename R> cudaError_t launch_midpoint(const KArgs<R> &a, int iters, int grid, int igrid, int rgrid,
-                                                  cudaStream_t s);
-// One semi-implicit predictor-corrector step's launches after its record (predictor, corrector;
-// the step counter is advanced separately).
-// (cgrid: grid of the corrector, at most one resident wave)
-template <typename R> cudaError_t launch_sib(const KArgs<R> &a, int grid, int cgrid, int rgrid, cudaStream_t s);
-// Resident 256-thread blocks per SM of the midpoint iterations (which = 0) or of the
-// semi-implicit corrector (which = 1) in the kernel variant `mode`.
+// Grids of an alternative integrator's launches: the first pass works on the tiles cut into `sub`
+// parts of `len` spins; `second` (the midpoint iterations, the semi-implicit corrector) is at most
+// one resident wave, `nfin` blocks beside it sum the record; `rows` is the long-row passes' grid.
+struct AltGrids {
+    int first, sub, len, second, nfin, rows;
+};
+// Most parts of a tile (the partials buffer holds this many per tile).
+constexpr int kAltSub = 4;
+// One midpoint step's launches: Euler predictor, `iters` fixed-point iterations, record, step
+// counter.
+template <typename R> cudaError_t launch_midpoint(const KArgs<R> &a, int iters, const AltGrids &g, cudaStream_t s);
+// One semi-implicit predictor-corrector step's launches: predictor, corrector, record, step counter.
+template <typename R> cudaError_t launch_sib(const KArgs<R> &a, const AltGrids &g, cudaStream_t s);
+// Resident blocks per SM of the midpoint iterations (which = 0), the semi-implicit corrector (1)
+// or their first pass (2) in the kernel variant `mode`.
 template <typename R> int alt_pass_blocks_per_sm(int which, int mode);
 // Exchange + applied field of (X, Y, Z) into (a.ex, a.ey, a.ez), a warp per row (long rows).
 template <typename R>

@@ -697,11 +697,12 @@ __device__ __forceinline__ void write_record(const SysDesc &sd, double r, double
     __syncthreads();
 }
 
-// Sum the tile partials of system s in tile order and write one record (8 doubles).
+// Sum the tile partials of system s in tile order (sub partials per tile) and write one record
+// (8 doubles).
 template <int BS, bool Coherent, bool Chains4 = false>
 __device__ __forceinline__ void finalize_system(const SysDesc *sys, const int32_t *sys_tiles, const double *partials,
-                                                int s, double *dst, double *red) {
-    const int32_t t0 = sys_tiles[s], t1 = sys_tiles[s + 1];
+                                                int s, double *dst, double *red, int sub = 1) {
+    const int32_t t0 = sys_tiles[s] * sub, t1 = sys_tiles[s + 1] * sub;
     double acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
     if constexpr (Chains4) {
         // four independent chains per thread (tiles t, t + BS, t + 2 BS, t + 3 BS of each
@@ -1273,49 +1274,13 @@ __global__ void __launch_bounds__(256) k_rows_field(const KArgs<R> a, const R *X
 // held; nothing is renormalised (f(m) is perpendicular to m).
 // ----------------------------------------------------------------------------------
 
-// sum_j (J_ij / mu_s,i) X_j over row i (scalar or tensor bonds, kPlain: scalar only), without
-// the applied field; one FMA per bond and component in CSR order.
+// sum_j (J_ij / mu_s,i) X_j over row i without the applied field: the step kernels' exchange sum
+// (row forms when the handle has them, else the CSR; long rows from the row passes) started at
+// zero.
 template <typename R, int Mode>
 __device__ __forceinline__ void exchange_bare(const KArgs<R> &a, const R *X, const R *Y, const R *Z, int64_t i,
                                               R &e0, R &e1, R &e2) {
-    if constexpr (Mode == kRows) {  // long rows: summed beforehand (without H_app) by the row passes
-        e0 = a.ex[i];
-        e1 = a.ey[i];
-        e2 = a.ez[i];
-        return;
-    }
-    const int32_t b = __ldg(a.row_ptr + i);
-    const int32_t e = __ldg(a.row_ptr + i + 1);
-    R x = 0, y = 0, z = 0;
-    if (Mode != kPlain && a.J_tensor) {
-        for (int32_t k = b; k < e; ++k) {
-            const int32_t j = chk(__ldg(a.col + k), a.n, a.err);
-            const R m0 = X[j], m1 = Y[j], m2 = Z[j];
-            const R *t = a.Jt + 9 * (int64_t)__ldg(a.Jtidx + k);
-            x = fma(__ldg(t + 0), m0, fma(__ldg(t + 1), m1, fma(__ldg(t + 2), m2, x)));
-            y = fma(__ldg(t + 3), m0, fma(__ldg(t + 4), m1, fma(__ldg(t + 5), m2, y)));
-            z = fma(__ldg(t + 6), m0, fma(__ldg(t + 7), m1, fma(__ldg(t + 8), m2, z)));
-        }
-    } else if (a.J_uniform) {
-        const R Jk = a.J_value;
-        for (int32_t k = b; k < e; ++k) {
-            const int32_t j = chk(__ldg(a.col + k), a.n, a.err);
-            x = fma(Jk, X[j], x);
-            y = fma(Jk, Y[j], y);
-            z = fma(Jk, Z[j], z);
-        }
-    } else {
-        for (int32_t k = b; k < e; ++k) {
-            const int32_t j = chk(__ldg(a.col + k), a.n, a.err);
-            const R Jk = __ldg(a.J + k);
-            x = fma(Jk, X[j], x);
-            y = fma(Jk, Y[j], y);
-            z = fma(Jk, Z[j], z);
-        }
-    }
-    e0 = x;
-    e1 = y;
-    e2 = z;
+    exchange_sum_h<R, false, base_mode(Mode)>(a, (R)0, (R)0, (R)0, X, Y, Z, i, e0, e1, e2);
 }
 
 // ----------------------------------------------------------------------------------
@@ -1346,37 +1311,60 @@ __device__ __forceinline__ void sib_a(R gp, R lam, R v0, R v1, R v2, R H0, R H1,
     a2 = -gp * fma(lam, v0 * H1 - v1 * H0, H2);
 }
 
-// Threads per block of the first pass of the alternative integrators.
+// Threads per block of the passes of the alternative integrators.
 constexpr int kAltBlock = 256;
 
-// First pass of the alternative integrators, tile by tile: the step's thermal field (counters
-// as the Heun step), the part of the second pass's field that is fixed over the step,
+// Resident blocks per SM the FP32-mixed first pass is compiled for (64 registers a thread; the
+// FP64 one for two, 128 registers).
+constexpr int kAltFirstBlocks = 4;
+// and the FP32-mixed second passes (40 registers): they wait for the neighbours' loads, so
+// resident warps count for more than the loads each thread has in flight (the semi-implicit
+// corrector on a 512 x 512 x 16 film: 82 us at the compiler's own 64 registers).
+constexpr int kAltSecondBlocks = 6;
+
+// First pass of the alternative integrators: the step's thermal field (counters as the Heun
+// step), the part of the second pass's field that is fixed over the step,
 // C = H_app + H_th + (1/2) sum_j J_ij S_j (the exchange field is linear, so the field of
 // (S + X)/2 is C + (1/2) sum_j J_ij X_j plus the on-site terms), into (hx, hy, hz); the first new
 // spin into (px, py, pz): the semi-implicit predictor (Sib) or the Euler predictor of the
-// midpoint rule; and the tile partials of the record of S, the state at the start of the step.
+// midpoint rule; and the partials of the record of S, the state at the start of the step.
+//
+// The work is cut into units: unit u is part u % sub of tile u / sub, `len` spins of it, with a
+// partial of its own (those past the end of a short tile are zero), so that the Heun passes'
+// large tiles do not leave the last round of blocks half empty here.
+//
+// Bound by issue.  In the FP32-mixed form the Gaussians come from the double-float transform
+// (the FP64 transform's values rounded to float, bit for bit, as in the Heun passes) and the
+// record terms are summed as float pairs, so the FP64 pipe runs no per-spin work; with the FP64
+// transform and the CSR this pass took 239 us on a 512 x 512 x 16 film.
 template <typename R, int Mode, bool Sib>
-__device__ __forceinline__ void alt_first_pass(const KArgs<R> &a, const SmemTables &tab, double *red) {
+__device__ __forceinline__ void alt_first_pass(const KArgs<R> &a, const StepTabT<R> &tab, double *red, int sub,
+                                               int len) {
+    constexpr int BM = base_mode(Mode);
     const uint64_t step = *a.step;
-    for (int64_t t = blockIdx.x; t < a.ntiles; t += gridDim.x) {
+    for (int64_t u = blockIdx.x; u < a.ntiles * sub; u += gridDim.x) {
+        const int64_t t = u / sub;
+        const int k0 = (int)(u - t * sub) * len;
         const TileDesc td = a.tiles[t];
+        const int k1 = k0 + len < td.count ? k0 + len : td.count;
         const SysDesc &sd = a.sys[td.sys];
         const R sqrtT = sqrtT_of_step(a, step, sd);
         const R ha0 = sys_H(sd, 0, R()), ha1 = sys_H(sd, 1, R()), ha2 = sys_H(sd, 2, R());
-        double acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-        for (int k = threadIdx.x; k < td.count; k += kAltBlock) {
+        TermAcc<R> ta;
+        ta.reset();
+        for (int k = k0 + threadIdx.x; k < k1; k += kAltBlock) {
             const int64_t i = td.start + k;
-            const MatDesc<R> &m = a.mats[mat_of(a, i)];
+            const MatDesc<R> &m = mat_at<Mode>(a, i);
             R t0 = 0, t1 = 0, t2 = 0;
             if (sqrtT > (R)0) {
                 const R sig = m.sig * sqrtT;
                 const Philox4 w =
                     philox4x32_10((uint32_t)(i - sd.offset + sd.pbase), (uint32_t)step, sd.ctr2, 0u, sd.key0, sd.key1);
-                double g0, g1, g2;
-                box_muller3(w, tab, g0, g1, g2);
-                t0 = sig * narrow<R>(g0);
-                t1 = sig * narrow<R>(g1);
-                t2 = sig * narrow<R>(g2);
+                R g0, g1, g2;
+                thermal_gaussians(a, tab, w, g0, g1, g2);
+                t0 = sig * g0;
+                t1 = sig * g1;
+                t2 = sig * g2;
             }
             const R s0 = a.sx[i], s1 = a.sy[i], s2 = a.sz[i];
             R x0, x1, x2;
@@ -1386,12 +1374,17 @@ __device__ __forceinline__ void alt_first_pass(const KArgs<R> &a, const SmemTabl
             a.hy[i] = fma((R)0.5, x1, c1);
             a.hz[i] = fma((R)0.5, x2, c2);
             R H0, H1, H2;
-            const R sde = det_field<R, Mode != kPlain>(m, s0, s1, s2, x0 + c0, x1 + c1, x2 + c2, H0, H1, H2);
+            const R sde = det_field<R, BM != kPlain>(m, s0, s1, s2, x0 + c0, x1 + c1, x2 + c2, H0, H1, H2);
             if (a.demag) add_demag(a, i, H0, H1, H2);
-            double v[5];
-            spin_terms<R, Mode != kPlain>(m, s0, s1, s2, x0 + ha0, x1 + ha1, x2 + ha2, sde, v);
-#pragma unroll
-            for (int c = 0; c < 5; ++c) acc[c] += v[c];
+            if constexpr (sizeof(R) == 4) {
+                R v[5];
+                spin_terms_r<R, BM != kPlain>(m, s0, s1, s2, x0 + ha0, x1 + ha1, x2 + ha2, sde, v);
+                ta.add(v);
+            } else {
+                double v[5];
+                spin_terms<R, BM != kPlain>(m, s0, s1, s2, x0 + ha0, x1 + ha1, x2 + ha2, sde, v);
+                ta.add(v);
+            }
             R p0, p1, p2;
             if constexpr (Sib) {
                 R a0, a1, a2;
@@ -1408,79 +1401,118 @@ __device__ __forceinline__ void alt_first_pass(const KArgs<R> &a, const SmemTabl
             a.py[i] = p1;
             a.pz[i] = p2;
         }
+        double acc[8];
+        ta.out(acc);
         const double r = block_sum8<kAltBlock>(acc, red);
-        if (threadIdx.x < kPartComps) a.partials[t * kPartComps + threadIdx.x] = r;
+        if (threadIdx.x < kPartComps) a.partials[u * kPartComps + threadIdx.x] = r;
     }
 }
 
-// Midpoint rule, first pass: the Euler predictor X = S + dt f(S).
-template <typename R, int Mode>
-__global__ void __launch_bounds__(kAltBlock) k_mid_euler(const KArgs<R> a) {
-    __shared__ SmemTables tab;
+// The record of the step from the first pass's partials (sub per tile), by the blocks
+// [0, nfin) of a later pass's launch, beside that pass.
+template <typename R>
+__device__ __forceinline__ void alt_finalize(const KArgs<R> &a, int nfin, int sub) {
     __shared__ double red[(kAltBlock / 32) * 8];
-    stage_tables(a, tab);
+    const uint64_t step = *a.step;
+    for (int s = blockIdx.x; s < a.nsys; s += nfin) {
+        double *dst = a.rec + ((int64_t)(step % (uint64_t)a.rec_cap) * a.nsys + s) * kRecComps;
+        finalize_system<kAltBlock, false>(a.sys, a.sys_tiles, a.partials, s, dst, red, sub);
+    }
+}
+
+// The last block of a step's last launch advances the step counter (every block has read it).
+template <typename R>
+__device__ __forceinline__ void alt_advance(const KArgs<R> &a) {
     __syncthreads();
-    alt_first_pass<R, Mode, false>(a, tab, red);
+    if (threadIdx.x == 0) {
+        __threadfence();
+        const unsigned int done = atomicAdd(a.ticket, 1u);
+        if (done == gridDim.x - 1) {
+            *a.ticket = 0u;
+            *a.step += 1ull;
+            __threadfence();
+        }
+    }
+}
+
+// Midpoint rule, first pass: the Euler predictor X = S + dt f(S); semi-implicit predictor (Sib):
+// S' = S_n + (dt/2)(S_n + S') x A(S_n).
+template <typename R, int Mode, bool Sib>
+__global__ void __launch_bounds__(kAltBlock, sizeof(R) == 4 ? kAltFirstBlocks : 2)
+    k_alt_first(const KArgs<R> a, int sub, int len) {
+    __shared__ StepTabT<R> tab;
+    __shared__ double red[(kAltBlock / 32) * 8];
+    stage_step_tables(a, tab);
+    __syncthreads();
+    alt_first_pass<R, Mode, Sib>(a, tab, red, sub, len);
 }
 
 // One fixed-point iteration: Y = S + dt f(m), m = (S + X)/2, with the field C + (1/2) sum_j J_ij X_j
 // plus the on-site terms of m.  A thread reads S only at its own spin, so the last iteration
-// writes Y over S (Last: and flags non-finite spins).
+// writes Y over S (Last: and flags non-finite spins, and advances the step counter).  Blocks
+// [0, nfin) sum the step's record instead (the first iteration; nfin = 0 otherwise).
 template <typename R, int Mode, bool Last>
-__global__ void k_mid_iter(const KArgs<R> a, const R *xx, const R *xy, const R *xz, R *yx, R *yy, R *yz) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < a.n; i += (int64_t)gridDim.x * blockDim.x) {
-        const MatDesc<R> &m = a.mats[mat_of(a, i)];
-        const R s0 = a.sx[i], s1 = a.sy[i], s2 = a.sz[i];
-        const R m0 = (R)0.5 * (s0 + xx[i]), m1 = (R)0.5 * (s1 + xy[i]), m2 = (R)0.5 * (s2 + xz[i]);
-        R x0, x1, x2;
-        exchange_bare<R, Mode>(a, xx, xy, xz, i, x0, x1, x2);
-        R H0, H1, H2;
-        det_field<R, Mode != kPlain>(m, m0, m1, m2, fma((R)0.5, x0, a.hx[i]), fma((R)0.5, x1, a.hy[i]),
-                                     fma((R)0.5, x2, a.hz[i]), H0, H1, H2);
-        if (a.demag) add_demag(a, i, H0, H1, H2);
-        R d0, d1, d2;
-        llg_rhs(m.gp, m.lambda, m0, m1, m2, H0, H1, H2, d0, d1, d2);
-        const R v0 = fma(m.dt, d0, s0), v1 = fma(m.dt, d1, s1), v2 = fma(m.dt, d2, s2);
-        if (Last && bad_inv(v0 * v0 + v1 * v1 + v2 * v2)) atomicOr(a.err, kErrNonFinite);
-        yx[i] = v0;
-        yy[i] = v1;
-        yz[i] = v2;
+__global__ void __launch_bounds__(kAltBlock, sizeof(R) == 4 ? kAltSecondBlocks : 1)
+    k_mid_iter(const KArgs<R> a, const R *xx, const R *xy, const R *xz, R *yx, R *yy, R *yz, int nfin, int sub) {
+    constexpr int BM = base_mode(Mode);
+    if ((int)blockIdx.x < nfin) {
+        alt_finalize(a, nfin, sub);
+    } else {
+        const int64_t first = (int64_t)(blockIdx.x - nfin) * kAltBlock + threadIdx.x;
+        for (int64_t i = first; i < a.n; i += (int64_t)(gridDim.x - nfin) * kAltBlock) {
+            const MatDesc<R> &m = mat_at<Mode>(a, i);
+            const R s0 = a.sx[i], s1 = a.sy[i], s2 = a.sz[i];
+            const R m0 = (R)0.5 * (s0 + xx[i]), m1 = (R)0.5 * (s1 + xy[i]), m2 = (R)0.5 * (s2 + xz[i]);
+            R x0, x1, x2;
+            exchange_bare<R, Mode>(a, xx, xy, xz, i, x0, x1, x2);
+            R H0, H1, H2;
+            det_field<R, BM != kPlain>(m, m0, m1, m2, fma((R)0.5, x0, a.hx[i]), fma((R)0.5, x1, a.hy[i]),
+                                       fma((R)0.5, x2, a.hz[i]), H0, H1, H2);
+            if (a.demag) add_demag(a, i, H0, H1, H2);
+            R d0, d1, d2;
+            llg_rhs(m.gp, m.lambda, m0, m1, m2, H0, H1, H2, d0, d1, d2);
+            const R v0 = fma(m.dt, d0, s0), v1 = fma(m.dt, d1, s1), v2 = fma(m.dt, d2, s2);
+            if (Last && bad_inv(v0 * v0 + v1 * v1 + v2 * v2)) atomicOr(a.err, kErrNonFinite);
+            yx[i] = v0;
+            yy[i] = v1;
+            yz[i] = v2;
+        }
     }
+    if constexpr (Last) alt_advance(a);
 }
 
-// Semi-implicit predictor: S' = S_n + (dt/2)(S_n + S') x A(S_n), with the first-pass outputs above.
+// Semi-implicit corrector: A at Sb = (S + S')/2 with the field C + (1/2) sum_j J_ij S'_j plus the
+// on-site terms of Sb; the new spin overwrites S (a thread reads S only at its own spin).  Blocks
+// [0, nfin) sum the step's record; the last block advances the step counter.
 template <typename R, int Mode>
-__global__ void __launch_bounds__(kAltBlock) k_sib_pred(const KArgs<R> a) {
-    __shared__ SmemTables tab;
-    __shared__ double red[(kAltBlock / 32) * 8];
-    stage_tables(a, tab);
-    __syncthreads();
-    alt_first_pass<R, Mode, true>(a, tab, red);
-}
-
-// Corrector: A at Sb = (S + S')/2 with the field C + (1/2) sum_j J_ij S'_j plus the on-site
-// terms of Sb; the new spin overwrites S (a thread reads S only at its own spin).
-template <typename R, int Mode>
-__global__ void k_sib_corr(const KArgs<R> a) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < a.n; i += (int64_t)gridDim.x * blockDim.x) {
-        const MatDesc<R> &m = a.mats[mat_of(a, i)];
-        const R s0 = a.sx[i], s1 = a.sy[i], s2 = a.sz[i];
-        const R m0 = (R)0.5 * (s0 + a.px[i]), m1 = (R)0.5 * (s1 + a.py[i]), m2 = (R)0.5 * (s2 + a.pz[i]);
-        R x0, x1, x2;
-        exchange_bare<R, Mode>(a, a.px, a.py, a.pz, i, x0, x1, x2);
-        R H0, H1, H2;
-        det_field<R, Mode != kPlain>(m, m0, m1, m2, fma((R)0.5, x0, a.hx[i]), fma((R)0.5, x1, a.hy[i]),
-                                     fma((R)0.5, x2, a.hz[i]), H0, H1, H2);
-        if (a.demag) add_demag(a, i, H0, H1, H2);
-        R a0, a1, a2;
-        sib_a(m.gp, m.lambda, m0, m1, m2, H0, H1, H2, a0, a1, a2);
-        R v0, v1, v2;
-        sib_solve((R)0.5 * m.dt, s0, s1, s2, a0, a1, a2, v0, v1, v2);
-        if (bad_inv(v0 * v0 + v1 * v1 + v2 * v2)) atomicOr(a.err, kErrNonFinite);
-        a.sx[i] = v0;
-        a.sy[i] = v1;
-        a.sz[i] = v2;
+__global__ void __launch_bounds__(kAltBlock, sizeof(R) == 4 ? kAltSecondBlocks : 1)
+    k_sib_corr(const KArgs<R> a, int nfin, int sub) {
+    constexpr int BM = base_mode(Mode);
+    if ((int)blockIdx.x < nfin) {
+        alt_finalize(a, nfin, sub);
+    } else {
+        const int64_t first = (int64_t)(blockIdx.x - nfin) * kAltBlock + threadIdx.x;
+        for (int64_t i = first; i < a.n; i += (int64_t)(gridDim.x - nfin) * kAltBlock) {
+            const MatDesc<R> &m = mat_at<Mode>(a, i);
+            const R s0 = a.sx[i], s1 = a.sy[i], s2 = a.sz[i];
+            const R m0 = (R)0.5 * (s0 + a.px[i]), m1 = (R)0.5 * (s1 + a.py[i]), m2 = (R)0.5 * (s2 + a.pz[i]);
+            R x0, x1, x2;
+            exchange_bare<R, Mode>(a, a.px, a.py, a.pz, i, x0, x1, x2);
+            R H0, H1, H2;
+            det_field<R, BM != kPlain>(m, m0, m1, m2, fma((R)0.5, x0, a.hx[i]), fma((R)0.5, x1, a.hy[i]),
+                                       fma((R)0.5, x2, a.hz[i]), H0, H1, H2);
+            if (a.demag) add_demag(a, i, H0, H1, H2);
+            R a0, a1, a2;
+            sib_a(m.gp, m.lambda, m0, m1, m2, H0, H1, H2, a0, a1, a2);
+            R v0, v1, v2;
+            sib_solve((R)0.5 * m.dt, s0, s1, s2, a0, a1, a2, v0, v1, v2);
+            if (bad_inv(v0 * v0 + v1 * v1 + v2 * v2)) atomicOr(a.err, kErrNonFinite);
+            a.sx[i] = v0;
+            a.sy[i] = v1;
+            a.sz[i] = v2;
+        }
     }
+    alt_advance(a);
 }
 
 // ----------------------------------------------------------------------------------

@@ -290,96 +290,78 @@ cudaError_t launch_demag(const KArgs<R> &a, const DemagArgs &d, cudaStream_t s) 
     return cudaGetLastError();
 }
 
-// The first pass of the alternative integrators over the tiles, then the record of the state
-// at the start of the step from its tile partials.
-template <typename R>
-int alt_first_grid(const KArgs<R> &a, int grid) {
-    return (int)(a.ntiles < (int64_t)grid ? (a.ntiles > 0 ? a.ntiles : 1) : grid);
-}
-
-template <typename R, int Mode>
-cudaError_t launch_midpoint_mode(const KArgs<R> &a, int iters, int grid, int igrid, int rgrid, cudaStream_t s) {
-    cudaError_t e = Mode == kRows ? launch_rows_field<R>(a, a.sx, a.sy, a.sz, rgrid, s) : cudaSuccess;
-    if (e != cudaSuccess) return e;
-    k_mid_euler<R, Mode><<<alt_first_grid(a, grid), kAltBlock, 0, s>>>(a);
-    e = cudaGetLastError();
-    if (e == cudaSuccess)
-        e = launch_finalize_ring(a.sys, a.sys_tiles, a.nsys, a.partials, a.rec, a.rec_cap, a.step, s);
-    R *x[3] = {a.px, a.py, a.pz}, *y[3] = {a.qx, a.qy, a.qz};
-    for (int k = 0; k + 1 < iters && e == cudaSuccess; ++k) {
-        if (Mode == kRows && (e = launch_rows_field<R>(a, x[0], x[1], x[2], rgrid, s)) != cudaSuccess) break;
-        k_mid_iter<R, Mode, false><<<igrid, 256, 0, s>>>(a, x[0], x[1], x[2], y[0], y[1], y[2]);
-        e = cudaGetLastError();
-        for (int c = 0; c < 3; ++c) {
-            R *t = x[c];
-            x[c] = y[c];
-            y[c] = t;
-        }
+// Kernels in the variant of heun_mode.
+#define SS_ALT_SWITCH(mode, ...)                                   \
+    switch (mode) {                                                \
+        case kRows: { constexpr int M = kRows; __VA_ARGS__; } break;       \
+        case kGeneral: { constexpr int M = kGeneral; __VA_ARGS__; } break; \
+        case kUniform: { constexpr int M = kUniform; __VA_ARGS__; } break; \
+        default: { constexpr int M = kPlain; __VA_ARGS__; } break;         \
     }
-    if (e == cudaSuccess && Mode == kRows) e = launch_rows_field<R>(a, x[0], x[1], x[2], rgrid, s);
-    if (e == cudaSuccess) {  // the last iterate goes straight to S
-        k_mid_iter<R, Mode, true><<<igrid, 256, 0, s>>>(a, x[0], x[1], x[2], a.sx, a.sy, a.sz);
+
+// One midpoint step: the first pass, then the iterations, the first of which also sums the
+// step's record and the last of which advances the step counter.
+template <typename R>
+cudaError_t launch_midpoint(const KArgs<R> &a, int iters, const AltGrids &g, cudaStream_t s) {
+    const int mode = heun_mode(a);
+    cudaError_t e = mode == kRows ? launch_rows_field<R>(a, a.sx, a.sy, a.sz, g.rows, s) : cudaSuccess;
+    if (e != cudaSuccess) return e;
+    SS_ALT_SWITCH(mode, k_alt_first<R, M, false><<<g.first, kAltBlock, 0, s>>>(a, g.sub, g.len));
+    e = cudaGetLastError();
+    const R *x[3] = {a.px, a.py, a.pz};
+    R *y[3] = {a.qx, a.qy, a.qz}, *p[3] = {a.px, a.py, a.pz}, *q[3] = {a.qx, a.qy, a.qz};
+    for (int k = 0; k < iters && e == cudaSuccess; ++k) {
+        if (mode == kRows && (e = launch_rows_field<R>(a, x[0], x[1], x[2], g.rows, s)) != cudaSuccess) break;
+        const int nfin = k == 0 ? g.nfin : 0;
+        if (k + 1 < iters) {
+            SS_ALT_SWITCH(mode, k_mid_iter<R, M, false><<<g.second + nfin, kAltBlock, 0, s>>>(
+                                    a, x[0], x[1], x[2], y[0], y[1], y[2], nfin, g.sub));
+        } else {  // the last iterate goes straight to S
+            SS_ALT_SWITCH(mode, k_mid_iter<R, M, true><<<g.second + nfin, kAltBlock, 0, s>>>(
+                                    a, x[0], x[1], x[2], a.sx, a.sy, a.sz, nfin, g.sub));
+        }
         e = cudaGetLastError();
+        for (int c = 0; c < 3; ++c) {  // the iterates alternate between the two buffers
+            x[c] = k % 2 == 0 ? q[c] : p[c];
+            y[c] = k % 2 == 0 ? p[c] : q[c];
+        }
     }
     return e;
 }
 
-template <typename R>
-cudaError_t launch_midpoint(const KArgs<R> &a, int iters, int grid, int igrid, int rgrid, cudaStream_t s) {
-    if (a.ex) return launch_midpoint_mode<R, kRows>(a, iters, grid, igrid, rgrid, s);
-    return (a.J_tensor || a.any_cubic) ? launch_midpoint_mode<R, kGeneral>(a, iters, grid, igrid, rgrid, s)
-                                       : launch_midpoint_mode<R, kPlain>(a, iters, grid, igrid, rgrid, s);
-}
-
-// Resident 256-thread blocks per SM of the second-pass kernels of the alternative integrators
-// (which = 0: the midpoint iterations, the smaller of their two variants; 1: the semi-implicit
-// corrector) in the variant `mode` (kPlain, kGeneral or kRows); 0 if the query fails.
+// Resident kAltBlock-thread blocks per SM of the alternative integrators' kernels in the variant
+// `mode` (which = 0: the midpoint iterations, the smaller of their two variants; 1: the
+// semi-implicit corrector; 2: the first pass, the smaller of its two); 0 if the query fails.
 template <typename R>
 int alt_pass_blocks_per_sm(int which, int mode) {
     int n0 = 0, n1 = 0;
     cudaError_t e = cudaErrorInvalidValue;
-#define SS_OCC(MODE)                                                                              \
-    if (which == 0) {                                                                             \
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n0, k_mid_iter<R, MODE, false>, 256, 0); \
-        if (e == cudaSuccess)                                                                     \
-            e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n1, k_mid_iter<R, MODE, true>, 256, 0); \
-        n0 = n1 < n0 ? n1 : n0;                                                                   \
-    } else {                                                                                      \
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n0, k_sib_corr<R, MODE>, 256, 0);      \
-    }
-    if (mode == kRows) {
-        SS_OCC(kRows)
-    } else if (mode == kGeneral) {
-        SS_OCC(kGeneral)
+#define SS_OCC2(K0, K1)                                                                     \
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n0, K0, kAltBlock, 0);               \
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n1, K1, kAltBlock, 0);
+    if (which == 0) {
+        SS_ALT_SWITCH(mode, SS_OCC2((k_mid_iter<R, M, false>), (k_mid_iter<R, M, true>)));
+    } else if (which == 1) {
+        SS_ALT_SWITCH(mode, SS_OCC2((k_sib_corr<R, M>), (k_sib_corr<R, M>)));
     } else {
-        SS_OCC(kPlain)
+        SS_ALT_SWITCH(mode, SS_OCC2((k_alt_first<R, M, false>), (k_alt_first<R, M, true>)));
     }
-#undef SS_OCC
-    return e == cudaSuccess ? n0 : 0;
+#undef SS_OCC2
+    return e == cudaSuccess ? (n1 < n0 ? n1 : n0) : 0;
 }
 
+// One semi-implicit step: the predictor, then the corrector, which also sums the step's record
+// and advances the step counter.
 template <typename R>
-cudaError_t launch_sib(const KArgs<R> &a, int grid, int cgrid, int rgrid, cudaStream_t s) {
-    const int mode = a.ex ? kRows : (a.J_tensor || a.any_cubic) ? kGeneral : kPlain;
-    cudaError_t e = mode == kRows ? launch_rows_field<R>(a, a.sx, a.sy, a.sz, rgrid, s) : cudaSuccess;
+cudaError_t launch_sib(const KArgs<R> &a, const AltGrids &g, cudaStream_t s) {
+    const int mode = heun_mode(a);
+    cudaError_t e = mode == kRows ? launch_rows_field<R>(a, a.sx, a.sy, a.sz, g.rows, s) : cudaSuccess;
     if (e != cudaSuccess) return e;
-    if (mode == kRows)
-        k_sib_pred<R, kRows><<<alt_first_grid(a, grid), kAltBlock, 0, s>>>(a);
-    else if (mode == kGeneral)
-        k_sib_pred<R, kGeneral><<<alt_first_grid(a, grid), kAltBlock, 0, s>>>(a);
-    else
-        k_sib_pred<R, kPlain><<<alt_first_grid(a, grid), kAltBlock, 0, s>>>(a);
+    SS_ALT_SWITCH(mode, k_alt_first<R, M, true><<<g.first, kAltBlock, 0, s>>>(a, g.sub, g.len));
     e = cudaGetLastError();
-    if (e == cudaSuccess)
-        e = launch_finalize_ring(a.sys, a.sys_tiles, a.nsys, a.partials, a.rec, a.rec_cap, a.step, s);
-    if (e == cudaSuccess && mode == kRows) e = launch_rows_field<R>(a, a.px, a.py, a.pz, rgrid, s);
+    if (e == cudaSuccess && mode == kRows) e = launch_rows_field<R>(a, a.px, a.py, a.pz, g.rows, s);
     if (e != cudaSuccess) return e;
-    if (mode == kRows)
-        k_sib_corr<R, kRows><<<cgrid, 256, 0, s>>>(a);
-    else if (mode == kGeneral)
-        k_sib_corr<R, kGeneral><<<cgrid, 256, 0, s>>>(a);
-    else
-        k_sib_corr<R, kPlain><<<cgrid, 256, 0, s>>>(a);
+    SS_ALT_SWITCH(mode, k_sib_corr<R, M><<<g.second + g.nfin, kAltBlock, 0, s>>>(a, g.nfin, g.sub));
     return cudaGetLastError();
 }
 
@@ -475,8 +457,8 @@ template cudaError_t launch_mc_colour_rec<SS_REAL>(const KArgs<SS_REAL> &, const
 template cudaError_t launch_mc_colour_warp<SS_REAL>(const KArgs<SS_REAL> &, const McArgs &, int, cudaStream_t);
 template cudaError_t launch_mc_prep<SS_REAL>(const KArgs<SS_REAL> &, const McArgs &, cudaStream_t);
 template int mc_blocks_per_sm<SS_REAL>(int, int);
-template cudaError_t launch_midpoint<SS_REAL>(const KArgs<SS_REAL> &, int, int, int, int, cudaStream_t);
-template cudaError_t launch_sib<SS_REAL>(const KArgs<SS_REAL> &, int, int, int, cudaStream_t);
+template cudaError_t launch_midpoint<SS_REAL>(const KArgs<SS_REAL> &, int, const AltGrids &, cudaStream_t);
+template cudaError_t launch_sib<SS_REAL>(const KArgs<SS_REAL> &, const AltGrids &, cudaStream_t);
 template int alt_pass_blocks_per_sm<SS_REAL>(int, int);
 #endif
 
