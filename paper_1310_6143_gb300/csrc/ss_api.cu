@@ -91,9 +91,11 @@ struct ss_system {
     int mat_bytes = 4;
     void *J = nullptr, *mats = nullptr;
     void *state[12] = {};  // sx sy sz px py pz qx qy qz hx hy hz
+    void *packed = nullptr;  // float4 S, S' and half step + field x, float2 field y, z (FP32-mixed runs of steps;
+                             // nullptr: not available, the steps work on the arrays of `state`)
     void *ahead[3] = {};   // Gaussians drawn ahead by the corrector (FP32-mixed only)
     int pre_slot = 1 << 30;
-    int ahead_q = 6;       // eighths of each tile drawn ahead by the corrector
+    int ahead_q = 5;       // eighths of each tile drawn ahead by the corrector
     bool J_uniform = false;  // every bond has the same J_ij / mu_s,i (J_value)
     bool J_tensor = false;   // bonds carry exchange tensors (Jt dictionary, Jtidx per bond)
     bool any_cubic = false;  // some material has cubic anisotropy
@@ -535,6 +537,10 @@ KArgs<R> make_args(const ss_system *h) {
     a.px = s[3]; a.py = s[4]; a.pz = s[5];
     a.qx = s[6]; a.qy = s[7]; a.qz = s[8];
     a.hx = s[9]; a.hy = s[10]; a.hz = s[11];
+    a.s4 = static_cast<float4 *>(h->packed);
+    a.p4 = a.s4 ? a.s4 + h->n : nullptr;
+    a.qh4 = a.s4 ? a.s4 + 2 * h->n : nullptr;
+    a.qh2 = a.s4 ? reinterpret_cast<float2 *>(a.s4 + 3 * h->n) : nullptr;
     a.gx = static_cast<R *>(h->ahead[0]);
     a.gy = static_cast<R *>(h->ahead[1]);
     a.gz = static_cast<R *>(h->ahead[2]);
@@ -648,6 +654,49 @@ int split_grid(const ss_system *h, int which) {
     return (int)std::max<int64_t>(1, std::min<int64_t>(h->ntiles, g));
 }
 
+// Runs of at least this many steps work on float4 spins: packing and unpacking the state moves
+// 84 bytes per spin (0.24 ms on the 1024 x 1024 x 16 film), and a step over float4 spins saves
+// about 0.07 ms there.
+constexpr int64_t kPackedMin = 4;
+
+// Whether a run of n steps in the graph or plain-launch mode works on float4 spins: FP32-mixed,
+// not a slab (its halo refresh reads S'), not the split step (the Gaussians come in arrays), and
+// with long rows only the packed-bond pass, which reads float4 spins itself.
+bool packed_run(const ss_system *h, int64_t n) {
+    return h->packed && n >= kPackedMin && !split_step(h) && (!h->rows || h->sell);
+}
+
+int packed_grid(const ss_system *h, int which) {
+    const int64_t g = (int64_t)h->sm_count * std::max(1, packed_blocks_per_sm<float>(h->block, step_mode(h), which));
+    return (int)std::max<int64_t>(1, std::min<int64_t>(h->ntiles, g));
+}
+
+// One step of a run over float4 spins.
+template <typename R>
+cudaError_t enqueue_packed_step(const ss_system *h, const KArgs<R> &a, int gp, int gc, int gr) {
+    KArgs<R> r = a;  // the long-row pass gathers from x4
+    cudaError_t e = cudaSuccess;
+    if (h->rows) {
+        r.x4 = reinterpret_cast<R *>(a.s4);
+        e = launch_rows_field<R>(r, nullptr, nullptr, nullptr, gr, h->stream);
+    }
+    if (e == cudaSuccess) e = launch_predictor4<R>(a, h->block, gp, h->stream);
+    if (e == cudaSuccess && h->rows) {
+        r.x4 = reinterpret_cast<R *>(a.p4);
+        e = launch_rows_field<R>(r, nullptr, nullptr, nullptr, gr, h->stream);
+    }
+    if (e == cudaSuccess) e = launch_corrector4<R>(a, h->block, gc, h->nfin, h->stream);
+    return e;
+}
+
+// S into float4 spins before the run, S and S' back into their arrays after it.
+cudaError_t packed_state(const ss_system *h, bool pack) {
+    if (h->precision != SS_FP32_MIXED) return cudaErrorInvalidValue;
+    const KArgs<float> a = make_args<float>(h);
+    const int grid = (int)std::min<int64_t>((h->n + 255) / 256, (int64_t)h->sm_count * 8);
+    return pack ? launch_pack_state<float>(a, grid, h->stream) : launch_unpack_state<float>(a, grid, h->stream);
+}
+
 int persistent_grid(const ss_system *h) {
     const int mode = own_rows_mode(h) == 0 && h->nmat == 1 ? 3 : own_rows_mode(h);
     const int per_sm = h->precision == SS_FP32_MIXED ? persistent_blocks_per_sm<float>(h->block, mode)
@@ -657,9 +706,17 @@ int persistent_grid(const ss_system *h) {
 }
 
 template <typename R>
-cudaError_t enqueue_steps_kernels(ss_system *h, int64_t n) {
+cudaError_t enqueue_steps_kernels(ss_system *h, int64_t n, bool packed) {
     KArgs<R> a = make_args<R>(h);
     use_rows(h, a);
+    if constexpr (sizeof(R) == 4) {
+        if (packed) {
+            const int gp = packed_grid(h, 0), gc = packed_grid(h, 1), gr = h->rows ? rows_grid(h) : 0;
+            cudaError_t e = cudaSuccess;
+            for (int64_t k = 0; k < n && e == cudaSuccess; ++k) e = enqueue_packed_step<R>(h, a, gp, gc, gr);
+            return e;
+        }
+    }
     if (split_step(h)) {
         const int gg = split_grid(h, 0), gp = split_grid(h, 1), gc = split_grid(h, 2);
         if (n <= 0) return cudaSuccess;
@@ -728,8 +785,10 @@ cudaError_t enqueue_persistent(ss_system *h, int64_t n) {
     return cudaSuccess;
 }
 
-cudaError_t enqueue_kernels(ss_system *h, int64_t n) {
-    return h->precision == SS_FP32_MIXED ? enqueue_steps_kernels<float>(h, n) : enqueue_steps_kernels<double>(h, n);
+// (packed: the steps of a run over float4 spins, between the two packed_state calls)
+cudaError_t enqueue_kernels(ss_system *h, int64_t n, bool packed) {
+    return h->precision == SS_FP32_MIXED ? enqueue_steps_kernels<float>(h, n, packed)
+                                         : enqueue_steps_kernels<double>(h, n, packed);
 }
 
 template <typename R>
@@ -894,7 +953,7 @@ cudaError_t ensure_graph(ss_system *h) {
     cudaGraph_t graph = nullptr;
     cudaError_t e = cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal);
     if (e != cudaSuccess) return e;
-    cudaError_t ek = enqueue_kernels(h, g);
+    cudaError_t ek = enqueue_kernels(h, g, packed_run(h, g));
     e = cudaStreamEndCapture(h->stream, &graph);
     if (ek != cudaSuccess) {
         if (graph) cudaGraphDestroy(graph);
@@ -1282,6 +1341,41 @@ ss_status set_rows(ss_system *h, int32_t mode) {
     return SS_OK;
 }
 
+// The default launch shape.  Block: the FP32-mixed kernels are compiled for more resident warps in
+// 512-thread blocks and for more registers in smaller ones (heun_blocks); short rows of a single
+// material are faster in the former from about a million spins on, everything else in the
+// latter.  FP64: 512 threads for large systems.
+// Spins per thread: the resident blocks take the tiles round by round, so a pass takes the rounds
+// times the spins per thread (and about 0.3 spins' time for each tile's reduction); the count, up
+// to 12, that makes this least.  fcc 64^3 in FP32-mixed form: two spins per thread are 4.5
+// rounds of 456 blocks, run as five; nine are one round exactly (66.2 -> 59.7 us per step).  From
+// 12 rounds of eight spins per thread on there is little to round off, and eight are as fast as any.
+void default_shape(ss_system *h) {
+    const bool mixed = h->precision == SS_FP32_MIXED;
+    const bool short_uniform = h->nmat == 1 && h->max_row <= kShortRow && !h->J_tensor && !h->any_cubic;
+    h->block = (mixed ? short_uniform && h->n >= (int64_t(1) << 20) : h->n >= (int64_t(1) << 22)) ? 512 : 256;
+    const int64_t resident = (int64_t)std::max(h->sm_count, 1) * (mixed ? (h->block == 512 ? 2 : 3) : 1);
+    int best = 8;
+    double least = 1e300;
+    for (int slots = 1; slots <= 12; ++slots) {
+        const int64_t tile = (int64_t)slots * h->block;
+        int64_t tiles = 0;
+        for (int64_t n : h->sys_n) tiles += (n + tile - 1) / tile;
+        const int64_t rounds = (tiles + resident - 1) / resident;
+        const double cost = (double)rounds * (slots + 0.3);
+        if (cost < least) {
+            least = cost;
+            best = slots;
+        }
+        if (slots == 8 && tiles >= 12 * resident) {
+            best = 8;
+            break;
+        }
+    }
+    h->tile = best * h->block;
+    h->ahead_q = 5;
+}
+
 // A slab's owned range and Philox base, passed from spin_slab_create to create_impl.
 struct SlabInit {
     int64_t n_own;                   // owned spins (the first n_own of the local arrays)
@@ -1398,22 +1492,16 @@ ss_status create_impl(const ss_params *systems, int32_t count, ss_system **out, 
         return cleanup(cuda_fail(h, e, "cudaMalloc"));
     st = h->precision == SS_FP32_MIXED ? upload_system<float>(h, hs) : upload_system<double>(h, hs);
     if (st != SS_OK) return cleanup(st);
-    // Launch shape: 512-thread blocks for large systems; spins per thread (a power of two,
-    // at most 8) chosen so that there are about eight tiles per resident block.
-    h->block = n >= (int64_t(1) << 22) ? 512 : 256;
-    {
-        int64_t spt = n / ((int64_t)std::max(h->sm_count, 1) * 8 * h->block);
-        int slots = 1;
-        while (slots < 8 && 2 * slots <= spt) slots *= 2;
-        h->tile = slots * h->block;
-        h->ahead_q = slots >= 8 ? 4 : 6;  // the faster split on GB300 for each case
-        if (slab) h->ahead_q = 0;         // a slab's passes draw their own Gaussians
-    }
+    default_shape(h);
+    if (slab) h->ahead_q = 0;  // a slab's passes draw their own Gaussians
     st = build_tiles(h);
     if (st == SS_OK) st = set_rows(h, slab ? 1 : 0);  // a slab's passes sum a row per thread
     if (st != SS_OK) return cleanup(st);
     st = h->precision == SS_FP32_MIXED ? init_random<float>(h, hs) : init_random<double>(h, hs);
     if (st != SS_OK) return cleanup(st);
+    if (h->precision == SS_FP32_MIXED && !slab &&
+        dalloc(h, &h->packed, (size_t)n * (3 * sizeof(float4) + sizeof(float2))) != cudaSuccess)
+        cudaGetLastError();  // not enough memory: the steps work on the arrays of `state`
     *out = h;
     return SS_OK;
 }
@@ -2138,6 +2226,8 @@ static ss_status advance_steps(ss_system *h, int64_t n) {
     } else if (mode == SS_EXEC_GRAPH) {
         mode = SS_EXEC_KERNELS;
     }
+    const bool packed = (mode == SS_EXEC_GRAPH || mode == SS_EXEC_KERNELS) && packed_run(h, n);
+    if (packed && (e = packed_state(h, true)) != cudaSuccess) return cuda_fail(h, e, "step launch");
     if (mode == SS_EXEC_GRAPH) {
         int64_t left = n;
         while (left >= h->graph_steps) {
@@ -2145,7 +2235,7 @@ static ss_status advance_steps(ss_system *h, int64_t n) {
             if (e != cudaSuccess) return cuda_fail(h, e, "cudaGraphLaunch");
             left -= h->graph_steps;
         }
-        e = enqueue_kernels(h, left);
+        e = enqueue_kernels(h, left, packed);
     } else if (mode == SS_EXEC_SYSTEM_BLOCKS) {
         e = enqueue_sysblocks(h, n);
     } else if (mode == SS_EXEC_CLUSTER) {
@@ -2169,8 +2259,9 @@ static ss_status advance_steps(ss_system *h, int64_t n) {
             return fail(h, SS_ERR_UNSUPPORTED, "persistent launch not possible: %s", cudaGetErrorString(e));
         }
     } else {
-        e = enqueue_kernels(h, n);
+        e = enqueue_kernels(h, n, packed);
     }
+    if (e == cudaSuccess && packed) e = packed_state(h, false);
     if (e != cudaSuccess) return cuda_fail(h, e, "step launch");
     h->step += n;
     return SS_OK;
@@ -2809,7 +2900,7 @@ ss_status spin_system_autotune(ss_system *h, int32_t trial_steps, ss_info *out_i
     for (int c = 0; c < 3; ++c)
         SS_CUDA(h, cudaMemcpyAsync((char *)save + c * n * rs, h->state[c], n * rs, cudaMemcpyDeviceToDevice, h->stream));
     struct Cand { int exec, block, tile, ahead, gauss; };
-    std::vector<Cand> cands;
+    std::vector<Cand> cands{{SS_EXEC_GRAPH, h->block, h->tile, h->ahead_q, 0}};  // the shape in force
     const bool mixed = h->precision == SS_FP32_MIXED;
     // 128-thread blocks, with up to four spins per thread, for systems of at most 4,096 spins
     // per SM: a small system spread over twice the SMs has twice the FP64 lanes for its thermal

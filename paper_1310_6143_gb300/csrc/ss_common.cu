@@ -87,27 +87,15 @@ __global__ void k_debug_gaussians_ff(uint64_t seed, uint32_t sys, uint32_t step,
             v[1] = g1;
             v[2] = g2;
         } else {
-            const FF R1 = ff_sqrt(ff_neg2log(w.w0, tab));
-            const FF R2 = ff_sqrt(ff_neg2log(w.w2, tab));
             float g[3];
             const bool ok = box_muller3_ff(w, tab, g[0], g[1], g[2]);
             if (mode == 4) {
                 v[0] = ok ? 0.0 : 1.0;
             } else {
                 // the unrounded double-float products, as box_muller3_ff forms them
-                const FFTurn a = ff_turn(w.w1, tab);
-                const FF sb = ff_rot(a.tv.x, a.tv.y, a.tv.z, a.tv.w, a);
-                const FF cb = ff_rot(a.tv.z, a.tv.w, -a.tv.x, -a.tv.y, a);
-                const bool swap = ((a.o + 1u) >> 1) & 1u;
-                FF S = swap ? cb : sb, Co = swap ? sb : cb;
-                if (a.o & 4u) S = ff_neg(S);
-                if ((a.o + 2u) & 4u) Co = ff_neg(Co);
-                const FFTurn b = ff_turn(w.w3, tab);
-                const bool swap2 = ((b.o + 1u) >> 1) & 1u;
-                FF C2 = swap2 ? ff_rot(b.tv.x, b.tv.y, b.tv.z, b.tv.w, b)
-                              : ff_rot(b.tv.z, b.tv.w, -b.tv.x, -b.tv.y, b);
-                if ((b.o + 2u) & 4u) C2 = ff_neg(C2);
-                const FF R[3] = {R1, R1, R2}, V[3] = {Co, S, C2};
+                const FFFactors q = ff_factors(w, tab);
+                const FF R[3] = {{q.R.hi.x, q.R.lo.x}, {q.R.hi.x, q.R.lo.x}, {q.R.hi.y, q.R.lo.y}};
+                const FF V[3] = {{q.V.hi.x, q.V.lo.x}, {q.V.hi.y, q.V.lo.y}, q.C2};
                 for (int c = 0; c < 3; ++c) {
                     const float gh = __fmul_rn(R[c].hi, V[c].hi);
                     const float ge = __fadd_rn(fmaf(R[c].hi, V[c].hi, -gh), fmaf(R[c].hi, V[c].lo, __fmul_rn(R[c].lo, V[c].hi)));
@@ -181,8 +169,8 @@ void build_ff_tables(float4 *t) {
     for (int m = 0; m < kTrigTab; ++m) {
         const long double a = twopi * (long double)m / 4096.0L;  // first octant of 4096 points
         float4 &e = t[kLogTab + m];
-        split(sinl(a), e.x, e.y);
-        split(cosl(a), e.z, e.w);
+        split(sinl(a), e.x, e.z);
+        split(cosl(a), e.y, e.w);
     }
     const long double ln2 = 0.693147180559945309417232121458176568L;
     float *l2 = reinterpret_cast<float *>(t + kLogTab + kTrigTab);

@@ -131,6 +131,9 @@ struct KArgs {
     R *px, *py, *pz;          // S' (predictor, renormalised)
     R *qx, *qy, *qz;          // S + dt/2 dS (predictor half step)
     R *hx, *hy, *hz;          // thermal field of the current step
+    float4 *s4, *p4;          // S and S' as (x, y, z, 0) per spin while a run of FP32-mixed steps
+    float4 *qh4;              // keeps them so (launch_pack_state .. launch_unpack_state); the half
+    float2 *qh2;              // step and the thermal field's x, then its y and z
     R *gx, *gy, *gz;          // Gaussians of the next step drawn by the corrector (FP32-mixed);
                               // the split step's Gaussians of even steps
     R *g2x, *g2y, *g2z;       // the split step's Gaussians of odd steps (FP32-mixed)
@@ -209,6 +212,13 @@ void set_global_error(const char *msg);
 // Launchers (ss_kernels_f32.cu / ss_kernels_f64.cu).
 template <typename R> cudaError_t launch_predictor(const KArgs<R> &a, int block, int grid, cudaStream_t s);
 template <typename R> cudaError_t launch_corrector(const KArgs<R> &a, int block, int grid, int nfin, cudaStream_t s);
+// The same passes over float4 spins (FP32-mixed): a run of steps packs the state first and
+// unpacks S and S' last.
+template <typename R> cudaError_t launch_predictor4(const KArgs<R> &a, int block, int grid, cudaStream_t s);
+template <typename R> cudaError_t launch_corrector4(const KArgs<R> &a, int block, int grid, int nfin, cudaStream_t s);
+template <typename R> int packed_blocks_per_sm(int block, int mode, int which);
+template <typename R> cudaError_t launch_pack_state(const KArgs<R> &a, int grid, cudaStream_t s);
+template <typename R> cudaError_t launch_unpack_state(const KArgs<R> &a, int grid, cudaStream_t s);
 template <typename R> cudaError_t launch_measure(const KArgs<R> &a, int block, int grid, cudaStream_t s);
 // The split FP32-mixed step: the Gaussian pass, then the Heun passes reading it (FP32 only).
 template <typename R> cudaError_t launch_gauss(const KArgs<R> &a, int block, int grid, cudaStream_t s, int priority);

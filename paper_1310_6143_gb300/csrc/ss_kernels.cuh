@@ -146,19 +146,45 @@ __device__ __forceinline__ int32_t chk(int64_t j, int64_t n, unsigned int *err) 
     return (int32_t)j;
 }
 
-template <typename R, bool Coherent, int Mode = kGeneral>
-__device__ __forceinline__ void exchange_sum_h(const KArgs<R> &a, R hx, R hy, R hz, const R *X, const R *Y,
-                                               const R *Z, int64_t i, R &e0, R &e1, R &e2);
+// The spins an exchange sum gathers: three arrays, or one float4 (x, y, z, 0) per spin, which is
+// one load and one address per neighbour instead of three.
+template <typename R, bool Coherent>
+struct Soa {
+    const R *X, *Y, *Z;
+    __device__ __forceinline__ void get(int64_t j, R &x, R &y, R &z) const {
+        x = ld<Coherent>(X + j);
+        y = ld<Coherent>(Y + j);
+        z = ld<Coherent>(Z + j);
+    }
+};
+struct Aos {
+    const float4 *V;
+    __device__ __forceinline__ void get(int64_t j, float &x, float &y, float &z) const {
+        const float4 v = __ldg(V + j);
+        x = v.x;
+        y = v.y;
+        z = v.z;
+    }
+};
+
+// The row form of spin i (0 when the handle reads the CSR).
+template <typename R>
+__device__ __forceinline__ int form_of(const KArgs<R> &a, int64_t i) {
+    if (!a.pat) return 0;
+    return a.pat_wide ? (int)__ldg(reinterpret_cast<const uint16_t *>(a.pat) + i) : (int)__ldg(a.pat + i);
+}
+
+template <typename R, bool Coherent, int Mode, typename Src>
+__device__ __forceinline__ void exchange_sum_h(const KArgs<R> &a, R hx, R hy, R hz, const Src &S, int64_t i, int form,
+                                               R &e0, R &e1, R &e2);
 
 // The exchange sum of a row stored as a row pattern (NS slots: kShortRow or kPatRow): the
 // pattern's offsets and length come as vector loads, every slot is summed, and the slots past
 // the row's end carry the spin's own index and J = 0, adding exact zeros after the row's CSR
 // terms (so the sum is the CSR sum).
-template <typename R, bool Coherent, int NS>
-__device__ __forceinline__ void pattern_sum(const KArgs<R> &a, const R *X, const R *Y, const R *Z, int64_t i, R &x,
-                                            R &y, R &z) {
+template <typename R, int NS, typename Src>
+__device__ __forceinline__ void pattern_sum(const KArgs<R> &a, const Src &S, int64_t i, int p, R &x, R &y, R &z) {
     constexpr int W = NS == kShortRow ? 8 : 16;
-    const int p = a.pat_wide ? (int)__ldg(reinterpret_cast<const uint16_t *>(a.pat) + i) : (int)__ldg(a.pat + i);
     int32_t off[W];
     const int4 *row = reinterpret_cast<const int4 *>(a.pat_off) + (int64_t)p * (W / 4);
 #pragma unroll
@@ -182,27 +208,28 @@ __device__ __forceinline__ void pattern_sum(const KArgs<R> &a, const R *X, const
 #pragma unroll
     for (int q = 0; q < NS; ++q) {
         const int32_t j = chk((int64_t)ii + off[q], a.n, a.err);
-        x = fma(Jr[q], ld<Coherent>(X + j), x);
-        y = fma(Jr[q], ld<Coherent>(Y + j), y);
-        z = fma(Jr[q], ld<Coherent>(Z + j), z);
+        R sx, sy, sz;
+        S.get(j, sx, sy, sz);
+        x = fma(Jr[q], sx, x);
+        y = fma(Jr[q], sy, y);
+        z = fma(Jr[q], sz, z);
     }
 }
 
 template <typename R, bool Coherent, int Mode = kGeneral>
 __device__ __forceinline__ void exchange_sum(const KArgs<R> &a, const SysDesc &sd, const R *X, const R *Y,
                                              const R *Z, int64_t i, R &e0, R &e1, R &e2) {
-    exchange_sum_h<R, Coherent, Mode>(a, sys_H(sd, 0, R()), sys_H(sd, 1, R()), sys_H(sd, 2, R()), X, Y, Z, i, e0,
-                                      e1, e2);
+    exchange_sum_h<R, Coherent, Mode>(a, sys_H(sd, 0, R()), sys_H(sd, 1, R()), sys_H(sd, 2, R()),
+                                      Soa<R, Coherent>{X, Y, Z}, i, form_of(a, i), e0, e1, e2);
 }
 
 // The exchange sum of a row of tensor bonds stored as a row pattern: the form's offsets, length
 // and tensor entries come as vector loads, and the row's bonds (the slots before its length)
 // are summed as the CSR loop sums them, the tensor of bond k applied to S_j.
-template <typename R, bool Coherent, int NS>
-__device__ __forceinline__ void pattern_sum_tensor(const KArgs<R> &a, const R *X, const R *Y, const R *Z, int64_t i,
-                                                   R &x, R &y, R &z) {
+template <typename R, int NS, typename Src>
+__device__ __forceinline__ void pattern_sum_tensor(const KArgs<R> &a, const Src &S, int64_t i, int p, R &x, R &y,
+                                                   R &z) {
     constexpr int W = NS == kShortRow ? 8 : 16;
-    const int p = a.pat_wide ? (int)__ldg(reinterpret_cast<const uint16_t *>(a.pat) + i) : (int)__ldg(a.pat + i);
     int32_t off[W], tid[W];
     const int4 *row = reinterpret_cast<const int4 *>(a.pat_off) + (int64_t)p * (W / 4);
     // the form's Jt entries: W int32 at the start of its W * sizeof(R) bytes of pat_J
@@ -226,7 +253,8 @@ __device__ __forceinline__ void pattern_sum_tensor(const KArgs<R> &a, const R *X
         if (q < len) {
             const int32_t j = chk((int64_t)ii + off[q], a.n, a.err);
             const R *t = a.Jt + 9 * (int64_t)tid[q];
-            const R sx = ld<Coherent>(X + j), sy = ld<Coherent>(Y + j), sz = ld<Coherent>(Z + j);
+            R sx, sy, sz;
+            S.get(j, sx, sy, sz);
             x = fma(__ldg(t + 0), sx, fma(__ldg(t + 1), sy, fma(__ldg(t + 2), sz, x)));
             y = fma(__ldg(t + 3), sx, fma(__ldg(t + 4), sy, fma(__ldg(t + 5), sz, y)));
             z = fma(__ldg(t + 6), sx, fma(__ldg(t + 7), sy, fma(__ldg(t + 8), sz, z)));
@@ -235,10 +263,10 @@ __device__ __forceinline__ void pattern_sum_tensor(const KArgs<R> &a, const R *X
 }
 
 // The sum started at the system's applied field (hx, hy, hz), passed in by callers that hold
-// it in registers for a whole tile.
-template <typename R, bool Coherent, int Mode>
-__device__ __forceinline__ void exchange_sum_h(const KArgs<R> &a, R hx, R hy, R hz, const R *X, const R *Y,
-                                               const R *Z, int64_t i, R &e0, R &e1, R &e2) {
+// it in registers for a whole tile, as is the spin's row form (form_of).
+template <typename R, bool Coherent, int Mode, typename Src>
+__device__ __forceinline__ void exchange_sum_h(const KArgs<R> &a, R hx, R hy, R hz, const Src &S, int64_t i, int form,
+                                               R &e0, R &e1, R &e2) {
     if constexpr (Mode == kRows) {  // long rows: summed beforehand by k_rows_sell / k_rows_field
         e0 = ld<Coherent>(a.ex + i);
         e1 = ld<Coherent>(a.ey + i);
@@ -248,9 +276,9 @@ __device__ __forceinline__ void exchange_sum_h(const KArgs<R> &a, R hx, R hy, R 
     R x = hx, y = hy, z = hz;
     if (a.pat && !(Mode == kGeneral && a.J_tensor)) {
         if (a.pat_w == 8)
-            pattern_sum<R, Coherent, kShortRow>(a, X, Y, Z, i, x, y, z);
+            pattern_sum<R, kShortRow>(a, S, i, form, x, y, z);
         else
-            pattern_sum<R, Coherent, kPatRow>(a, X, Y, Z, i, x, y, z);
+            pattern_sum<R, kPatRow>(a, S, i, form, x, y, z);
         e0 = x;
         e1 = y;
         e2 = z;
@@ -258,9 +286,9 @@ __device__ __forceinline__ void exchange_sum_h(const KArgs<R> &a, R hx, R hy, R 
     }
     if (Mode == kGeneral && a.J_tensor && a.pat) {
         if (a.pat_w == 8)
-            pattern_sum_tensor<R, Coherent, kShortRow>(a, X, Y, Z, i, x, y, z);
+            pattern_sum_tensor<R, kShortRow>(a, S, i, form, x, y, z);
         else
-            pattern_sum_tensor<R, Coherent, kPatRow>(a, X, Y, Z, i, x, y, z);
+            pattern_sum_tensor<R, kPatRow>(a, S, i, form, x, y, z);
         e0 = x;
         e1 = y;
         e2 = z;
@@ -272,7 +300,8 @@ __device__ __forceinline__ void exchange_sum_h(const KArgs<R> &a, R hx, R hy, R 
         for (int32_t k = b; k < e; ++k) {
             const int32_t j = chk(__ldg(a.col + k), a.n, a.err);
             const R *t = a.Jt + 9 * (int64_t)__ldg(a.Jtidx + k);
-            const R sx = ld<Coherent>(X + j), sy = ld<Coherent>(Y + j), sz = ld<Coherent>(Z + j);
+            R sx, sy, sz;
+            S.get(j, sx, sy, sz);
             x = fma(__ldg(t + 0), sx, fma(__ldg(t + 1), sy, fma(__ldg(t + 2), sz, x)));
             y = fma(__ldg(t + 3), sx, fma(__ldg(t + 4), sy, fma(__ldg(t + 5), sz, y)));
             z = fma(__ldg(t + 6), sx, fma(__ldg(t + 7), sy, fma(__ldg(t + 8), sz, z)));
@@ -288,18 +317,22 @@ __device__ __forceinline__ void exchange_sum_h(const KArgs<R> &a, R hx, R hy, R 
             if (b + q < e) {
                 const int32_t j = chk(__ldg(a.col + b + q), a.n, a.err);
                 const R Jk = a.J_uniform ? a.J_value : __ldg(a.J + b + q);
-                x = fma(Jk, ld<Coherent>(X + j), x);
-                y = fma(Jk, ld<Coherent>(Y + j), y);
-                z = fma(Jk, ld<Coherent>(Z + j), z);
+                R sx, sy, sz;
+                S.get(j, sx, sy, sz);
+                x = fma(Jk, sx, x);
+                y = fma(Jk, sy, y);
+                z = fma(Jk, sz, z);
             }
         }
     } else {
         for (int32_t k = b; k < e; ++k) {
             const int32_t j = chk(__ldg(a.col + k), a.n, a.err);
             const R Jk = a.J_uniform ? a.J_value : __ldg(a.J + k);
-            x = fma(Jk, ld<Coherent>(X + j), x);
-            y = fma(Jk, ld<Coherent>(Y + j), y);
-            z = fma(Jk, ld<Coherent>(Z + j), z);
+            R sx, sy, sz;
+            S.get(j, sx, sy, sz);
+            x = fma(Jk, sx, x);
+            y = fma(Jk, sy, y);
+            z = fma(Jk, sz, z);
         }
     }
     e0 = x;
@@ -539,11 +572,26 @@ __device__ __forceinline__ void flush_partials(const double *red, int nq, double
     }
 }
 
+// Where a Heun pass gathers its spins.
+template <typename R, bool Coherent, bool V4>
+__device__ __forceinline__ auto heun_src(const KArgs<R> &a, const R *X, const R *Y, const R *Z, const float4 *V) {
+    (void)a;
+    if constexpr (V4) {
+        static_assert(sizeof(R) == 4 && !Coherent, "float4 spins: FP32-mixed, one pass per launch");
+        return Aos{V};
+    } else {
+        (void)V;
+        return Soa<R, Coherent>{X, Y, Z};
+    }
+}
+
 // Predictor over one tile.  Writes S', Q and H_th; acc receives this thread's sums of the
 // per-spin reduction terms.  Split: the step's Gaussians were written beforehand by k_gauss
 // (every spin reads them, nothing is drawn here) and H_th is not stored (the corrector forms
 // the same product again).
-template <typename R, int BS, bool Coherent, int Mode = kGeneral, bool Split = false>
+// V4 (FP32-mixed): S is read from and S' written to float4 arrays, the half step and the thermal
+// field go into a float4 and a float2 per spin (see k_predictor).
+template <typename R, int BS, bool Coherent, int Mode = kGeneral, bool Split = false, bool V4 = false>
 __device__ __forceinline__ void predictor_tile(const KArgs<R> &a, const TileDesc &td, uint64_t step,
                                                const StepTabT<R> *tab, int pre_slot, double (&acc)[8],
                                                const R *Gx, const R *Gy, const R *Gz) {
@@ -553,37 +601,47 @@ __device__ __forceinline__ void predictor_tile(const KArgs<R> &a, const TileDesc
     const uint32_t key0 = sd.key0, key1 = sd.key1, ctr2 = sd.ctr2;
     const int64_t off = sd.offset - sd.pbase;  // Philox spin index i - off
     const R ha0 = sys_H(sd, 0, R()), ha1 = sys_H(sd, 1, R()), ha2 = sys_H(sd, 2, R());
+    const auto src = heun_src<R, Coherent, V4>(a, a.sx, a.sy, a.sz, a.s4);
     TermAcc<R> ta;
     ta.reset();
     // The slot index is rotated by the warp index, so that the warps of a block reach their
     // transform-heavy slots (the Gaussians not drawn ahead) at different times.
     int rot = (threadIdx.x >> 5) % a.slots;
+    int next_form = (int)threadIdx.x < td.count ? form_of(a, td.start + threadIdx.x) : 0;
     for (int k = threadIdx.x; k < td.count; k += BS, rot = rot + 1 == a.slots ? 0 : rot + 1) {
         const int64_t i = td.start + k;
+        const int form = next_form;  // read a slot ahead: the chain form -> offsets -> spins starts at the offsets
+        if (k + BS < td.count) next_form = form_of(a, i + BS);
         const MatDesc<R> &m = mat_at<Mode>(a, i);
-        const R s0 = ld<Coherent>(a.sx + i), s1 = ld<Coherent>(a.sy + i), s2 = ld<Coherent>(a.sz + i);
+        R s0, s1, s2;
+        src.get(i, s0, s1, s2);
+        const bool given = sqrtT > (R)0 && (Split || rot >= pre_slot);  // drawn beforehand (k_gauss, or the
+                                                                        // previous corrector)
+        R g0 = 0, g1 = 0, g2 = 0;
+        if (given) {  // read before the neighbours, whose loads they then overlap
+            g0 = ld<Coherent>(Gx + i);
+            g1 = ld<Coherent>(Gy + i);
+            g2 = ld<Coherent>(Gz + i);
+        }
         R e0, e1, e2;
-        exchange_sum_h<R, Coherent, BM>(a, ha0, ha1, ha2, a.sx, a.sy, a.sz, i, e0, e1, e2);
+        exchange_sum_h<R, Coherent, BM>(a, ha0, ha1, ha2, src, i, form, e0, e1, e2);
         R H0, H1, H2;
         const R sde = det_field<R, BM != kPlain>(m, s0, s1, s2, e0, e1, e2, H0, H1, H2);
         if (a.demag) add_demag(a, i, H0, H1, H2);
         R t0 = 0, t1 = 0, t2 = 0;
         if (sqrtT > (R)0) {
             const R sig = m.sig * sqrtT;
-            if (Split || rot >= pre_slot) {  // drawn beforehand (k_gauss, or the previous corrector)
-                t0 = mul_rn(sig, ld<Coherent>(Gx + i));
-                t1 = mul_rn(sig, ld<Coherent>(Gy + i));
-                t2 = mul_rn(sig, ld<Coherent>(Gz + i));
-            } else if constexpr (!Split) {
-                const Philox4 w = philox4x32_10((uint32_t)(i - off), (uint32_t)step, ctr2, 0u, key0, key1);
-                R g0, g1, g2;
-                thermal_gaussians(a, *tab, w, g0, g1, g2);
-                t0 = mul_rn(sig, g0);
-                t1 = mul_rn(sig, g1);
-                t2 = mul_rn(sig, g2);
+            if constexpr (!Split) {
+                if (!given) {
+                    const Philox4 w = philox4x32_10((uint32_t)(i - off), (uint32_t)step, ctr2, 0u, key0, key1);
+                    thermal_gaussians(a, *tab, w, g0, g1, g2);
+                }
             }
+            t0 = mul_rn(sig, g0);
+            t1 = mul_rn(sig, g1);
+            t2 = mul_rn(sig, g2);
         }
-        if constexpr (!Split) {
+        if constexpr (!Split && !V4) {
             a.hx[i] = t0;
             a.hy[i] = t1;
             a.hz[i] = t2;
@@ -596,13 +654,19 @@ __device__ __forceinline__ void predictor_tile(const KArgs<R> &a, const TileDesc
         const R dt = m.dt;
         const R v0 = fma(dt, d0, s0), v1 = fma(dt, d1, s1), v2 = fma(dt, d2, s2);
         const R inv = rsqrt_r(fma(v2, v2, fma(v1, v1, mul_rn(v0, v0))));
-        a.px[i] = mul_rn(v0, inv);
-        a.py[i] = mul_rn(v1, inv);
-        a.pz[i] = mul_rn(v2, inv);
         const R hdt = (R)0.5 * dt;
-        a.qx[i] = fma(hdt, d0, s0);
-        a.qy[i] = fma(hdt, d1, s1);
-        a.qz[i] = fma(hdt, d2, s2);
+        if constexpr (V4) {
+            a.p4[i] = make_float4(mul_rn(v0, inv), mul_rn(v1, inv), mul_rn(v2, inv), 0.0f);
+            a.qh4[i] = make_float4(fma(hdt, d0, s0), fma(hdt, d1, s1), fma(hdt, d2, s2), t0);
+            a.qh2[i] = make_float2(t1, t2);
+        } else {
+            a.px[i] = mul_rn(v0, inv);
+            a.py[i] = mul_rn(v1, inv);
+            a.pz[i] = mul_rn(v2, inv);
+            a.qx[i] = fma(hdt, d0, s0);
+            a.qy[i] = fma(hdt, d1, s1);
+            a.qz[i] = fma(hdt, d2, s2);
+        }
         if constexpr (sizeof(R) == 4) {
             R v[5];
             spin_terms_r<R, BM != kPlain>(m, s0, s1, s2, e0, e1, e2, sde, v);
@@ -616,7 +680,7 @@ __device__ __forceinline__ void predictor_tile(const KArgs<R> &a, const TileDesc
     ta.out(acc);
 }
 
-template <typename R, int BS, bool Coherent, int Mode = kGeneral, bool Split = false>
+template <typename R, int BS, bool Coherent, int Mode = kGeneral, bool Split = false, bool V4 = false>
 __device__ __forceinline__ void corrector_tile(const KArgs<R> &a, const TileDesc &td, uint64_t step,
                                                const StepTabT<R> *tab, const R *Gx = nullptr,
                                                const R *Gy = nullptr, const R *Gz = nullptr) {
@@ -629,13 +693,29 @@ __device__ __forceinline__ void corrector_tile(const KArgs<R> &a, const TileDesc
     const uint32_t key0 = sd.key0, key1 = sd.key1, ctr2 = sd.ctr2;
     const int64_t off = sd.offset - sd.pbase;  // Philox spin index i - off
     const R ha0 = sys_H(sd, 0, R()), ha1 = sys_H(sd, 1, R()), ha2 = sys_H(sd, 2, R());
+    const auto src = heun_src<R, Coherent, V4>(a, a.px, a.py, a.pz, a.p4);
     int rot = (threadIdx.x >> 5) % a.slots;  // the predictor's rotated slot index
+    int next_form = (int)threadIdx.x < td.count ? form_of(a, td.start + threadIdx.x) : 0;
     for (int k = threadIdx.x; k < td.count; k += BS, rot = rot + 1 == a.slots ? 0 : rot + 1) {
         const int64_t i = td.start + k;
+        const int form = next_form;  // a slot ahead, as the predictor
+        if (k + BS < td.count) next_form = form_of(a, i + BS);
         const MatDesc<R> &m = mat_at<Mode>(a, i);
-        const R s0 = ld<Coherent>(a.px + i), s1 = ld<Coherent>(a.py + i), s2 = ld<Coherent>(a.pz + i);
+        R s0, s1, s2;
+        src.get(i, s0, s1, s2);
+        R q0, q1, q2, t0 = 0, t1 = 0, t2 = 0;  // the half step and the thermal field
+        if constexpr (V4) {
+            const float4 u = __ldg(a.qh4 + i);
+            const float2 v = __ldg(a.qh2 + i);
+            q0 = u.x;
+            q1 = u.y;
+            q2 = u.z;
+            t0 = u.w;
+            t1 = v.x;
+            t2 = v.y;
+        }
         R e0, e1, e2;
-        exchange_sum_h<R, Coherent, BM>(a, ha0, ha1, ha2, a.px, a.py, a.pz, i, e0, e1, e2);
+        exchange_sum_h<R, Coherent, BM>(a, ha0, ha1, ha2, src, i, form, e0, e1, e2);
         R H0, H1, H2;
         det_field<R, BM != kPlain>(m, s0, s1, s2, e0, e1, e2, H0, H1, H2);
         if (a.demag) add_demag(a, i, H0, H1, H2);
@@ -647,21 +727,33 @@ __device__ __forceinline__ void corrector_tile(const KArgs<R> &a, const TileDesc
                 H2 += mul_rn(sig, ld<Coherent>(Gz + i));
             }
         } else {
-            H0 += ld<Coherent>(a.hx + i);
-            H1 += ld<Coherent>(a.hy + i);
-            H2 += ld<Coherent>(a.hz + i);
+            if constexpr (!V4) {
+                t0 = ld<Coherent>(a.hx + i);
+                t1 = ld<Coherent>(a.hy + i);
+                t2 = ld<Coherent>(a.hz + i);
+            }
+            H0 += t0;
+            H1 += t1;
+            H2 += t2;
         }
         R d0, d1, d2;
         llg_rhs(m.gp, m.lambda, s0, s1, s2, H0, H1, H2, d0, d1, d2);
         const R hdt = (R)0.5 * m.dt;
-        const R v0 = fma(hdt, d0, ld<Coherent>(a.qx + i));
-        const R v1 = fma(hdt, d1, ld<Coherent>(a.qy + i));
-        const R v2 = fma(hdt, d2, ld<Coherent>(a.qz + i));
+        if constexpr (!V4) {
+            q0 = ld<Coherent>(a.qx + i);
+            q1 = ld<Coherent>(a.qy + i);
+            q2 = ld<Coherent>(a.qz + i);
+        }
+        const R v0 = fma(hdt, d0, q0), v1 = fma(hdt, d1, q1), v2 = fma(hdt, d2, q2);
         const R inv = rsqrt_r(fma(v2, v2, fma(v1, v1, mul_rn(v0, v0))));
         if (bad_inv(inv)) atomicOr(a.err, kErrNonFinite);  // NaN or infinite length
-        a.sx[i] = mul_rn(v0, inv);
-        a.sy[i] = mul_rn(v1, inv);
-        a.sz[i] = mul_rn(v2, inv);
+        if constexpr (V4) {
+            a.s4[i] = make_float4(mul_rn(v0, inv), mul_rn(v1, inv), mul_rn(v2, inv), 0.0f);
+        } else {
+            a.sx[i] = mul_rn(v0, inv);
+            a.sy[i] = mul_rn(v1, inv);
+            a.sz[i] = mul_rn(v2, inv);
+        }
         if (!Split && rot >= a.pre_slot && sqrtT_next > (R)0) {
             const Philox4 w = philox4x32_10((uint32_t)(i - off), (uint32_t)(step + 1), ctr2, 0u, key0, key1);
             R g0, g1, g2;
@@ -737,7 +829,7 @@ __device__ __forceinline__ void finalize_system(const SysDesc *sys, const int32_
 
 // Predictor passes over the block's tiles t = blockIdx.x + j gridDim.x, in chunks of
 // kTileChunk tiles whose partials are summed after one barrier.
-template <typename R, int BS, bool Coherent, int Mode = kGeneral, bool Split = false>
+template <typename R, int BS, bool Coherent, int Mode = kGeneral, bool Split = false, bool V4 = false>
 __device__ __forceinline__ void predictor_pass(const KArgs<R> &a, uint64_t step, const StepTabT<R> *tab,
                                                int pre_slot, double *red, const R *Gx, const R *Gy,
                                                const R *Gz) {
@@ -748,7 +840,7 @@ __device__ __forceinline__ void predictor_pass(const KArgs<R> &a, uint64_t step,
             const int64_t t = t0 + nq * stride;
             if (t >= a.ntiles) break;
             double acc[8];
-            predictor_tile<R, BS, Coherent, Mode, Split>(a, a.tiles[t], step, tab, pre_slot, acc, Gx, Gy, Gz);
+            predictor_tile<R, BS, Coherent, Mode, Split, V4>(a, a.tiles[t], step, tab, pre_slot, acc, Gx, Gy, Gz);
             warp_partials<BS>(acc, red, nq);
         }
         __syncthreads();
@@ -757,16 +849,42 @@ __device__ __forceinline__ void predictor_pass(const KArgs<R> &a, uint64_t step,
     }
 }
 
+// The state at the start and at the end of a run of steps over float4 spins.
+static __global__ void __launch_bounds__(256) k_pack_state(const KArgs<float> a) {
+    for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < a.n; i += (int64_t)gridDim.x * 256)
+        a.s4[i] = make_float4(a.sx[i], a.sy[i], a.sz[i], 0.0f);
+}
+static __global__ void __launch_bounds__(256) k_unpack_state(const KArgs<float> a) {
+    for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < a.n; i += (int64_t)gridDim.x * 256) {
+        const float4 s = a.s4[i], p = a.p4[i];
+        a.sx[i] = s.x;
+        a.sy[i] = s.y;
+        a.sz[i] = s.z;
+        a.px[i] = p.x;
+        a.py[i] = p.y;
+        a.pz[i] = p.z;
+    }
+}
+
+// Resident blocks per SM the FP32-mixed Heun passes are compiled for: two of 512 threads (64
+// registers) or 24 warps in smaller blocks (80 registers).  Both passes wait for the gathers, so
+// resident warps and loads in flight per thread trade against each other: rows of six bonds are
+// faster at 64 registers (the 1024 x 1024 x 16 film 0.620 against 0.673 ms per step), rows of
+// twelve at 80 (fcc 64^3 59.7 against 65.1 us, the 20 nm core-shell sphere 48 against 53 us), and
+// a batch of 256 grains runs the same on either (254.8, 252.8 us).  default_shape picks the block.
+__host__ __device__ constexpr int heun_blocks(int bs) { return bs >= 512 ? 2 : 768 / bs; }
+
+// The Heun predictor.  V4 (FP32-mixed runs of several steps): the spins come as one float4 each.
+// Three arrays cost a gather three loads and three addresses, which is what the 64 or 80
+// registers then hold instead of neighbours in flight; a float4 costs one of each.  S' goes out
+// as a float4, and the half step and the thermal field, which only their own spin reads back, as
+// a float4 and a float2.  134 bytes of traffic per spin and step against 110, but the passes move
+// less than 40 % of what HBM gives: the film 0.692 -> 0.620 ms per step.
+//
 // FP64: one resident block per SM is enough for the FP64 pipe, and the minimum-blocks bound
 // lets the compiler keep the transform in registers (without it the FP64 form spills at 64).
-template <typename R, int BS, int Mode = kGeneral>
-#ifndef SS_PRED_WARPS
-#define SS_PRED_WARPS 32
-#endif
-#ifndef SS_CORR_WARPS
-#define SS_CORR_WARPS 32
-#endif
-__global__ void __launch_bounds__(BS, sizeof(R) == 8 ? 1 : SS_PRED_WARPS * 32 / BS) k_predictor(const KArgs<R> a) {
+template <typename R, int BS, int Mode = kGeneral, bool V4 = false>
+__global__ void __launch_bounds__(BS, sizeof(R) == 8 ? 1 : heun_blocks(BS)) k_predictor(const KArgs<R> a) {
     __shared__ StepTabT<R> tab;
     __shared__ double red[kTileChunk * (BS / 32) * 8];
     stage_step_tables(a, tab);
@@ -774,13 +892,13 @@ __global__ void __launch_bounds__(BS, sizeof(R) == 8 ? 1 : SS_PRED_WARPS * 32 / 
     const uint64_t step = *a.step;
     // Gaussians drawn ahead are valid only if the previous corrector ran for this step.
     const int pre_slot = (a.g_step != nullptr && *a.g_step == step) ? a.pre_slot : 1 << 30;
-    predictor_pass<R, BS, false, Mode>(a, step, &tab, pre_slot, red, a.gx, a.gy, a.gz);
+    predictor_pass<R, BS, false, Mode, false, V4>(a, step, &tab, pre_slot, red, a.gx, a.gy, a.gz);
 }
 
 // Blocks [0, nfin) sum the predictor's tile partials into the record ring; the rest run
 // the corrector over the tiles.  The last block to finish advances the step counter.
-template <typename R, int BS, bool DrawAhead, int Mode = kGeneral>
-__global__ void __launch_bounds__(BS, sizeof(R) == 8 ? 0 : SS_CORR_WARPS * 32 / BS) k_corrector(const KArgs<R> a, int nfin) {
+template <typename R, int BS, bool DrawAhead, int Mode = kGeneral, bool V4 = false>
+__global__ void __launch_bounds__(BS, sizeof(R) == 8 ? 0 : heun_blocks(BS)) k_corrector(const KArgs<R> a, int nfin) {
     __shared__ double red[(BS / 32) * 8];
     const uint64_t step = *a.step;
     if ((int)blockIdx.x < nfin) {
@@ -794,7 +912,7 @@ __global__ void __launch_bounds__(BS, sizeof(R) == 8 ? 0 : SS_CORR_WARPS * 32 / 
         __syncthreads();
         const int64_t nb = gridDim.x - nfin;
         for (int64_t t = blockIdx.x - nfin; t < a.ntiles; t += nb)
-            corrector_tile<R, BS, false, Mode>(a, a.tiles[t], step, &tab);
+            corrector_tile<R, BS, false, Mode, false, V4>(a, a.tiles[t], step, &tab);
     } else {
         const int64_t nb = gridDim.x - nfin;
         for (int64_t t = blockIdx.x - nfin; t < a.ntiles; t += nb)
@@ -821,7 +939,7 @@ __global__ void __launch_bounds__(BS, sizeof(R) == 8 ? 0 : SS_CORR_WARPS * 32 / 
 // keep more warps in flight.  The Gaussians move 12 bytes per spin out and 24 back per step,
 // what the stored thermal field and the drawn-ahead Gaussians of the fused step moved.
 template <int BS>
-__global__ void __launch_bounds__(BS) k_gauss(const KArgs<float> a) {
+__global__ void __launch_bounds__(BS, 1024 / BS) k_gauss(const KArgs<float> a) {
     __shared__ FFTables tab;
     stage_ff_tables(a.fftab, tab);
     __syncthreads();
@@ -1279,8 +1397,8 @@ __global__ void __launch_bounds__(256) k_rows_field(const KArgs<R> a, const R *X
 // zero.
 template <typename R, int Mode>
 __device__ __forceinline__ void exchange_bare(const KArgs<R> &a, const R *X, const R *Y, const R *Z, int64_t i,
-                                              R &e0, R &e1, R &e2) {
-    exchange_sum_h<R, false, base_mode(Mode)>(a, (R)0, (R)0, (R)0, X, Y, Z, i, e0, e1, e2);
+                                              int form, R &e0, R &e1, R &e2) {
+    exchange_sum_h<R, false, base_mode(Mode)>(a, (R)0, (R)0, (R)0, Soa<R, false>{X, Y, Z}, i, form, e0, e1, e2);
 }
 
 // ----------------------------------------------------------------------------------
@@ -1318,8 +1436,8 @@ constexpr int kAltBlock = 256;
 // FP64 one for two, 128 registers).
 constexpr int kAltFirstBlocks = 4;
 // and the FP32-mixed second passes (40 registers): they wait for the neighbours' loads, so
-// resident warps count for more than the loads each thread has in flight (the semi-implicit
-// corrector on a 512 x 512 x 16 film: 82 us at the compiler's own 64 registers).
+// resident warps count for more than a few spills (the semi-implicit
+// corrector on a 512 x 512 x 16 film: 82 us at the compiler's own 64 registers, 73 at 48, 68 at 40).
 constexpr int kAltSecondBlocks = 6;
 
 // First pass of the alternative integrators: the step's thermal field (counters as the Heun
@@ -1352,8 +1470,11 @@ __device__ __forceinline__ void alt_first_pass(const KArgs<R> &a, const StepTabT
         const R ha0 = sys_H(sd, 0, R()), ha1 = sys_H(sd, 1, R()), ha2 = sys_H(sd, 2, R());
         TermAcc<R> ta;
         ta.reset();
+        int next_form = k0 + (int)threadIdx.x < k1 ? form_of(a, td.start + k0 + threadIdx.x) : 0;
         for (int k = k0 + threadIdx.x; k < k1; k += kAltBlock) {
             const int64_t i = td.start + k;
+            const int form = next_form;
+            if (k + kAltBlock < k1) next_form = form_of(a, i + kAltBlock);
             const MatDesc<R> &m = mat_at<Mode>(a, i);
             R t0 = 0, t1 = 0, t2 = 0;
             if (sqrtT > (R)0) {
@@ -1368,7 +1489,7 @@ __device__ __forceinline__ void alt_first_pass(const KArgs<R> &a, const StepTabT
             }
             const R s0 = a.sx[i], s1 = a.sy[i], s2 = a.sz[i];
             R x0, x1, x2;
-            exchange_bare<R, Mode>(a, a.sx, a.sy, a.sz, i, x0, x1, x2);
+            exchange_bare<R, Mode>(a, a.sx, a.sy, a.sz, i, form, x0, x1, x2);
             const R c0 = ha0 + t0, c1 = ha1 + t1, c2 = ha2 + t2;
             a.hx[i] = fma((R)0.5, x0, c0);
             a.hy[i] = fma((R)0.5, x1, c1);
@@ -1459,12 +1580,16 @@ __global__ void __launch_bounds__(kAltBlock, sizeof(R) == 4 ? kAltSecondBlocks :
         alt_finalize(a, nfin, sub);
     } else {
         const int64_t first = (int64_t)(blockIdx.x - nfin) * kAltBlock + threadIdx.x;
-        for (int64_t i = first; i < a.n; i += (int64_t)(gridDim.x - nfin) * kAltBlock) {
+        const int64_t stride = (int64_t)(gridDim.x - nfin) * kAltBlock;
+        int next_form = first < a.n ? form_of(a, first) : 0;
+        for (int64_t i = first; i < a.n; i += stride) {
+            const int form = next_form;
+            if (i + stride < a.n) next_form = form_of(a, i + stride);
             const MatDesc<R> &m = mat_at<Mode>(a, i);
             const R s0 = a.sx[i], s1 = a.sy[i], s2 = a.sz[i];
             const R m0 = (R)0.5 * (s0 + xx[i]), m1 = (R)0.5 * (s1 + xy[i]), m2 = (R)0.5 * (s2 + xz[i]);
             R x0, x1, x2;
-            exchange_bare<R, Mode>(a, xx, xy, xz, i, x0, x1, x2);
+            exchange_bare<R, Mode>(a, xx, xy, xz, i, form, x0, x1, x2);
             R H0, H1, H2;
             det_field<R, BM != kPlain>(m, m0, m1, m2, fma((R)0.5, x0, a.hx[i]), fma((R)0.5, x1, a.hy[i]),
                                        fma((R)0.5, x2, a.hz[i]), H0, H1, H2);
@@ -1492,12 +1617,16 @@ __global__ void __launch_bounds__(kAltBlock, sizeof(R) == 4 ? kAltSecondBlocks :
         alt_finalize(a, nfin, sub);
     } else {
         const int64_t first = (int64_t)(blockIdx.x - nfin) * kAltBlock + threadIdx.x;
-        for (int64_t i = first; i < a.n; i += (int64_t)(gridDim.x - nfin) * kAltBlock) {
+        const int64_t stride = (int64_t)(gridDim.x - nfin) * kAltBlock;
+        int next_form = first < a.n ? form_of(a, first) : 0;
+        for (int64_t i = first; i < a.n; i += stride) {
+            const int form = next_form;
+            if (i + stride < a.n) next_form = form_of(a, i + stride);
             const MatDesc<R> &m = mat_at<Mode>(a, i);
             const R s0 = a.sx[i], s1 = a.sy[i], s2 = a.sz[i];
             const R m0 = (R)0.5 * (s0 + a.px[i]), m1 = (R)0.5 * (s1 + a.py[i]), m2 = (R)0.5 * (s2 + a.pz[i]);
             R x0, x1, x2;
-            exchange_bare<R, Mode>(a, a.px, a.py, a.pz, i, x0, x1, x2);
+            exchange_bare<R, Mode>(a, a.px, a.py, a.pz, i, form, x0, x1, x2);
             R H0, H1, H2;
             det_field<R, BM != kPlain>(m, m0, m1, m2, fma((R)0.5, x0, a.hx[i]), fma((R)0.5, x1, a.hy[i]),
                                        fma((R)0.5, x2, a.hz[i]), H0, H1, H2);
@@ -1760,7 +1889,7 @@ __device__ __forceinline__ bool mc_trial(const KArgs<R> &a, const McArgs &m, int
 }
 
 template <typename R, int BS, int Mode = kGeneral>
-__global__ void __launch_bounds__(BS) k_mc_colour(const KArgs<R> a, const McArgs m) {
+__global__ void __launch_bounds__(BS, sizeof(R) == 4 ? 1024 / BS : 1) k_mc_colour(const KArgs<R> a, const McArgs m) {
     __shared__ StepTabT<R> tab;
     stage_step_tables(a, tab);
     __syncthreads();
@@ -1820,7 +1949,7 @@ __device__ __forceinline__ void mc_row_sum8(const KArgs<R> &a, int32_t b, int32_
 // acceptance factor), for the long-row colour passes: their trials then run without the
 // transform's tables or its serial work (mc_randoms is what mc_trial draws otherwise).
 template <typename R, int BS>
-__global__ void __launch_bounds__(BS) k_mc_prep(const KArgs<R> a, const McArgs m) {
+__global__ void __launch_bounds__(BS, sizeof(R) == 4 ? 1024 / BS : 1) k_mc_prep(const KArgs<R> a, const McArgs m) {
     __shared__ StepTabT<R> tab;
     stage_step_tables(a, tab);
     __syncthreads();
@@ -1946,7 +2075,7 @@ __global__ void __launch_bounds__(BS) k_mc_colour_warp1(const KArgs<R> a, const 
 // A colour pass tile by tile that also sums the record terms of the pre-step state of its
 // spins (tile partials in the block's fixed order), for lattices of at most two classes.
 template <typename R, int BS, int Mode, bool First>
-__global__ void __launch_bounds__(BS) k_mc_colour_rec(const KArgs<R> a, const McArgs m) {
+__global__ void __launch_bounds__(BS, sizeof(R) == 4 ? 1024 / BS : 1) k_mc_colour_rec(const KArgs<R> a, const McArgs m) {
     __shared__ StepTabT<R> tab;
     __shared__ double red[(BS / 32) * 8];
     stage_step_tables(a, tab);

@@ -54,6 +54,89 @@ cudaError_t launch_corrector(const KArgs<R> &a, int block, int grid, int nfin, c
     return cudaGetLastError();
 }
 
+// The FP32-mixed Heun passes over float4 spins (the corrector always draws ahead here).
+template <typename R>
+cudaError_t launch_predictor4(const KArgs<R> &a, int block, int grid, cudaStream_t s) {
+    if constexpr (sizeof(R) == 4) {
+#define SS_P4(MODE) SS_BLOCK_SWITCH(block, k_predictor<R, BS, MODE, true><<<grid, BS, 0, s>>>(a))
+        switch (heun_mode(a)) {
+            case kRows: SS_P4(kRows); break;
+            case kGeneral: SS_P4(kGeneral); break;
+            case kUniform: SS_P4(kUniform); break;
+            default: SS_P4(kPlain); break;
+        }
+#undef SS_P4
+        return cudaGetLastError();
+    } else {
+        return cudaErrorNotSupported;
+    }
+}
+
+template <typename R>
+cudaError_t launch_corrector4(const KArgs<R> &a, int block, int grid, int nfin, cudaStream_t s) {
+    if constexpr (sizeof(R) == 4) {
+#define SS_C4(MODE) SS_BLOCK_SWITCH(block, k_corrector<R, BS, true, MODE, true><<<grid + nfin, BS, 0, s>>>(a, nfin))
+        switch (heun_mode(a)) {
+            case kRows: SS_C4(kRows); break;
+            case kGeneral: SS_C4(kGeneral); break;
+            case kUniform: SS_C4(kUniform); break;
+            default: SS_C4(kPlain); break;
+        }
+#undef SS_C4
+        return cudaGetLastError();
+    } else {
+        return cudaErrorNotSupported;
+    }
+}
+
+// Resident blocks per SM of the passes over float4 spins (which = 0: predictor, 1: corrector).
+template <typename R>
+int packed_blocks_per_sm(int block, int mode, int which) {
+    int nb = 0;
+    cudaError_t e = cudaErrorInvalidValue;
+    if constexpr (sizeof(R) == 4) {
+#define SS_OCC(MODE)                                                                                                \
+    if (which == 0) {                                                                                               \
+        SS_BLOCK_SWITCH(block, e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_predictor<R, BS, MODE, true>, \
+                                                                                 BS, 0));                           \
+    } else {                                                                                                        \
+        SS_BLOCK_SWITCH(block, e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(                                   \
+                                   &nb, k_corrector<R, BS, true, MODE, true>, BS, 0));                              \
+    }
+        if (mode == kRows) {
+            SS_OCC(kRows)
+        } else if (mode == kGeneral) {
+            SS_OCC(kGeneral)
+        } else if (mode == kUniform) {
+            SS_OCC(kUniform)
+        } else {
+            SS_OCC(kPlain)
+        }
+#undef SS_OCC
+    }
+    return e == cudaSuccess ? nb : 0;
+}
+
+template <typename R>
+cudaError_t launch_pack_state(const KArgs<R> &a, int grid, cudaStream_t s) {
+    if constexpr (sizeof(R) == 4) {
+        k_pack_state<<<grid, 256, 0, s>>>(a);
+        return cudaGetLastError();
+    } else {
+        return cudaErrorNotSupported;
+    }
+}
+
+template <typename R>
+cudaError_t launch_unpack_state(const KArgs<R> &a, int grid, cudaStream_t s) {
+    if constexpr (sizeof(R) == 4) {
+        k_unpack_state<<<grid, 256, 0, s>>>(a);
+        return cudaGetLastError();
+    } else {
+        return cudaErrorNotSupported;
+    }
+}
+
 // The split FP32-mixed step (a Gaussian pass, then the two Heun passes reading it): variants
 // kUniform, kPlain and kGeneral of the thread-per-row exchange sum.
 // priority: the launch's scheduling priority (cudaLaunchAttributePriority; 0 = the stream's)
@@ -367,7 +450,9 @@ cudaError_t launch_sib(const KArgs<R> &a, const AltGrids &g, cudaStream_t s) {
 
 template <typename R>
 cudaError_t launch_rows_field(const KArgs<R> &a, const R *X, const R *Y, const R *Z, int grid, cudaStream_t s) {
-    if (a.sell) {
+    if (a.sell && !X) {  // the caller's spins are float4 already (a.x4)
+        k_rows_sell<R><<<grid, 256, 0, s>>>(a);
+    } else if (a.sell) {
         const int64_t pb = (a.n + 255) / 256;
         k_pack4<R><<<(int)(pb < 4 * (int64_t)grid ? pb : 4 * (int64_t)grid), 256, 0, s>>>(a, X, Y, Z);
         cudaError_t e = cudaGetLastError();
@@ -460,6 +545,12 @@ template int mc_blocks_per_sm<SS_REAL>(int, int);
 template cudaError_t launch_midpoint<SS_REAL>(const KArgs<SS_REAL> &, int, const AltGrids &, cudaStream_t);
 template cudaError_t launch_sib<SS_REAL>(const KArgs<SS_REAL> &, const AltGrids &, cudaStream_t);
 template int alt_pass_blocks_per_sm<SS_REAL>(int, int);
+#elif SS_PART == 5  // the FP32-mixed Heun passes over float4 spins
+template cudaError_t launch_predictor4<SS_REAL>(const KArgs<SS_REAL> &, int, int, cudaStream_t);
+template cudaError_t launch_corrector4<SS_REAL>(const KArgs<SS_REAL> &, int, int, int, cudaStream_t);
+template int packed_blocks_per_sm<SS_REAL>(int, int, int);
+template cudaError_t launch_pack_state<SS_REAL>(const KArgs<SS_REAL> &, int, cudaStream_t);
+template cudaError_t launch_unpack_state<SS_REAL>(const KArgs<SS_REAL> &, int, cudaStream_t);
 #endif
 
 }  // namespace ss
