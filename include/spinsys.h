@@ -358,8 +358,11 @@ ss_status spin_system_set_exchange_rows(ss_system *h, int32_t mode);
  * tables; the sums then read one or two bytes per spin instead of the row's offsets and
  * columns, and add the same terms in the same order, so the results are identical.  "Few"
  * means at most 65,536 forms and at most one form slot (8 per form for rows of up to 6 bonds,
- * 16 beyond) per two bonds, so that the tables stay well below the CSR's size (the 20 nm
- * core-shell sphere, 76,795 forms, reads the CSR).  on = 1 (the default) uses the forms when they were built, 0 reads the CSR;
+ * 16 beyond) per two bonds, so that the tables stay well below the CSR's size.  Scalar rows of at
+ * most 12 bonds that take more forms (the 20 nm core-shell sphere: 76,795), with at most 255
+ * distinct J_ij/mu_s,i and fewer than 2^24 spins, are stored in columns of packed bonds instead
+ * (4 bytes per bond, rows padded to 6 or 12 with zero bonds): again the same terms in the same
+ * order.  on = 1 (the default) uses the forms or columns when they were built, 0 reads the CSR;
  * ss_info.row_patterns gives the number of forms in use (0: CSR).  With tensor bonds (Eq.
  * HJijSMS) a form holds each bond's tensor, as an entry of the handle's tensor dictionary, in
  * place of J_ij/mu_s,i.  SS_ERR_INVALID_ARG for another value. */

@@ -121,6 +121,10 @@ struct ss_system {
     int32_t pat_w = 8;                  // slots of a pattern row (8 or 16, see KArgs)
     bool pat_wide = false;              // two-byte pattern indices (more than 256 forms)
     bool use_pat = true;                // spin_system_set_row_patterns
+    // Packed bonds in columns, for short rows without row forms (build_ell)
+    uint32_t *ell = nullptr;
+    void *ell_J = nullptr;
+    int ell_w = 0;
     // Slab of a decomposed system (spin_slab_create): the owned spins are the first slab_own
     // of the arrays, the halo copies follow; tiles cover the owned spins, boundary tiles first
     int64_t slab_own = -1;              // -1: not a slab
@@ -504,6 +508,9 @@ KArgs<R> make_args(const ss_system *h) {
     a.pat_J = pat ? static_cast<const R *>(h->pat_J) : nullptr;
     a.pat_w = h->pat_w;
     a.pat_wide = h->pat_wide ? 1 : 0;
+    a.ell = h->use_pat ? h->ell : nullptr;
+    a.ell_J = static_cast<const R *>(h->ell_J);
+    a.ell_w = h->ell_w;
     a.mat_uniform = h->nmat == 1 ? 1 : 0;
     std::memcpy(&a.mat0, h->mat0, sizeof(MatDesc<R>));
     a.Jt = static_cast<const R *>(h->Jt);
@@ -1049,8 +1056,7 @@ void fill_material(MatDesc<R> &m, const MatKey &k, const ss_params *p) {
     const double mu = k.v[0], ku = k.v[1];
     const double gamma = p->gamma > 0.0 ? p->gamma : kGammaDefault;
     const double lam = p->alpha;
-    std::memset(&m, 0, sizeof(m));
-    m.inv_mu = (R)(1.0 / mu);
+    std::memset(static_cast<void *>(&m), 0, sizeof(m));
     m.ani = (R)(2.0 * ku / mu);
     for (int c = 0; c < 3; ++c) m.e[c] = (R)k.v[2 + c];
     for (int c = 0; c < 6; ++c) {
@@ -1066,8 +1072,81 @@ void fill_material(MatDesc<R> &m, const MatKey &k, const ss_params *p) {
     m.kc = (R)k.v[11];
     m.kcf = (R)(-2.0 * k.v[11] / mu);
     m.sys = k.sys;
-    m.has_neel = k.has_neel;
+    m.has_neel = (int16_t)k.has_neel;
     m.has_cubic = k.v[11] != 0.0 ? 1 : 0;
+}
+
+// The distinct J_ij / mu_s,i of the bonds (at most 255, and 0 for padding) and each bond's entry.
+template <typename R>
+bool bond_dictionary(const std::vector<R> &J, int64_t nnz, std::vector<R> &dict, std::vector<uint8_t> &bid, int &zero) {
+    using Bits = typename std::conditional<sizeof(R) == 8, uint64_t, uint32_t>::type;
+    constexpr int kSlots = 1024;
+    std::vector<Bits> key(kSlots);
+    std::vector<int> id(kSlots, -1);
+    Bits last = 0;
+    bid.resize((size_t)nnz);
+    zero = -1;
+    for (int64_t k = 0; k < nnz; ++k) {
+        Bits b;
+        std::memcpy(&b, &J[k], sizeof(R));
+        if (k > 0 && b == last) {  // (bonds of a row mostly repeat)
+            bid[(size_t)k] = bid[(size_t)k - 1];
+            continue;
+        }
+        last = b;
+        uint32_t hsh = (uint32_t)(((uint64_t)b * 0x9E3779B97F4A7C15ull) >> 54);  // 10 bits
+        while (id[hsh] >= 0 && key[hsh] != b) hsh = (hsh + 1) & (kSlots - 1);
+        if (id[hsh] < 0) {
+            if (dict.size() == 255) return false;
+            key[hsh] = b;
+            id[hsh] = (int)dict.size();
+            if (b == 0) zero = id[hsh];
+            dict.push_back(J[k]);
+        }
+        bid[(size_t)k] = (uint8_t)id[hsh];
+    }
+    if (zero < 0) {
+        zero = (int)dict.size();
+        dict.push_back((R)0);
+    }
+    return true;
+}
+
+// Packed bonds in columns for rows of at most kPatRow scalar bonds that have no row forms (see
+// ell_sum).  Without the memory for them, or with more distinct J or spins than a word holds, the
+// CSR is read.
+template <typename R>
+ss_status build_ell(ss_system *h, const std::vector<int32_t> &rp, const std::vector<int32_t> &col,
+                    const std::vector<R> &J) {
+    const int64_t n = h->n, nnz = h->nnz;
+    if (h->npat > 0 || h->J_tensor || nnz <= 0 || h->max_row > kPatRow || n >= (int64_t(1) << 24)) return SS_OK;
+    const int W = h->max_row <= kShortRow ? kShortRow : kPatRow;
+    std::vector<R> dict;
+    std::vector<uint8_t> bid;
+    int zero;
+    if (!bond_dictionary<R>(J, nnz, dict, bid, zero)) return SS_OK;
+    void *J_dev = nullptr;
+    uint32_t *ell = nullptr;
+    if (dalloc(h, (void **)&ell, (size_t)W * n * sizeof(uint32_t)) != cudaSuccess ||
+        dalloc(h, &J_dev, dict.size() * sizeof(R)) != cudaSuccess) {
+        cudaGetLastError();
+        if (ell) dfree(h, ell);
+        return SS_OK;
+    }
+    std::vector<uint32_t> words((size_t)W * n);
+    for (int64_t i = 0; i < n; ++i) {
+        const int32_t b = rp[i], len = rp[i + 1] - b;
+        for (int32_t k = 0; k < W; ++k)
+            words[(size_t)(k * n + i)] = k < len ? ((uint32_t)col[b + k] << 8) | bid[(size_t)(b + k)]
+                                                 : ((uint32_t)i << 8) | (uint32_t)zero;
+    }
+    SS_CUDA(h, cudaMemcpyAsync(ell, words.data(), words.size() * sizeof(uint32_t), cudaMemcpyHostToDevice, h->stream));
+    SS_CUDA(h, cudaMemcpyAsync(J_dev, dict.data(), dict.size() * sizeof(R), cudaMemcpyHostToDevice, h->stream));
+    SS_CUDA(h, cudaStreamSynchronize(h->stream));  // the host vectors go out of scope
+    h->ell = ell;
+    h->ell_J = J_dev;
+    h->ell_w = W;
+    return SS_OK;
 }
 
 // Rows averaging this many bonds or more get a warp each for the exchange sum (FP32-mixed,
@@ -1186,36 +1265,10 @@ ss_status upload_system(ss_system *h, const std::vector<HostSys> &hs) {
     // of 32 rows (bond k of the slice's row l at 32 k + l), each padded to its longest row with
     // J = 0 bonds.
     if (!tensor && nnz >= kSellMin * n && n < (int64_t(1) << 24)) {
-        using Bits = typename std::conditional<sizeof(R) == 8, uint64_t, uint32_t>::type;
-        constexpr int kSlots = 1024;
-        std::vector<Bits> key(kSlots);
-        std::vector<int> id(kSlots, -1);
         std::vector<R> dict;
-        std::vector<uint8_t> bid((size_t)nnz);
-        bool ok = true;
+        std::vector<uint8_t> bid;
         int zero = -1;
-        for (int64_t k = 0; k < nnz && ok; ++k) {
-            Bits b;
-            std::memcpy(&b, &J[k], sizeof(R));
-            uint32_t hsh = (uint32_t)(((uint64_t)b * 0x9E3779B97F4A7C15ull) >> 54);  // 10 bits
-            while (id[hsh] >= 0 && key[hsh] != b) hsh = (hsh + 1) & (kSlots - 1);
-            if (id[hsh] < 0) {
-                if (dict.size() == 255) {
-                    ok = false;
-                    break;
-                }
-                key[hsh] = b;
-                id[hsh] = (int)dict.size();
-                if (b == 0) zero = id[hsh];
-                dict.push_back(J[k]);
-            }
-            bid[(size_t)k] = (uint8_t)id[hsh];
-        }
-        if (ok) {
-            if (zero < 0) {
-                zero = (int)dict.size();
-                dict.push_back((R)0);
-            }
+        if (bond_dictionary<R>(J, nnz, dict, bid, zero)) {
             const int64_t nsl = (n + 31) / 32;
             std::vector<int64_t> off((size_t)nsl + 1, 0);
             for (int64_t s = 0; s < nsl; ++s) {
@@ -1271,7 +1324,8 @@ ss_status upload_system(ss_system *h, const std::vector<HostSys> &hs) {
     SS_CUDA(h, cudaMemcpyAsync(h->mats, mats.data(), mats.size() * sizeof(MatDesc<R>), cudaMemcpyHostToDevice,
                                h->stream));
     {
-        const ss_status ps = build_patterns<R>(h, rp, col, J, Jtidx);
+        ss_status ps = build_patterns<R>(h, rp, col, J, Jtidx);
+        if (ps == SS_OK) ps = build_ell<R>(h, rp, col, J);
         if (ps != SS_OK) return ps;
     }
     for (int b = 0; b < 12; ++b) SS_CUDA(h, dalloc(h, &h->state[b], (size_t)n * rs));
@@ -1342,32 +1396,35 @@ ss_status set_rows(ss_system *h, int32_t mode) {
 }
 
 // The default launch shape.  Block: the FP32-mixed kernels are compiled for more resident warps in
-// 512-thread blocks and for more registers in smaller ones (heun_blocks); short rows of a single
-// material are faster in the former from about a million spins on, everything else in the
-// latter.  FP64: 512 threads for large systems.
-// Spins per thread: the resident blocks take the tiles round by round, so a pass takes the rounds
-// times the spins per thread (and about 0.3 spins' time for each tile's reduction); the count, up
-// to 12, that makes this least.  fcc 64^3 in FP32-mixed form: two spins per thread are 4.5
-// rounds of 456 blocks, run as five; nine are one round exactly (66.2 -> 59.7 us per step).  From
-// 12 rounds of eight spins per thread on there is little to round off, and eight are as fast as any.
+// 512-thread blocks and for more registers in smaller ones (heun_blocks); rows of at most six
+// bonds are faster in the former from about two million spins on (film of 1.05 M: 47.8 us per
+// step with 256 threads, 49.3 with 512; 256 grains of 5.2 M together: 256 and 248), everything
+// else in the latter.  FP64: 512 threads from four million spins on.
+// Spins per thread, up to 12: the count that leaves the busiest SM the least to do, its tiles times
+// the spins per thread (and about 0.3 spins' time for each tile's reduction).  The FP32-mixed
+// passes also need warps to hide their gathers: 16 a SM cost about 4 %, eight 30 % (FP64: eight 5 %).  fcc 64^3 in FP32-mixed form: 2 spins per thread leave the busiest SM 14
+// tiles for 13.5 on average, 9 three for exactly three (66.2 -> 59.7 us per step).  From 24 tiles
+// of eight spins per thread a SM on there is little to round off, and eight are as fast as any.
 void default_shape(ss_system *h) {
     const bool mixed = h->precision == SS_FP32_MIXED;
-    const bool short_uniform = h->nmat == 1 && h->max_row <= kShortRow && !h->J_tensor && !h->any_cubic;
-    h->block = (mixed ? short_uniform && h->n >= (int64_t(1) << 20) : h->n >= (int64_t(1) << 22)) ? 512 : 256;
-    const int64_t resident = (int64_t)std::max(h->sm_count, 1) * (mixed ? (h->block == 512 ? 2 : 3) : 1);
+    const bool wide = h->n >= (int64_t(1) << (mixed ? 21 : 22)) && (!mixed || h->max_row <= kShortRow);
+    h->block = wide ? 512 : 256;
+    const int64_t sms = std::max(h->sm_count, 1);
     int best = 8;
     double least = 1e300;
     for (int slots = 1; slots <= 12; ++slots) {
         const int64_t tile = (int64_t)slots * h->block;
         int64_t tiles = 0;
         for (int64_t n : h->sys_n) tiles += (n + tile - 1) / tile;
-        const int64_t rounds = (tiles + resident - 1) / resident;
-        const double cost = (double)rounds * (slots + 0.3);
+        const int64_t per_sm = (tiles + sms - 1) / sms;
+        double cost = (double)per_sm * (slots + 0.3);
+        const double warps = (double)per_sm * h->block / 32.0;
+        cost *= mixed ? 1.0 + 0.3 * std::pow(std::max(0.0, 24.0 - warps) / 16.0, 3.0) : (warps < 16.0 ? 1.05 : 1.0);
         if (cost < least) {
             least = cost;
             best = slots;
         }
-        if (slots == 8 && tiles >= 12 * resident) {
+        if (slots == 8 && tiles >= 24 * sms) {
             best = 8;
             break;
         }

@@ -50,26 +50,24 @@ struct SysDesc {
 
 // One material: a distinct (system, mu_s, k_u, easy axis, Neel tensor) combination.
 // Per-spin arrays are replaced by a material index per spin; identical sites share an
-// entry, so a homogeneous lattice reads one broadcast entry.
+// entry, so a homogeneous lattice reads one broadcast entry.  What every spin's update reads
+// comes first and starts on 16 bytes.
 template <typename R>
-struct MatDesc {
-    R inv_mu;     // 1 / mu_s                                      (1/(J/T))
+struct alignas(16) MatDesc {
     R ani;        // 2 k_u / mu_s                                  (T)
     R e[3];       // easy axis
-    R kf[6];      // (2 / mu_s) K, field tensor of the Neel term    (T)
     R gp;         // gamma / (1 + lambda^2)
     R lambda;     // damping
     R dt;         // time step
     R sig;        // sqrt(2 lambda kB / (gamma mu_s dt)); sigma = sig * sqrt(T)
     R mu;         // mu_s
     R ku;         // k_u
+    int32_t sys;
+    int16_t has_neel, has_cubic;
+    R kf[6];      // (2 / mu_s) K, field tensor of the Neel term    (T)
     R K[6];       // Neel tensor (energy)
     R kc;         // cubic anisotropy k_c (energy (k_c/2) sum S^4)
     R kcf;        // -2 k_c / mu_s (field factor of S^3)
-    int32_t sys;
-    int32_t has_neel;
-    int32_t has_cubic;
-    int32_t pad;
 };
 
 // A contiguous range of spins of one system, processed by one block per pass.
@@ -98,6 +96,9 @@ struct KArgs {
     const R *pat_J;           // [npat][pat_w] J_ij / mu_s,i of each bond, 0 past the row's end;
                               // with tensor bonds int32 Jt entries instead (J is not read)
     int pat_w;                // 8: rows of at most kShortRow bonds; 16: at most kPatRow
+    const uint32_t *ell;      // rows without row forms: bond k of row i at ell[k * n + i] as in `sell` (col <<
+    const R *ell_J;           // 8 | entry of ell_J), ell_w of them, padded with J = 0; or nullptr
+    int ell_w;
     MatDesc<R> mat0;          // the only material when mat_uniform is set
     int mat_uniform;          // 1: every spin has material 0 (mat is not read)
     const R *Jt;              // [9 ndict] distinct exchange tensors / mu_s,i, row by row

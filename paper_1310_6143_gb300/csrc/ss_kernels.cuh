@@ -262,6 +262,28 @@ __device__ __forceinline__ void pattern_sum_tensor(const KArgs<R> &a, const Src 
     }
 }
 
+// The exchange sum of a row stored as NS packed bonds in columns (bond k of every row adjacent):
+// the words and then the gathers of the whole row are in flight at once, where the CSR loop
+// waits for each bond's column before its gather.  Padding is the spin itself with J = 0, which
+// adds exact zeros after the row's terms.  For rows that take too many forms: the 20 nm
+// core-shell sphere (76,795 forms) 48.3 us per step from the CSR (its predictor 1,392
+// instructions a warp at 33 % issue), 36.1 from the columns, both at five spins per thread.
+template <typename R, int NS, typename Src>
+__device__ __forceinline__ void ell_sum(const KArgs<R> &a, const Src &S, int64_t i, R &x, R &y, R &z) {
+    uint32_t w[NS];
+#pragma unroll
+    for (int q = 0; q < NS; ++q) w[q] = __ldg(a.ell + q * a.n + i);
+#pragma unroll
+    for (int q = 0; q < NS; ++q) {
+        const R Jk = __ldg(a.ell_J + (w[q] & 255u));
+        R sx, sy, sz;
+        S.get(chk(w[q] >> 8, a.n, a.err), sx, sy, sz);
+        x = fma(Jk, sx, x);
+        y = fma(Jk, sy, y);
+        z = fma(Jk, sz, z);
+    }
+}
+
 // The sum started at the system's applied field (hx, hy, hz), passed in by callers that hold
 // it in registers for a whole tile, as is the spin's row form (form_of).
 template <typename R, bool Coherent, int Mode, typename Src>
@@ -289,6 +311,16 @@ __device__ __forceinline__ void exchange_sum_h(const KArgs<R> &a, R hx, R hy, R 
             pattern_sum_tensor<R, kShortRow>(a, S, i, form, x, y, z);
         else
             pattern_sum_tensor<R, kPatRow>(a, S, i, form, x, y, z);
+        e0 = x;
+        e1 = y;
+        e2 = z;
+        return;
+    }
+    if (a.ell && !(Mode == kGeneral && a.J_tensor)) {
+        if (a.ell_w == kShortRow)
+            ell_sum<R, kShortRow>(a, S, i, x, y, z);
+        else
+            ell_sum<R, kPatRow>(a, S, i, x, y, z);
         e0 = x;
         e1 = y;
         e2 = z;
@@ -869,9 +901,9 @@ static __global__ void __launch_bounds__(256) k_unpack_state(const KArgs<float> 
 // Resident blocks per SM the FP32-mixed Heun passes are compiled for: two of 512 threads (64
 // registers) or 24 warps in smaller blocks (80 registers).  Both passes wait for the gathers, so
 // resident warps and loads in flight per thread trade against each other: rows of six bonds are
-// faster at 64 registers (the 1024 x 1024 x 16 film 0.620 against 0.673 ms per step), rows of
-// twelve at 80 (fcc 64^3 59.7 against 65.1 us, the 20 nm core-shell sphere 48 against 53 us), and
-// a batch of 256 grains runs the same on either (254.8, 252.8 us).  default_shape picks the block.
+// faster at 64 registers (the 1024 x 1024 x 16 film 0.620 against 0.673 ms per step, 256 grains
+// 248 against 256 us), rows of twelve at 80 (fcc 64^3 59.7 against 65.1 us, the 20 nm core-shell
+// sphere 36 against 40 us).  default_shape picks the block.
 __host__ __device__ constexpr int heun_blocks(int bs) { return bs >= 512 ? 2 : 768 / bs; }
 
 // The Heun predictor.  V4 (FP32-mixed runs of several steps): the spins come as one float4 each.
@@ -1757,8 +1789,7 @@ __device__ __forceinline__ const SmemTables &fp64_tables(const KArgs<float> &a, 
 template <typename R>
 __device__ __forceinline__ int mc_randoms(const KArgs<R> &a, int64_t i, uint64_t step, const StepTabT<R> &tab,
                                           R &g0, R &g1, R &g2, double &lnu) {
-    const MatDesc<R> &mt = a.mats[mat_of(a, i)];
-    const SysDesc &sd = a.sys[mt.sys];
+    const SysDesc &sd = a.sys[a.mats[mat_of(a, i)].sys];
     const uint32_t spin = (uint32_t)(i - sd.offset + sd.pbase);
     const Philox4 wa = philox4x32_10(spin, (uint32_t)step, sd.ctr2, 2u, sd.key0, sd.key1);
     const Philox4 wb = philox4x32_10(spin, (uint32_t)step, sd.ctr2, 3u, sd.key0, sd.key1);
