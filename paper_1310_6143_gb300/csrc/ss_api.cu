@@ -182,9 +182,11 @@ struct ss_system {
     // each step pass, when the rows are long enough (set_rows) or on request
     int rows_req = 0;            // 0 automatic, 1 a thread per row, 2 a warp per row
     bool rows = false;           // a warp per row in force
-    uint32_t *sell = nullptr;    // packed bonds col << 8 | dictionary entry, slices of 32 rows
-    int64_t *sell_off = nullptr; // [nslice + 1] word offset of each slice
+    uint32_t *sell = nullptr;    // packed bonds of the distinct slices of 32 rows (k_rows_sell)
+    int64_t *sell_off = nullptr; // [distinct slices + 1] word offset of each
+    int2 *slice = nullptr;       // [nslice] (distinct slice, first row)
     int64_t nslice = 0;
+    int period = 1;              // distance of a slice's rows
     void *Jd = nullptr;          // the dictionary of J_ij / mu_s,i (with 0 for the padding)
     int nJd = 0;
     void *x4 = nullptr;          // (x, y, z, 0) copy of the spins the sliced pass reads
@@ -492,6 +494,22 @@ ss_status build_patterns(ss_system *h, const std::vector<int32_t> &rp, const std
     return SS_OK;
 }
 
+// The classes of a period: spins i = b, b + period, ... of each b, padded to whole slices.
+struct Classes {
+    int64_t n;
+    int period, rest, hi, lo;
+    Classes(int64_t n_, int period_) : n(n_), period(period_), rest((int)(n_ % period_)) {
+        lo = (int)((n / period + 31) / 32);
+        hi = (int)((n / period + 1 + 31) / 32);
+    }
+    int64_t first(int64_t b) const { return b <= rest ? b * hi : (int64_t)rest * hi + (b - rest) * lo; }
+    int64_t slices() const { return first(period); }
+    int64_t pos(int64_t i) const { return 32 * first(i % period) + i / period; }  // as x4_pos on the device
+};
+
+// Spins of a float4 array: with sliced long rows the classes' padding as well.
+int64_t packed_spins(const ss_system *h) { return std::max<int64_t>(h->n, 32 * h->nslice); }
+
 template <typename R>
 KArgs<R> make_args(const ss_system *h) {
     KArgs<R> a{};
@@ -521,7 +539,15 @@ KArgs<R> make_args(const ss_system *h) {
     a.rows_bare = 0;
     a.sell = h->sell;
     a.sell_off = h->sell_off;
+    a.slice = h->slice;
     a.nslice = h->nslice;
+    {
+        const Classes c(h->n, h->period);
+        a.period = c.period;
+        a.period_rest = c.rest;
+        a.period_hi = c.hi;
+        a.period_lo = c.lo;
+    }
     a.x4 = static_cast<R *>(h->x4);
     a.Jd = static_cast<const R *>(h->Jd);
     a.nJd = h->nJd;
@@ -545,9 +571,10 @@ KArgs<R> make_args(const ss_system *h) {
     a.qx = s[6]; a.qy = s[7]; a.qz = s[8];
     a.hx = s[9]; a.hy = s[10]; a.hz = s[11];
     a.s4 = static_cast<float4 *>(h->packed);
-    a.p4 = a.s4 ? a.s4 + h->n : nullptr;
-    a.qh4 = a.s4 ? a.s4 + 2 * h->n : nullptr;
-    a.qh2 = a.s4 ? reinterpret_cast<float2 *>(a.s4 + 3 * h->n) : nullptr;
+    const int64_t n4 = packed_spins(h);
+    a.p4 = a.s4 ? a.s4 + n4 : nullptr;
+    a.qh4 = a.s4 ? a.s4 + 2 * n4 : nullptr;
+    a.qh2 = a.s4 ? reinterpret_cast<float2 *>(a.s4 + 3 * n4) : nullptr;
     a.gx = static_cast<R *>(h->ahead[0]);
     a.gy = static_cast<R *>(h->ahead[1]);
     a.gz = static_cast<R *>(h->ahead[2]);
@@ -699,7 +726,8 @@ cudaError_t enqueue_packed_step(const ss_system *h, const KArgs<R> &a, int gp, i
 // S into float4 spins before the run, S and S' back into their arrays after it.
 cudaError_t packed_state(const ss_system *h, bool pack) {
     if (h->precision != SS_FP32_MIXED) return cudaErrorInvalidValue;
-    const KArgs<float> a = make_args<float>(h);
+    KArgs<float> a = make_args<float>(h);
+    use_rows(h, a);
     const int grid = (int)std::min<int64_t>((h->n + 255) / 256, (int64_t)h->sm_count * 8);
     return pack ? launch_pack_state<float>(a, grid, h->stream) : launch_unpack_state<float>(a, grid, h->stream);
 }
@@ -1112,19 +1140,114 @@ bool bond_dictionary(const std::vector<R> &J, int64_t nnz, std::vector<R> &dict,
     return true;
 }
 
+// The slices of k_rows_sell.  The period is the one of a few whose slices' bonds touch the fewest
+// 128-byte lines of the spins' copy (a sample of the rows; a larger one has to be a tenth better),
+// as long as the positions fit a bond word.
+ss_status build_slices(ss_system *h, const std::vector<int32_t> &rp, const std::vector<int32_t> &col,
+                       const std::vector<uint8_t> &bid, int zero) {
+    const int64_t n = h->n;
+    int period = 1;
+    int64_t least = INT64_MAX;
+    for (int p : {1, 2, 3, 4, 6, 8}) {
+        const Classes c(n, p);
+        if (32 * c.slices() >= (int64_t(1) << 24) || p > n) continue;
+        int64_t lines = 0;
+        std::vector<int64_t> seen;
+        for (int q = 0; q < 8; ++q) {  // slices spread over the rows, some of their bonds
+            const int64_t i0 = (n - 1) * q / 8;
+            int32_t len = INT32_MAX;
+            for (int l = 0; l < 32 && i0 + (int64_t)l * p < n; ++l) len = std::min(len, rp[i0 + (int64_t)l * p + 1] - rp[i0 + (int64_t)l * p]);
+            for (int32_t k = 0; k < len; k += 1 + len / 16) {
+                seen.clear();
+                for (int l = 0; l < 32 && i0 + (int64_t)l * p < n; ++l) seen.push_back(c.pos(col[rp[i0 + (int64_t)l * p] + k]) >> 3);
+                std::sort(seen.begin(), seen.end());
+                lines += std::unique(seen.begin(), seen.end()) - seen.begin();
+            }
+        }
+        if (lines < least - least / 10) {
+            least = lines;
+            period = p;
+        }
+    }
+    const Classes c(n, period);
+    const int64_t nsl = c.slices();
+    std::vector<int32_t> pos((size_t)n);
+    for (int64_t b = 0; b < period; ++b) {
+        int32_t at = (int32_t)(32 * c.first(b));
+        for (int64_t i = b; i < n; i += period) pos[(size_t)i] = at++;
+    }
+    std::vector<int2> slice((size_t)nsl);
+    std::vector<int64_t> off(1, 0);
+    std::vector<uint32_t> sell, words;
+    std::unordered_multimap<uint64_t, int32_t> form_of;  // hash of a slice's words -> form (contents compared)
+    for (int64_t b = 0; b < period; ++b) {
+        for (int64_t s = c.first(b); s < c.first(b + 1); ++s) {
+            const int64_t row0 = b + (int64_t)period * 32 * (s - c.first(b));
+            int32_t w = 0;
+            for (int64_t i = row0; i < std::min<int64_t>(n, row0 + 32 * (int64_t)period); i += period) w = std::max(w, rp[i + 1] - rp[i]);
+            words.resize(32 * (size_t)w);
+            const int32_t base = (int32_t)(32 * s);
+            for (int l = 0; l < 32; ++l) {
+                const int64_t i = row0 + (int64_t)l * period;
+                const int32_t len = i < n ? rp[i + 1] - rp[i] : 0;
+                const uint32_t pad = ((uint32_t)l << 8) | (uint32_t)zero;
+                uint32_t *out = words.data() + l;
+                const int32_t *cj = i < n ? col.data() + rp[i] : nullptr;
+                const uint8_t *bj = i < n ? bid.data() + rp[i] : nullptr;
+                for (int32_t k = 0; k < len; ++k) out[32 * (size_t)k] = ((uint32_t)(pos[(size_t)cj[k]] - base) << 8) | bj[k];
+                for (int32_t k = len; k < w; ++k) out[32 * (size_t)k] = pad;
+            }
+            uint64_t hsh = (uint64_t)w, mul = 0x9E3779B97F4A7C15ull;  // of a sample: contents are compared below
+            for (size_t q = 0; q < words.size(); q += 29) {
+                hsh += (words[q] ^ 0x5bd1e995u) * mul;
+                mul += 0xBF58476D1CE4E5BAull;
+            }
+            hsh ^= hsh >> 31;
+            int32_t form = -1;
+            const auto range = form_of.equal_range(hsh);
+            for (auto it = range.first; it != range.second && form < 0; ++it) {
+                const int64_t o = off[(size_t)it->second], len = off[(size_t)it->second + 1] - o;
+                if (len == (int64_t)words.size() && std::equal(words.begin(), words.end(), sell.begin() + o)) form = it->second;
+            }
+            if (form < 0) {
+                form = (int32_t)off.size() - 1;
+                form_of.emplace(hsh, form);
+                sell.insert(sell.end(), words.begin(), words.end());
+                off.push_back((int64_t)sell.size());
+            }
+            slice[(size_t)s] = make_int2(form, (int)row0);
+        }
+    }
+    if (sell.empty()) sell.push_back(0);
+    SS_CUDA(h, dalloc(h, (void **)&h->sell, sell.size() * sizeof(uint32_t)));
+    SS_CUDA(h, dalloc(h, (void **)&h->sell_off, off.size() * sizeof(int64_t)));
+    SS_CUDA(h, dalloc(h, (void **)&h->slice, slice.size() * sizeof(int2)));
+    SS_CUDA(h, cudaMemcpyAsync(h->sell, sell.data(), sell.size() * sizeof(uint32_t), cudaMemcpyHostToDevice, h->stream));
+    SS_CUDA(h, cudaMemcpyAsync(h->sell_off, off.data(), off.size() * sizeof(int64_t), cudaMemcpyHostToDevice, h->stream));
+    SS_CUDA(h, cudaMemcpyAsync(h->slice, slice.data(), slice.size() * sizeof(int2), cudaMemcpyHostToDevice, h->stream));
+    SS_CUDA(h, cudaStreamSynchronize(h->stream));  // the host vectors go out of scope
+    h->nslice = nsl;
+    h->period = period;
+    return SS_OK;
+}
+
 // Packed bonds in columns for rows of at most kPatRow scalar bonds that have no row forms (see
-// ell_sum).  Without the memory for them, or with more distinct J or spins than a word holds, the
-// CSR is read.
+// ell_sum), written on the device from the CSR there.  Without the memory for them, or with more
+// distinct J or spins than a word holds, the CSR is read.
 template <typename R>
-ss_status build_ell(ss_system *h, const std::vector<int32_t> &rp, const std::vector<int32_t> &col,
-                    const std::vector<R> &J) {
+ss_status build_ell(ss_system *h, const std::vector<R> &J) {
     const int64_t n = h->n, nnz = h->nnz;
     if (h->npat > 0 || h->J_tensor || nnz <= 0 || h->max_row > kPatRow || n >= (int64_t(1) << 24)) return SS_OK;
     const int W = h->max_row <= kShortRow ? kShortRow : kPatRow;
-    std::vector<R> dict;
-    std::vector<uint8_t> bid;
-    int zero;
-    if (!bond_dictionary<R>(J, nnz, dict, bid, zero)) return SS_OK;
+    std::vector<R> dict(1, (R)0);  // entry 0: the padding
+    size_t last = 0;
+    for (int64_t k = 0; k < nnz; ++k) {
+        if (std::memcmp(&J[k], &dict[last], sizeof(R)) == 0) continue;  // (bonds of a row mostly repeat)
+        for (last = 0; last < dict.size() && std::memcmp(&J[k], &dict[last], sizeof(R)) != 0;) ++last;
+        if (last < dict.size()) continue;
+        if (dict.size() == 256) return SS_OK;
+        dict.push_back(J[k]);
+    }
     void *J_dev = nullptr;
     uint32_t *ell = nullptr;
     if (dalloc(h, (void **)&ell, (size_t)W * n * sizeof(uint32_t)) != cudaSuccess ||
@@ -1133,15 +1256,9 @@ ss_status build_ell(ss_system *h, const std::vector<int32_t> &rp, const std::vec
         if (ell) dfree(h, ell);
         return SS_OK;
     }
-    std::vector<uint32_t> words((size_t)W * n);
-    for (int64_t i = 0; i < n; ++i) {
-        const int32_t b = rp[i], len = rp[i + 1] - b;
-        for (int32_t k = 0; k < W; ++k)
-            words[(size_t)(k * n + i)] = k < len ? ((uint32_t)col[b + k] << 8) | bid[(size_t)(b + k)]
-                                                 : ((uint32_t)i << 8) | (uint32_t)zero;
-    }
-    SS_CUDA(h, cudaMemcpyAsync(ell, words.data(), words.size() * sizeof(uint32_t), cudaMemcpyHostToDevice, h->stream));
     SS_CUDA(h, cudaMemcpyAsync(J_dev, dict.data(), dict.size() * sizeof(R), cudaMemcpyHostToDevice, h->stream));
+    SS_CUDA(h, launch_build_ell<R>(h->row_ptr, h->col, static_cast<const R *>(h->J), static_cast<const R *>(J_dev),
+                                   (int)dict.size(), n, W, ell, h->stream));
     SS_CUDA(h, cudaStreamSynchronize(h->stream));  // the host vectors go out of scope
     h->ell = ell;
     h->ell_J = J_dev;
@@ -1269,36 +1386,12 @@ ss_status upload_system(ss_system *h, const std::vector<HostSys> &hs) {
         std::vector<uint8_t> bid;
         int zero = -1;
         if (bond_dictionary<R>(J, nnz, dict, bid, zero)) {
-            const int64_t nsl = (n + 31) / 32;
-            std::vector<int64_t> off((size_t)nsl + 1, 0);
-            for (int64_t s = 0; s < nsl; ++s) {
-                int32_t w = 0;
-                for (int64_t i = 32 * s; i < std::min<int64_t>(n, 32 * s + 32); ++i) w = std::max(w, rp[i + 1] - rp[i]);
-                off[(size_t)s + 1] = off[(size_t)s] + 32 * (int64_t)w;
-            }
-            std::vector<uint32_t> sell((size_t)std::max<int64_t>(off[(size_t)nsl], 1));
-            for (int64_t s = 0; s < nsl; ++s) {
-                const int64_t w = (off[(size_t)s + 1] - off[(size_t)s]) / 32;
-                for (int l = 0; l < 32; ++l) {
-                    const int64_t i = 32 * s + l;
-                    const int64_t len = i < n ? rp[i + 1] - rp[i] : 0;
-                    const uint32_t pad = ((uint32_t)(i < n ? i : 0) << 8) | (uint32_t)zero;
-                    for (int64_t k = 0; k < w; ++k)
-                        sell[(size_t)(off[(size_t)s] + 32 * k + l)] =
-                            k < len ? ((uint32_t)col[rp[i] + k] << 8) | bid[(size_t)(rp[i] + k)] : pad;
-                }
-            }
+            const ss_status ps = build_slices(h, rp, col, bid, zero);
+            if (ps != SS_OK) return ps;
             SS_CUDA(h, dalloc(h, &h->Jd, dict.size() * sizeof(R)));
-            SS_CUDA(h, dalloc(h, (void **)&h->sell, sell.size() * sizeof(uint32_t)));
-            SS_CUDA(h, dalloc(h, (void **)&h->sell_off, off.size() * sizeof(int64_t)));
             SS_CUDA(h, cudaMemcpyAsync(h->Jd, dict.data(), dict.size() * sizeof(R), cudaMemcpyHostToDevice, h->stream));
-            SS_CUDA(h, cudaMemcpyAsync(h->sell, sell.data(), sell.size() * sizeof(uint32_t), cudaMemcpyHostToDevice,
-                                       h->stream));
-            SS_CUDA(h, cudaMemcpyAsync(h->sell_off, off.data(), off.size() * sizeof(int64_t), cudaMemcpyHostToDevice,
-                                       h->stream));
             SS_CUDA(h, cudaStreamSynchronize(h->stream));
             h->nJd = (int)dict.size();
-            h->nslice = nsl;
         }
     }
     h->J_uniform = nnz > 0 && !tensor;
@@ -1325,7 +1418,7 @@ ss_status upload_system(ss_system *h, const std::vector<HostSys> &hs) {
                                h->stream));
     {
         ss_status ps = build_patterns<R>(h, rp, col, J, Jtidx);
-        if (ps == SS_OK) ps = build_ell<R>(h, rp, col, J);
+        if (ps == SS_OK) ps = build_ell<R>(h, J);
         if (ps != SS_OK) return ps;
     }
     for (int b = 0; b < 12; ++b) SS_CUDA(h, dalloc(h, &h->state[b], (size_t)n * rs));
@@ -1385,7 +1478,10 @@ ss_status set_rows(ss_system *h, int32_t mode) {
     if (on && !h->E[0]) {
         const size_t rs = real_size(h);
         for (int c = 0; c < 3; ++c) SS_CUDA(h, dalloc(h, &h->E[c], (size_t)h->n * rs));
-        if (h->sell) SS_CUDA(h, dalloc(h, &h->x4, 4 * (size_t)h->n * rs));
+        if (h->sell) {  // (the padding of the classes is gathered with J = 0: finite)
+            SS_CUDA(h, dalloc(h, &h->x4, 128 * (size_t)h->nslice * rs));
+            SS_CUDA(h, cudaMemsetAsync(h->x4, 0, 128 * (size_t)h->nslice * rs, h->stream));
+        }
     }
     h->rows_req = mode;
     if (on != h->rows) drop_graph(h);
@@ -1556,9 +1652,13 @@ ss_status create_impl(const ss_params *systems, int32_t count, ss_system **out, 
     if (st != SS_OK) return cleanup(st);
     st = h->precision == SS_FP32_MIXED ? init_random<float>(h, hs) : init_random<double>(h, hs);
     if (st != SS_OK) return cleanup(st);
-    if (h->precision == SS_FP32_MIXED && !slab &&
-        dalloc(h, &h->packed, (size_t)n * (3 * sizeof(float4) + sizeof(float2))) != cudaSuccess)
-        cudaGetLastError();  // not enough memory: the steps work on the arrays of `state`
+    if (h->precision == SS_FP32_MIXED && !slab) {
+        const size_t bytes = (size_t)packed_spins(h) * (3 * sizeof(float4) + sizeof(float2));
+        if (dalloc(h, &h->packed, bytes) != cudaSuccess)
+            cudaGetLastError();  // not enough memory: the steps work on the arrays of `state`
+        else if (h->nslice > 0 && (e = cudaMemsetAsync(h->packed, 0, bytes, h->stream)) != cudaSuccess)
+            return cleanup(cuda_fail(h, e, "cudaMemsetAsync"));  // (the classes' padding has to be finite)
+    }
     *out = h;
     return SS_OK;
 }

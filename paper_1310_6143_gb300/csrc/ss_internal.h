@@ -108,12 +108,17 @@ struct KArgs {
     int rows_bare;            // 1: the long-row passes write sum_j J_ij X_j alone (no H_app)
     R *ex, *ey, *ez;          // [n] exchange + applied field of the spins being updated, computed
                               // beforehand by k_rows_field (a warp per row), or nullptr
-    const uint32_t *sell;     // packed bonds col << 8 | entry of Jd in slices of 32 rows: bond k of
-                              // row 32 s + l at sell[sell_off[s] + 32 k + l], padded with J = 0;
-                              // or nullptr
-    const int64_t *sell_off;  // [nslice + 1]
+    const uint32_t *sell;     // packed bonds in slices of 32 rows (see k_rows_sell): bond k of a slice's
+                              // row l at sell[sell_off[form] + 32 k + l]: (x4 position of the neighbour -
+                              // that of the slice's first row, modulo 2^24) << 8 | entry of Jd; or nullptr
+    const int64_t *sell_off;  // [forms + 1]
+    const int2 *slice;        // [nslice] (form, first row) of each slice; row l is first + l * period
     int64_t nslice;
-    R *x4;                    // [4n] the spins read by the sliced pass, (x, y, z, 0) per spin
+    int period;               // the rows of a slice are this far apart
+    int period_rest;          // n mod period, and the slices of a class of ceil(n / period) and of
+    int period_hi, period_lo; // floor(n / period) rows (x4_pos)
+    R *x4;                    // [4 * 32 nslice] the spins read by the sliced pass, (x, y, z, 0) each, slice by
+                              // slice
     const R *Jd;              // [nJd <= 256] distinct J_ij / mu_s,i of the packed bonds (and 0)
     int nJd;
     const int32_t *mc_of;     // [n] macrocell of each spin (demagnetising field)
@@ -209,6 +214,12 @@ constexpr unsigned int kErrBounds = 4u;   // checked builds: an index out of its
 
 // Host helper (ss_api.cu): sets the message returned by ss_last_error(NULL).
 void set_global_error(const char *msg);
+
+// The columns of packed bonds (KArgs.ell, W words per row) of a CSR on the device; every J is in
+// the dictionary, whose entry 0 is the padding's 0.
+template <typename R>
+cudaError_t launch_build_ell(const int32_t *row_ptr, const int32_t *col, const R *J, const R *dict, int ndict,
+                             int64_t n, int W, uint32_t *ell, cudaStream_t s);
 
 // Launchers (ss_kernels_f32.cu / ss_kernels_f64.cu).
 template <typename R> cudaError_t launch_predictor(const KArgs<R> &a, int block, int grid, cudaStream_t s);

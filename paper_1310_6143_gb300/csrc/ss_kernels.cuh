@@ -24,6 +24,8 @@
 #include <cooperative_groups.h>
 #include <stdint.h>
 
+#include <type_traits>
+
 #include "ss_internal.h"
 #include "ss_ff.cuh"
 #include "ss_math.cuh"
@@ -166,6 +168,9 @@ struct Aos {
         z = v.z;
     }
 };
+
+template <typename R>
+__device__ __forceinline__ int64_t x4_pos(const KArgs<R> &a, int64_t i);
 
 // The row form of spin i (0 when the handle reads the CSR).
 template <typename R>
@@ -645,8 +650,9 @@ __device__ __forceinline__ void predictor_tile(const KArgs<R> &a, const TileDesc
         const int form = next_form;  // read a slot ahead: the chain form -> offsets -> spins starts at the offsets
         if (k + BS < td.count) next_form = form_of(a, i + BS);
         const MatDesc<R> &m = mat_at<Mode>(a, i);
+        const int64_t i4 = V4 && Mode == kRows ? x4_pos(a, i) : i;  // the row passes gather from s4 and p4
         R s0, s1, s2;
-        src.get(i, s0, s1, s2);
+        src.get(i4, s0, s1, s2);
         const bool given = sqrtT > (R)0 && (Split || rot >= pre_slot);  // drawn beforehand (k_gauss, or the
                                                                         // previous corrector)
         R g0 = 0, g1 = 0, g2 = 0;
@@ -688,7 +694,7 @@ __device__ __forceinline__ void predictor_tile(const KArgs<R> &a, const TileDesc
         const R inv = rsqrt_r(fma(v2, v2, fma(v1, v1, mul_rn(v0, v0))));
         const R hdt = (R)0.5 * dt;
         if constexpr (V4) {
-            a.p4[i] = make_float4(mul_rn(v0, inv), mul_rn(v1, inv), mul_rn(v2, inv), 0.0f);
+            a.p4[i4] = make_float4(mul_rn(v0, inv), mul_rn(v1, inv), mul_rn(v2, inv), 0.0f);
             a.qh4[i] = make_float4(fma(hdt, d0, s0), fma(hdt, d1, s1), fma(hdt, d2, s2), t0);
             a.qh2[i] = make_float2(t1, t2);
         } else {
@@ -733,8 +739,9 @@ __device__ __forceinline__ void corrector_tile(const KArgs<R> &a, const TileDesc
         const int form = next_form;  // a slot ahead, as the predictor
         if (k + BS < td.count) next_form = form_of(a, i + BS);
         const MatDesc<R> &m = mat_at<Mode>(a, i);
+        const int64_t i4 = V4 && Mode == kRows ? x4_pos(a, i) : i;
         R s0, s1, s2;
-        src.get(i, s0, s1, s2);
+        src.get(i4, s0, s1, s2);
         R q0, q1, q2, t0 = 0, t1 = 0, t2 = 0;  // the half step and the thermal field
         if constexpr (V4) {
             const float4 u = __ldg(a.qh4 + i);
@@ -780,7 +787,7 @@ __device__ __forceinline__ void corrector_tile(const KArgs<R> &a, const TileDesc
         const R inv = rsqrt_r(fma(v2, v2, fma(v1, v1, mul_rn(v0, v0))));
         if (bad_inv(inv)) atomicOr(a.err, kErrNonFinite);  // NaN or infinite length
         if constexpr (V4) {
-            a.s4[i] = make_float4(mul_rn(v0, inv), mul_rn(v1, inv), mul_rn(v2, inv), 0.0f);
+            a.s4[i4] = make_float4(mul_rn(v0, inv), mul_rn(v1, inv), mul_rn(v2, inv), 0.0f);
         } else {
             a.sx[i] = mul_rn(v0, inv);
             a.sy[i] = mul_rn(v1, inv);
@@ -881,14 +888,16 @@ __device__ __forceinline__ void predictor_pass(const KArgs<R> &a, uint64_t step,
     }
 }
 
-// The state at the start and at the end of a run of steps over float4 spins.
+// The state at the start and at the end of a run of steps over float4 spins (with long rows in the
+// order the row passes gather from).
 static __global__ void __launch_bounds__(256) k_pack_state(const KArgs<float> a) {
     for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < a.n; i += (int64_t)gridDim.x * 256)
-        a.s4[i] = make_float4(a.sx[i], a.sy[i], a.sz[i], 0.0f);
+        a.s4[a.ex ? x4_pos(a, i) : i] = make_float4(a.sx[i], a.sy[i], a.sz[i], 0.0f);
 }
 static __global__ void __launch_bounds__(256) k_unpack_state(const KArgs<float> a) {
     for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < a.n; i += (int64_t)gridDim.x * 256) {
-        const float4 s = a.s4[i], p = a.p4[i];
+        const int64_t at = a.ex ? x4_pos(a, i) : i;
+        const float4 s = a.s4[at], p = a.p4[at];
         a.sx[i] = s.x;
         a.sy[i] = s.y;
         a.sz[i] = s.z;
@@ -1248,19 +1257,39 @@ __global__ void __launch_bounds__(BS) k_system_blocks(const KArgs<R> a, long lon
 // 2: tensors.  (Packed scalar bonds go through k_rows_sell below.)
 // ----------------------------------------------------------------------------------
 // Packed bonds in slices (the scalar-J case with at most 255 distinct J_ij / mu_s,i): lane l
-// of the warp owning slice s sums row 32 s + l, all lanes stepping through bond k together,
-// so the bond words load coalesced and the neighbours' spins come as one 16-byte (FP32) or
-// 32-byte (FP64) gather from the (x, y, z, 0) copy.  Consecutive rows keep the slice's
-// neighbourhood compact (on a lattice numbered cell by cell, a few cells), which is what
-// L1 reuse of the gathered spins depends on.  Each row is summed in its CSR order from
-// H_app, like the thread-per-row sum (padding adds 0 * S exactly).
+// of the warp owning a slice sums its row l, all lanes stepping through bond k together, so the
+// bond words load coalesced and the neighbours' spins come as one 16-byte (FP32) or 32-byte (FP64)
+// gather from the (x, y, z, 0) copy.  Each row is summed in its CSR order from H_app, like the
+// thread-per-row sum (padding adds 0 * S exactly).
+//
+// The rows of a slice are `period` apart and the copy is laid out slice by slice, so that on a
+// lattice numbered cell by cell a slice holds one basis site of 32 cells and bond k of its rows
+// gathers one contiguous run of 512 bytes (FP32); with 32 consecutive rows (fcc: eight cells of
+// four sites) it touched 32 sectors and used half of each.  Words are relative to the slice, and
+// slices with the same words -- on a lattice, all those in the same position along the short axis
+// and away from the others' ends -- share them, which then come from the L2 instead of HBM (fcc
+// 32^3 to 4a: 556 -> 44 MB of words).  One FP32 pass there: 286 -> about 140 us, still waiting for
+// the gathers' L1 misses.  U bonds in flight a warp: 2 1.65, 3 1.36, 4 1.22, 8 1.32, 16 1.53 ms per four steps
+// (more evict each other's lines); words loaded past the L1 1.71, two slices to a warp 2.0 ms.
+//
+// Where spin i lies in the copy: class i mod period, then i / period, classes padded to whole slices.
+template <typename R>
+__device__ __forceinline__ int64_t x4_pos(const KArgs<R> &a, int64_t i) {
+    if (a.period == 1) return i;
+    const uint32_t c = (uint32_t)i / (uint32_t)a.period, b = (uint32_t)i - c * (uint32_t)a.period;
+    const int rest = a.period_rest, over = (int)b - rest;
+    const int first = over <= 0 ? (int)b * a.period_hi : rest * a.period_hi + over * a.period_lo;
+    return 32 * (int64_t)first + c;
+}
+
 template <typename R>
 __global__ void k_pack4(const KArgs<R> a, const R *X, const R *Y, const R *Z) {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < a.n; i += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t at = x4_pos(a, i);
         if constexpr (sizeof(R) == 4) {
-            reinterpret_cast<float4 *>(a.x4)[i] = make_float4(X[i], Y[i], Z[i], 0.f);
+            reinterpret_cast<float4 *>(a.x4)[at] = make_float4(X[i], Y[i], Z[i], 0.f);
         } else {
-            double2 *d = reinterpret_cast<double2 *>(a.x4) + 2 * i;
+            double2 *d = reinterpret_cast<double2 *>(a.x4) + 2 * at;
             d[0] = make_double2(X[i], Y[i]);
             d[1] = make_double2(Z[i], 0.0);
         }
@@ -1283,70 +1312,55 @@ __device__ __forceinline__ void load_spin4(const R *x4, int32_t j, R &s0, R &s1,
     }
 }
 
+// Threads per block of the sliced pass: two slices, so that the blocks spread evenly over the SMs
+// (fcc 32^3: 4,096 slices in blocks of eight left the busiest SM 32 for 27 on average).
+constexpr int kSellBlock = 64;
+
 template <typename R>
-__global__ void __launch_bounds__(256) k_rows_sell(const KArgs<R> a) {
+__global__ void __launch_bounds__(kSellBlock) k_rows_sell(const KArgs<R> a) {
     __shared__ R jd[256];
-    for (int t = threadIdx.x; t < a.nJd; t += blockDim.x) jd[t] = a.Jd[t];
+    for (int t = threadIdx.x; t < a.nJd; t += kSellBlock) jd[t] = a.Jd[t];
     __syncthreads();
+    constexpr int U = sizeof(R) == 8 ? 8 : 4;
     const int lane = threadIdx.x & 31;
-    const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    const int64_t warp = ((int64_t)blockIdx.x * kSellBlock + threadIdx.x) >> 5;
+    const int64_t nwarps = ((int64_t)gridDim.x * kSellBlock) >> 5;
+    const int64_t npos = 32 * a.nslice;
     for (int64_t s = warp; s < a.nslice; s += nwarps) {
-        const int64_t row = s * 32 + lane;
-        const int64_t o = __ldg(a.sell_off + s);
-        const int w = (int)((__ldg(a.sell_off + s + 1) - o) >> 5);
+        const int2 sl = __ldg(a.slice + s);
+        const int64_t row = sl.y + (int64_t)lane * a.period;
+        const uint32_t base = (uint32_t)(32 * s);
+        const int64_t o = __ldg(a.sell_off + sl.x);
+        const int w = (int)((__ldg(a.sell_off + sl.x + 1) - o) >> 5);
         const uint32_t *p = a.sell + o + lane;
         R x = 0, y = 0, z = 0;
-        const SysDesc *sd = nullptr;
         if (row < a.n && !a.rows_bare) {
-            sd = &a.sys[a.mats[mat_of(a, row)].sys];
-            x = sys_H(*sd, 0, R());
-            y = sys_H(*sd, 1, R());
-            z = sys_H(*sd, 2, R());
+            const SysDesc &sd = a.sys[a.mats[mat_of(a, row)].sys];
+            x = sys_H(sd, 0, R());
+            y = sys_H(sd, 1, R());
+            z = sys_H(sd, 2, R());
         }
-        if constexpr (sizeof(R) == 8) {
-            // FP64: eight bonds at a time, their words, then their gathers, then the sums in
-            // bond order (5.80 against 6.34 ms per pass on fcc 64^3 to 4a; sixteen at a time
-            // gives 5.83 ms; in FP32 the plain loop below is faster, 1.52 against 1.70 ms with
-            // eight and 1.99 ms with four)
-            constexpr int U = 8;
-            int k = 0;
-            for (; k + U <= w; k += U) {
-                uint32_t bw[U];
+        // U bonds at a time: their words, then their gathers, then the sums in bond order
+        auto bonds = [&](int k, auto count) {
+            constexpr int N = decltype(count)::value;
+            uint32_t bw[N];
 #pragma unroll
-                for (int u = 0; u < U; ++u) bw[u] = __ldg(p + 32 * (int64_t)(k + u));
-                R s0[U], s1[U], s2[U];
+            for (int u = 0; u < N; ++u) bw[u] = __ldg(p + 32 * (int64_t)(k + u));
+            R s0[N], s1[N], s2[N];
 #pragma unroll
-                for (int u = 0; u < U; ++u) load_spin4(a.x4, chk(bw[u] >> 8, a.n, a.err), s0[u], s1[u], s2[u]);
+            for (int u = 0; u < N; ++u)
+                load_spin4(a.x4, chk((base + (bw[u] >> 8)) & 0xFFFFFFu, npos, a.err), s0[u], s1[u], s2[u]);
 #pragma unroll
-                for (int u = 0; u < U; ++u) {
-                    const R Jk = jd[chk(bw[u] & 255u, a.nJd, a.err)];
-                    x = fma(Jk, s0[u], x);
-                    y = fma(Jk, s1[u], y);
-                    z = fma(Jk, s2[u], z);
-                }
+            for (int u = 0; u < N; ++u) {
+                const R Jk = jd[chk(bw[u] & 255u, a.nJd, a.err)];
+                x = fma(Jk, s0[u], x);
+                y = fma(Jk, s1[u], y);
+                z = fma(Jk, s2[u], z);
             }
-            for (; k < w; ++k) {
-                const uint32_t b = __ldg(p + 32 * (int64_t)k);
-                const R Jk = jd[chk(b & 255u, a.nJd, a.err)];
-                R s0, s1, s2;
-                load_spin4(a.x4, chk(b >> 8, a.n, a.err), s0, s1, s2);
-                x = fma(Jk, s0, x);
-                y = fma(Jk, s1, y);
-                z = fma(Jk, s2, z);
-            }
-        } else {
-#pragma unroll 8
-            for (int k = 0; k < w; ++k) {
-                const uint32_t b = __ldg(p + 32 * (int64_t)k);
-                const R Jk = jd[chk(b & 255u, a.nJd, a.err)];
-                R s0, s1, s2;
-                load_spin4(a.x4, chk(b >> 8, a.n, a.err), s0, s1, s2);
-                x = fma(Jk, s0, x);
-                y = fma(Jk, s1, y);
-                z = fma(Jk, s2, z);
-            }
-        }
+        };
+        int k = 0;
+        for (; k + U <= w; k += U) bonds(k, std::integral_constant<int, U>());
+        for (; k < w; ++k) bonds(k, std::integral_constant<int, 1>());
         if (row < a.n) {
             a.ex[row] = x;
             a.ey[row] = y;

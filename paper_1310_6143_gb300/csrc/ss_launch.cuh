@@ -450,14 +450,16 @@ cudaError_t launch_sib(const KArgs<R> &a, const AltGrids &g, cudaStream_t s) {
 
 template <typename R>
 cudaError_t launch_rows_field(const KArgs<R> &a, const R *X, const R *Y, const R *Z, int grid, cudaStream_t s) {
-    if (a.sell && !X) {  // the caller's spins are float4 already (a.x4)
-        k_rows_sell<R><<<grid, 256, 0, s>>>(a);
-    } else if (a.sell) {
-        const int64_t pb = (a.n + 255) / 256;
-        k_pack4<R><<<(int)(pb < 4 * (int64_t)grid ? pb : 4 * (int64_t)grid), 256, 0, s>>>(a, X, Y, Z);
-        cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess) return e;
-        k_rows_sell<R><<<grid, 256, 0, s>>>(a);
+    if (a.sell) {
+        if (X) {  // (else the caller's spins are in x4 already)
+            const int64_t pb = (a.n + 255) / 256;
+            k_pack4<R><<<(int)(pb < 4 * (int64_t)grid ? pb : 4 * (int64_t)grid), 256, 0, s>>>(a, X, Y, Z);
+            const cudaError_t e = cudaGetLastError();
+            if (e != cudaSuccess) return e;
+        }
+        const int64_t blocks = (a.nslice + kSellBlock / 32 - 1) / (kSellBlock / 32);
+        const int64_t most = (int64_t)1 << 20;
+        k_rows_sell<R><<<(int)(blocks < most ? blocks : most), kSellBlock, 0, s>>>(a);
     } else if (a.J_tensor)
         k_rows_field<R, 2><<<grid, 256, 0, s>>>(a, X, Y, Z);
     else
