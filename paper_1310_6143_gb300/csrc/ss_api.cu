@@ -160,6 +160,7 @@ struct ss_system {
     // record summed in the colour passes (at most two colour classes): per class its tiles
     // (runs of mc_order within one system) and their partial slots, slots system by system
     bool mc_rec = false;
+    bool mc_small = false;                   // small classes: 64-trial tiles
     TileDesc *mc_tiles[2] = {};
     int32_t *mc_slot[2] = {};
     int64_t mc_ntiles[2] = {};
@@ -1745,8 +1746,7 @@ ss_status heun_pass_impl(ss_system *h, int32_t pass, int64_t tile0, int64_t ntil
     KArgs<R> a = make_args<R>(h);
     if (pass == 2) {  // the step's record from every tile's partials, then the next step
         SS_CUDA(h, launch_finalize_ring(h->sys, h->sys_tiles, h->nsys, h->partials, h->rec, h->rec_cap, h->ctl,
-                                        h->stream));
-        SS_CUDA(h, launch_advance_step(h->ctl, h->stream));
+                                        a.ticket, h->stream));
         h->step += 1;
         return SS_OK;
     }
@@ -1933,10 +1933,24 @@ ss_status mc_prepare(ss_system *h) {
     SS_CUDA(h, cudaMemcpyAsync(dorder, order.data(), order.size() * sizeof(int32_t), cudaMemcpyHostToDevice,
                                h->stream));
     if (ncol <= 2 && n > 0) {
-        // tiles of at most `tile` trials within one system, per colour class (1,024, or 256 when
-        // a class would give fewer than four tiles per SM); partial slots system by system
-        // (class 0's tiles of the system, then class 1's)
-        const int64_t kMcTile = h->mc_cstart[1] >= (int64_t)h->sm_count * 4 * 1024 ? 1024 : 256;
+        // tiles of at most `tile` trials within one system, per colour class; partial slots system by
+        // system (class 0's tiles of the system, then class 1's).  Classes of fewer than 256 trials
+        // per SM take 64 (k_mc_colour_rec), others whole 256-thread rounds, as many as leave the
+        // busiest SM the least to do (as default_shape).
+        const int64_t sms = std::max(h->sm_count, 1), most = h->mc_cstart[1];
+        h->mc_small = most < 256 * sms;
+        int64_t kMcTile = 64;
+        if (!h->mc_small) {
+            double least = 1e300;
+            for (int r = 1; r <= 10; ++r) {
+                const int64_t tiles = (most + 256 * r - 1) / (256 * r);
+                const double cost = (double)((tiles + sms - 1) / sms) * (r + 0.3);
+                if (cost < least) {
+                    least = cost;
+                    kMcTile = 256 * r;
+                }
+            }
+        }
         std::vector<TileDesc> tl[2];
         std::vector<int32_t> sl[2];
         std::vector<int32_t> sys_slots((size_t)h->nsys + 1, 0);
@@ -2150,6 +2164,9 @@ cudaError_t enqueue_mc(ss_system *h, int64_t nsteps) {
     cudaError_t e = cudaSuccess;
     if (h->mc_rec && !h->rows) {  // the record summed in the colour passes
         m.partials = h->mc_partials;
+        m.sys_slots = h->mc_sys_slots;
+        const bool inline_rec = h->nsys <= kMcInlineSystems;
+        const int64_t wave = (int64_t)h->sm_count * std::max(1, mc_rec_blocks_per_sm<R>(own_rows_mode(h)));
         for (int64_t k = 0; k < nsteps && e == cudaSuccess; ++k) {
             for (int c = 0; c < ncol && e == cudaSuccess; ++c) {
                 m.c0 = h->mc_cstart[c];
@@ -2158,14 +2175,13 @@ cudaError_t enqueue_mc(ss_system *h, int64_t nsteps) {
                 m.slot = h->mc_slot[c];
                 m.ntiles = h->mc_ntiles[c];
                 m.first = c == 0 ? 1 : 0;
-                if (m.ntiles == 0) continue;
-                const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(m.ntiles, resident));
-                e = launch_mc_colour_rec<R>(a, m, grid, h->stream);
+                m.last = inline_rec && c == ncol - 1 ? 1 : 0;  // (every class has a spin)
+                const int grid = (int)std::max<int64_t>(1, h->mc_small ? m.ntiles : std::min<int64_t>(m.ntiles, wave));
+                e = launch_mc_colour_rec<R>(a, m, h->mc_small, grid, h->stream);
             }
-            if (e == cudaSuccess)
+            if (e == cudaSuccess && !inline_rec)
                 e = launch_finalize_ring(h->sys, h->mc_sys_slots, h->nsys, h->mc_partials, h->rec, h->rec_cap, a.step,
-                                         h->stream);
-            if (e == cudaSuccess) e = launch_advance_step(a.step, h->stream);
+                                         a.ticket, h->stream);
         }
         return e;
     }
@@ -2182,7 +2198,8 @@ cudaError_t enqueue_mc(ss_system *h, int64_t nsteps) {
         if (h->rows) e = launch_rows_field<R>(ar, ar.sx, ar.sy, ar.sz, rgrid, h->stream);
         if (e == cudaSuccess) e = launch_measure<R>(ar, h->block, gmeas, h->stream);
         if (e == cudaSuccess)
-            e = launch_finalize_ring(h->sys, h->sys_tiles, h->nsys, h->partials, h->rec, h->rec_cap, a.step, h->stream);
+            e = launch_finalize_ring(h->sys, h->sys_tiles, h->nsys, h->partials, h->rec, h->rec_cap, a.step, nullptr,
+                                     h->stream);
         if (h->rows && e == cudaSuccess) e = launch_mc_prep<R>(a, m, h->stream);
         for (int c = 0; c < ncol && e == cudaSuccess; ++c) {
             m.c0 = h->mc_cstart[c];

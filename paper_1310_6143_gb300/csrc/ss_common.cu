@@ -22,10 +22,12 @@ cudaError_t launch_finalize(const SysDesc *sys, const int32_t *sys_tiles, int ns
     return cudaGetLastError();
 }
 
+// ticket: the launch ends the step (see k_finalize_ring), or nullptr.
 cudaError_t launch_finalize_ring(const SysDesc *sys, const int32_t *sys_tiles, int nsys, const double *partials,
-                                 double *rec, int64_t rec_cap, const unsigned long long *step, cudaStream_t s) {
+                                 double *rec, int64_t rec_cap, unsigned long long *step, unsigned int *ticket,
+                                 cudaStream_t s) {
     const int grid = nsys < 1024 ? nsys : 1024;
-    k_finalize_ring<256><<<grid > 0 ? grid : 1, 256, 0, s>>>(sys, sys_tiles, nsys, partials, rec, rec_cap, step);
+    k_finalize_ring<256><<<grid > 0 ? grid : 1, 256, 0, s>>>(sys, sys_tiles, nsys, partials, rec, rec_cap, step, ticket);
     return cudaGetLastError();
 }
 

@@ -193,7 +193,12 @@ struct McArgs {
     int64_t ntiles;
     double *partials;         // [slots * kPartComps]
     int first;                // 1: the first class (its rows' bonds are summed, both ends unchanged)
+    int last;                 // 1: the launch ends the step (record and step counter)
+    const int32_t *sys_slots; // [nsys + 1] first partial slot of each system
 };
+
+// Colour passes that end a step sum the record of at most this many systems.
+constexpr int kMcInlineSystems = 8;
 
 // Macrocell demagnetising field (Section "Demagnetising fields").
 struct DemagArgs {
@@ -255,7 +260,10 @@ template <typename R> cudaError_t launch_mc_colour_warp(const KArgs<R> &a, const
 // The trial randoms of the device's current step for every spin (McArgs.pre_*).
 template <typename R> cudaError_t launch_mc_prep(const KArgs<R> &a, const McArgs &m, cudaStream_t s);
 // One colour pass over the tiles of m that also sums the record terms of the pre-step state.
-template <typename R> cudaError_t launch_mc_colour_rec(const KArgs<R> &a, const McArgs &m, int grid, cudaStream_t s);
+// small: 64-thread blocks for classes of few trials.
+template <typename R> cudaError_t launch_mc_colour_rec(const KArgs<R> &a, const McArgs &m, bool small, int grid,
+                                                       cudaStream_t s);
+template <typename R> int mc_rec_blocks_per_sm(int mode);  // (the 256-thread pass)
 template <typename R> cudaError_t launch_mc_colour(const KArgs<R> &a, const McArgs &m, int block, int grid,
                                                    cudaStream_t s);
 template <typename R> int mc_blocks_per_sm(int block, int mode);  // mode: kPlain or kGeneral
@@ -283,7 +291,8 @@ cudaError_t launch_rows_field(const KArgs<R> &a, const R *X, const R *Y, const R
 template <typename R> int rows_blocks_per_sm();
 // The record of the current device step (ring entry step % rec_cap).
 cudaError_t launch_finalize_ring(const SysDesc *sys, const int32_t *sys_tiles, int nsys, const double *partials,
-                                 double *rec, int64_t rec_cap, const unsigned long long *step, cudaStream_t s);
+                                 double *rec, int64_t rec_cap, unsigned long long *step, unsigned int *ticket,
+                                 cudaStream_t s);
 cudaError_t launch_finalize(const SysDesc *sys, const int32_t *sys_tiles, int nsys, const double *partials,
                             double *dst, cudaStream_t s);
 cudaError_t launch_debug_philox(const uint32_t *ctr0, const uint32_t *key, long long count, uint32_t *out,

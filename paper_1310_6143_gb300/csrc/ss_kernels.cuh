@@ -1097,15 +1097,25 @@ __global__ void __launch_bounds__(BS) k_measure(const KArgs<R> a) {
 }
 
 // As k_finalize, into the record ring's entry of the current device step (so that the
-// launch holds no host-side step and can be captured once and replayed).
+// launch holds no host-side step and can be captured once and replayed).  With a ticket the
+// last block advances the step counter: the launch ends the step.
 template <int BS>
 __global__ void __launch_bounds__(BS) k_finalize_ring(const SysDesc *sys, const int32_t *sys_tiles, int nsys,
                                                       const double *partials, double *rec, int64_t rec_cap,
-                                                      const unsigned long long *step) {
+                                                      unsigned long long *step, unsigned int *ticket) {
     __shared__ double red[(BS / 32) * 8];
-    double *dst = rec + (int64_t)(*step % (unsigned long long)rec_cap) * nsys * kRecComps;
+    const unsigned long long now = *step;
+    double *dst = rec + (int64_t)(now % (unsigned long long)rec_cap) * nsys * kRecComps;
     for (int s = blockIdx.x; s < nsys; s += gridDim.x)
         finalize_system<BS, false, true>(sys, sys_tiles, partials, s, dst + (int64_t)s * kRecComps, red);
+    if (ticket && threadIdx.x == 0) {
+        __threadfence();
+        if (atomicAdd(ticket, 1u) == gridDim.x - 1) {
+            *ticket = 0u;
+            *step = now + 1ull;
+            __threadfence();
+        }
+    }
 }
 
 template <int BS>
@@ -1799,11 +1809,12 @@ __device__ __forceinline__ const SmemTables &fp64_tables(const KArgs<float> &a, 
 }
 
 // The random part of spin i's trial at `step`: the move type (0 flip, 1 Gaussian, 2 random),
-// the Gaussian triple (drawn for moves 1 and 2) and the acceptance factor -(-2 ln u)/2.
+// the Gaussian triple (drawn for moves 1 and 2) and the acceptance word.
 template <typename R>
 __device__ __forceinline__ int mc_randoms(const KArgs<R> &a, int64_t i, uint64_t step, const StepTabT<R> &tab,
-                                          R &g0, R &g1, R &g2, double &lnu) {
-    const SysDesc &sd = a.sys[a.mats[mat_of(a, i)].sys];
+                                          R &g0, R &g1, R &g2, uint32_t &w1) {
+    const MatDesc<R> &mt = a.mats[mat_of(a, i)];
+    const SysDesc &sd = a.sys[mt.sys];
     const uint32_t spin = (uint32_t)(i - sd.offset + sd.pbase);
     const Philox4 wa = philox4x32_10(spin, (uint32_t)step, sd.ctr2, 2u, sd.key0, sd.key1);
     const Philox4 wb = philox4x32_10(spin, (uint32_t)step, sd.ctr2, 3u, sd.key0, sd.key1);
@@ -1815,13 +1826,40 @@ __device__ __forceinline__ int mc_randoms(const KArgs<R> &a, int64_t i, uint64_t
             gaussians_f32(wa, tab, a.tab, g0, g1, g2);
         }
     }
-    lnu = -0.5 * neg2log_u(wb.w1, fp64_tables(a, tab));
+    w1 = wb.w1;
     return move;
+}
+
+// The acceptance factor of a word, ln u = -(-2 ln u)/2.
+template <typename R>
+__device__ __forceinline__ double mc_lnu(const KArgs<R> &a, const StepTabT<R> &tab, uint32_t w1) {
+    return -0.5 * neg2log_u(w1, fp64_tables(a, tab));
+}
+
+// dE <= -kB T ln u (mkT = -kB T; at T = 0 dE <= 0).  The FP32-mixed form decides by the single-
+// precision logarithm wherever that is certain: __logf is documented to 2^-21.4 absolute on
+// [0.5, 2] and 3 ulp elsewhere, and u's own rounding adds 6e-8, so kB T (1 + |ln u|) 1e-5 is over
+// ten times the threshold's error.  About one trial in 10^5 falls inside it and takes the FP64
+// logarithm, so every decision is the FP64 one.
+__device__ __forceinline__ bool mc_accept(const KArgs<double> &a, const SmemTables &tab, double mkT, double dE,
+                                          uint32_t w1) {
+    return mkT < 0.0 ? dE <= mkT * mc_lnu(a, tab, w1) : dE <= 0.0;
+}
+static __device__ __noinline__ bool mc_accept_fp64(const double2 *tab, double mkT, double dE, uint32_t w1) {
+    return dE <= mkT * (-0.5 * neg2log_u(w1, *reinterpret_cast<const SmemTables *>(tab)));
+}
+__device__ __forceinline__ bool mc_accept(const KArgs<float> &a, const FFTables &, double mkT, float dE, uint32_t w1) {
+    if (!(mkT < 0.0)) return dE <= 0.0f;
+    const float kT = -narrow_any<float>(mkT);
+    const float l = -__logf(fmaf((float)w1, 0x1p-32f, 0x1p-33f));
+    const float d = dE - kT * l;
+    if (kT > 1e-30f && fabsf(d) > kT * fmaf(l, 1e-5f, 1e-5f)) return d < 0.0f;
+    return mc_accept_fp64(a.tab, mkT, widen(dE), w1);
 }
 
 template <typename R, int Mode, int Rec, bool GivenH = false, bool Pre = false>
 __device__ __forceinline__ bool mc_trial(const KArgs<R> &a, const McArgs &m, int64_t i, uint64_t step,
-                                         const StepTabT<R> *tab, int &sysid, double v[5], R gh0 = 0, R gh1 = 0,
+                                         const StepTabT<R> *tab, int &sysid, R v[5], R gh0 = 0, R gh1 = 0,
                                          R gh2 = 0) {
     bool accept;
     const MatDesc<R> &mt = a.mats[mat_of(a, i)];
@@ -1835,7 +1873,8 @@ __device__ __forceinline__ bool mc_trial(const KArgs<R> &a, const McArgs &m, int
         par = m.par_sys[mt.sys];
     }
     R g0 = (R)0, g1 = (R)0, g2 = (R)0;
-    double lnu;
+    double lnu = 0.0;
+    uint32_t w1 = 0;
     int move;
     if constexpr (Pre) {  // drawn beforehand by k_mc_prep
         move = m.pre_move[i];
@@ -1845,7 +1884,7 @@ __device__ __forceinline__ bool mc_trial(const KArgs<R> &a, const McArgs &m, int
         g2 = pg[2 * a.n + i];
         lnu = m.pre_acc[i];
     } else {
-        move = mc_randoms(a, i, step, *tab, g0, g1, g2, lnu);
+        move = mc_randoms(a, i, step, *tab, g0, g1, g2, w1);
     }
     const R s0 = a.sx[i], s1 = a.sy[i], s2 = a.sz[i];
     R n0, n1, n2;
@@ -1900,23 +1939,27 @@ __device__ __forceinline__ bool mc_trial(const KArgs<R> &a, const McArgs &m, int
         dE -= d0 * k0 + d1 * k1 + d2 * k2;
     }
     // accept when dE <= -kB T ln u = (-kB T)(-1/2)(-2 ln u); at T = 0 when dE <= 0
-    const double dEd = widen(dE);
-    accept = par.x < 0.0 ? dEd <= par.x * lnu : dEd <= 0.0;
+    if constexpr (Pre) {
+        const double dEd = widen(dE);
+        accept = par.x < 0.0 ? dEd <= par.x * lnu : dEd <= 0.0;
+    } else {
+        accept = mc_accept(a, *tab, par.x, dE, w1);
+    }
     if (accept) {
         a.sx[i] = n0;
         a.sy[i] = n1;
         a.sz[i] = n2;
     }
-    if constexpr (Rec != 0) {  // terms in the working type, summed in FP64 (as spin_terms)
+    if constexpr (Rec != 0) {  // (as spin_terms_r)
         const R mu = mt.mu;
-        v[0] = widen(mu * s0);
-        v[1] = widen(mu * s1);
-        v[2] = widen(mu * s2);
+        v[0] = mu * s0;
+        v[1] = mu * s1;
+        v[2] = mu * s2;
         const R sh = s0 * sys_H(sd, 0, R()) + s1 * sys_H(sd, 1, R()) + s2 * sys_H(sd, 2, R());  // S.H_app
         if (Rec == 1)
-            v[3] = widen(-mu * (s0 * h0 + s1 * h1 + s2 * h2) + (R)0.5 * mu * sh);
+            v[3] = -mu * (s0 * h0 + s1 * h1 + s2 * h2) + (R)0.5 * mu * sh;
         else
-            v[3] = widen((R)-0.5 * mu * sh);
+            v[3] = (R)-0.5 * mu * sh;
         const R se = s0 * mt.e[0] + s1 * mt.e[1] + s2 * mt.e[2];
         R ea = -mt.ku * se * se;
         if (Mode != kPlain && mt.has_cubic) {
@@ -1927,21 +1970,21 @@ __device__ __forceinline__ bool mc_trial(const KArgs<R> &a, const McArgs &m, int
             ea -= mt.K[0] * s0 * s0 + mt.K[1] * s1 * s1 + mt.K[2] * s2 * s2
                 + (R)2 * (mt.K[3] * s0 * s1 + mt.K[4] * s0 * s2 + mt.K[5] * s1 * s2);
         }
-        v[4] = widen(ea);
+        v[4] = ea;
     }
     sysid = mt.sys;
     return accept;
 }
 
 template <typename R, int BS, int Mode = kGeneral>
-__global__ void __launch_bounds__(BS, sizeof(R) == 4 ? 1024 / BS : 1) k_mc_colour(const KArgs<R> a, const McArgs m) {
+__global__ void __launch_bounds__(BS, (sizeof(R) == 4 ? 1024 : 512) / BS) k_mc_colour(const KArgs<R> a, const McArgs m) {
     __shared__ StepTabT<R> tab;
     stage_step_tables(a, tab);
     __syncthreads();
     const uint64_t step = *a.step;
     for (int64_t k = m.c0 + (int64_t)blockIdx.x * BS + threadIdx.x; k < m.c1; k += (int64_t)gridDim.x * BS) {
         int sysid;
-        double v[5];
+        R v[5];
         const bool accept = mc_trial<R, Mode, 0>(a, m, chk(__ldg(m.order + k), a.n, a.err), step, &tab, sysid, v);
         // accepted moves per system, one atomic per (warp, system)
         const unsigned act = __activemask();
@@ -2004,12 +2047,12 @@ __global__ void __launch_bounds__(BS, sizeof(R) == 4 ? 1024 / BS : 1) k_mc_prep(
     double *pa = const_cast<double *>(m.pre_acc);
     for (int64_t i = (int64_t)blockIdx.x * BS + threadIdx.x; i < a.n; i += (int64_t)gridDim.x * BS) {
         R g0 = (R)0, g1 = (R)0, g2 = (R)0;
-        double lnu;
-        mv[i] = (uint8_t)mc_randoms(a, i, step, tab, g0, g1, g2, lnu);
+        uint32_t w1;
+        mv[i] = (uint8_t)mc_randoms(a, i, step, tab, g0, g1, g2, w1);
         pg[i] = g0;
         pg[a.n + i] = g1;
         pg[2 * a.n + i] = g2;
-        pa[i] = lnu;
+        pa[i] = mc_lnu(a, tab, w1);
     }
 }
 
@@ -2063,7 +2106,7 @@ __global__ void __launch_bounds__(BS) k_mc_colour_warp(const KArgs<R> a, const M
         int sysid = -1;
         if (i >= 0) {
             const SysDesc &sd = a.sys[a.mats[mat_of(a, i)].sys];
-            double v[5];
+            R v[5];
             accept = mc_trial<R, Mode, 0, true, true>(a, m, i, step, nullptr, sysid, v, sys_H(sd, 0, R()) + mx,
                                                  sys_H(sd, 1, R()) + my, sys_H(sd, 2, R()) + mz);
         }
@@ -2109,7 +2152,7 @@ __global__ void __launch_bounds__(BS) k_mc_colour_warp1(const KArgs<R> a, const 
         if (lane == 0) {
             const SysDesc &sd = a.sys[a.mats[mat_of(a, i)].sys];
             int sysid;
-            double v[5];
+            R v[5];
             const bool accept = mc_trial<R, Mode, 0, true, true>(a, m, i, step, nullptr, sysid, v, sys_H(sd, 0, R()) + x,
                                                            sys_H(sd, 1, R()) + y, sys_H(sd, 2, R()) + z);
             if (accept) atomicAdd(m.acc + sysid, 1ull);
@@ -2118,31 +2161,64 @@ __global__ void __launch_bounds__(BS) k_mc_colour_warp1(const KArgs<R> a, const 
 }
 
 // A colour pass tile by tile that also sums the record terms of the pre-step state of its
-// spins (tile partials in the block's fixed order), for lattices of at most two classes.
-template <typename R, int BS, int Mode, bool First>
-__global__ void __launch_bounds__(BS, sizeof(R) == 4 ? 1024 / BS : 1) k_mc_colour_rec(const KArgs<R> a, const McArgs m) {
-    __shared__ StepTabT<R> tab;
+// spins (tile partials in the block's fixed order), for lattices of at most two classes.  The
+// last pass of a step also ends it (m.last): its last block sums the record of up to
+// kMcInlineSystems systems and advances the step counter, which as launches of their own took
+// 17 + 4 of 274 us on a 512 x 512 x 16 film and 8 + 4 of 54 on sc 28^3 in FP64 (ncu).
+//
+// Small classes take 64-thread blocks that read the transform's tables where they lie: a trial is a
+// chain of some 90 FP64 instructions, which an SM sub-partition issues one in 64 cycles, so the
+// trials are spread over every SM, and 64 trials do not repay copying 40 KB of tables.
+template <typename R, int BS, int Mode, bool First, bool Staged>
+__global__ void __launch_bounds__(BS, (sizeof(R) == 4 ? 1024 : 512) / BS) k_mc_colour_rec(const KArgs<R> a, const McArgs m) {
     __shared__ double red[(BS / 32) * 8];
-    stage_step_tables(a, tab);
-    __syncthreads();
+    const StepTabT<R> *tab;
+    if constexpr (Staged) {
+        __shared__ StepTabT<R> copy;
+        stage_step_tables(a, copy);
+        __syncthreads();
+        tab = &copy;
+    } else if constexpr (sizeof(R) == 8) {
+        tab = reinterpret_cast<const StepTabT<R> *>(a.tab);
+    } else {
+        tab = reinterpret_cast<const StepTabT<R> *>(a.fftab);
+    }
     const uint64_t step = *a.step;
     for (int64_t t = blockIdx.x; t < m.ntiles; t += gridDim.x) {
         const TileDesc td = m.tiles[t];
-        double acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+        TermAcc<R> ta;
+        ta.reset();
         for (int k = threadIdx.x; k < td.count; k += BS) {
             int sysid;
-            double v[5];
+            R v[5];
             const bool accept = mc_trial<R, Mode, First ? 1 : 2>(a, m, chk(__ldg(m.order + td.start + k), a.n, a.err),
-                                                                 step, &tab, sysid, v);
-#pragma unroll
-            for (int c = 0; c < 5; ++c) acc[c] += v[c];
+                                                                 step, tab, sysid, v);
+            ta.add(v);
             // a tile lies in one system: one atomic per warp
             const unsigned act = __activemask();
             const unsigned yes = __ballot_sync(act, accept);
             if ((int)(threadIdx.x & 31) == __ffs(act) - 1) atomicAdd(m.acc + sysid, (unsigned long long)__popc(yes));
         }
+        double acc[8];
+        ta.out(acc);
         const double r = block_sum8<BS>(acc, red);
         if (threadIdx.x < kPartComps) m.partials[(int64_t)m.slot[t] * kPartComps + threadIdx.x] = r;
+    }
+    if (!m.last) return;
+    __shared__ bool ends;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) ends = atomicAdd(a.ticket, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!ends) return;
+    __threadfence();  // every other block's partials
+    double *dst = a.rec + (int64_t)(step % (uint64_t)a.rec_cap) * a.nsys * kRecComps;
+    for (int s = 0; s < a.nsys; ++s)
+        finalize_system<BS, true>(a.sys, m.sys_slots, m.partials, s, dst + (int64_t)s * kRecComps, red);
+    if (threadIdx.x == 0) {
+        *a.ticket = 0u;
+        *a.step = step + 1ull;
+        __threadfence();
     }
 }
 

@@ -335,21 +335,34 @@ cudaError_t launch_mc_prep(const KArgs<R> &a, const McArgs &m, cudaStream_t s) {
 }
 
 template <typename R>
-cudaError_t launch_mc_colour_rec(const KArgs<R> &a, const McArgs &m, int grid, cudaStream_t s) {
-    constexpr int BS = 256;
+cudaError_t launch_mc_colour_rec(const KArgs<R> &a, const McArgs &m, bool small, int grid, cudaStream_t s) {
+#define SS_MC_REC(MODE, FIRST)                                                       \
+    if (small)                                                                       \
+        k_mc_colour_rec<R, 64, MODE, FIRST, false><<<grid, 64, 0, s>>>(a, m);        \
+    else                                                                             \
+        k_mc_colour_rec<R, 256, MODE, FIRST, true><<<grid, 256, 0, s>>>(a, m);
     const bool general = a.J_tensor || a.any_cubic;
-    if (m.first) {
-        if (general)
-            k_mc_colour_rec<R, BS, kGeneral, true><<<grid, BS, 0, s>>>(a, m);
-        else
-            k_mc_colour_rec<R, BS, kPlain, true><<<grid, BS, 0, s>>>(a, m);
+    if (m.first && general) {
+        SS_MC_REC(kGeneral, true)
+    } else if (m.first) {
+        SS_MC_REC(kPlain, true)
+    } else if (general) {
+        SS_MC_REC(kGeneral, false)
     } else {
-        if (general)
-            k_mc_colour_rec<R, BS, kGeneral, false><<<grid, BS, 0, s>>>(a, m);
-        else
-            k_mc_colour_rec<R, BS, kPlain, false><<<grid, BS, 0, s>>>(a, m);
+        SS_MC_REC(kPlain, false)
     }
+#undef SS_MC_REC
     return cudaGetLastError();
+}
+
+template <typename R>
+int mc_rec_blocks_per_sm(int mode) {
+    int nb = 0;
+    const cudaError_t e =
+        mode == kPlain
+            ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_mc_colour_rec<R, 256, kPlain, true, true>, 256, 0)
+            : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_mc_colour_rec<R, 256, kGeneral, true, true>, 256, 0);
+    return e == cudaSuccess ? nb : 0;
 }
 
 template <typename R>
@@ -540,7 +553,8 @@ template int persistent_blocks_per_sm<SS_REAL>(int, int);
 template cudaError_t launch_demag<SS_REAL>(const KArgs<SS_REAL> &, const DemagArgs &, cudaStream_t);
 #elif SS_PART == 3  // Monte Carlo and the alternative integrators
 template cudaError_t launch_mc_colour<SS_REAL>(const KArgs<SS_REAL> &, const McArgs &, int, int, cudaStream_t);
-template cudaError_t launch_mc_colour_rec<SS_REAL>(const KArgs<SS_REAL> &, const McArgs &, int, cudaStream_t);
+template cudaError_t launch_mc_colour_rec<SS_REAL>(const KArgs<SS_REAL> &, const McArgs &, bool, int, cudaStream_t);
+template int mc_rec_blocks_per_sm<SS_REAL>(int);
 template cudaError_t launch_mc_colour_warp<SS_REAL>(const KArgs<SS_REAL> &, const McArgs &, int, cudaStream_t);
 template cudaError_t launch_mc_prep<SS_REAL>(const KArgs<SS_REAL> &, const McArgs &, cudaStream_t);
 template int mc_blocks_per_sm<SS_REAL>(int, int);
