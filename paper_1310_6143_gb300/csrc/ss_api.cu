@@ -1095,13 +1095,16 @@ void fill_material(MatDesc<R> &m, const MatKey &k, const ss_params *p) {
     m.gp = (R)(gamma / (1.0 + lam * lam));
     m.lambda = (R)lam;
     m.dt = (R)p->dt;
+    m.gdt = (R)(-(gamma / (1.0 + lam * lam)) * p->dt);
+    m.hgdt = (R)0.5 * m.gdt;
     m.sig = (R)std::sqrt(2.0 * lam * kBoltzmann / (gamma * mu * p->dt));
     m.mu = (R)mu;
     m.ku = (R)ku;
     m.kc = (R)k.v[11];
     m.kcf = (R)(-2.0 * k.v[11] / mu);
     m.sys = k.sys;
-    m.has_neel = (int16_t)k.has_neel;
+    m.has_neel = (int8_t)k.has_neel;
+    m.axis_z = k.v[2] == 0.0 && k.v[3] == 0.0 && k.v[4] == 1.0 ? 1 : 0;
     m.has_cubic = k.v[11] != 0.0 ? 1 : 0;
 }
 

@@ -152,8 +152,7 @@ __global__ void __launch_bounds__(32 * 4 * kClusterMaxGroups) k_cluster_steps(co
     const R k1 = pick3(rc, m.kf[3], m.kf[1], m.kf[5]);
     const R k2 = pick3(rc, m.kf[4], m.kf[5], m.kf[2]);
     // the material's constants in registers for the whole chunk
-    const R ex = m.e[0], ey = m.e[1], ez = m.e[2], ani = m.ani, mgp = -m.gp, lam = m.lambda, dt = m.dt;
-    const R hdt = (R)0.5 * dt, kcf = m.kcf, mu = m.mu;
+    const R ex = m.e[0], ey = m.e[1], ez = m.e[2], ani = m.ani, lam = m.lambda, kcf = m.kcf, mu = m.mu;
     const bool cubic = Cubic && m.has_cubic, neel = m.has_neel != 0;
 
     if (act && comp) S[role * P + ls] = pick3(role, a.sx, a.sy, a.sz)[i];
@@ -259,10 +258,10 @@ __global__ void __launch_bounds__(32 * 4 * kClusterMaxGroups) k_cluster_steps(co
             const R c0 = Cs[ls], c1 = Cs[P + ls], c2 = Cs[2 * P + ls];
             const R xc = role == 0 ? fma(s1, c2, -mul_rn(s2, c1))
                                    : (role == 1 ? fma(s2, c0, -mul_rn(s0, c2)) : fma(s0, c1, -mul_rn(s1, c0)));
-            const R dc = mul_rn(mgp, fma(lam, xc, cc));
+            const R wc = fma(lam, xc, cc);
             const R sc = pick3(role, s0, s1, s2);
-            qc = fma(hdt, dc, sc);
-            Vs[role * P + ls] = fma(dt, dc, sc);
+            qc = heun_add<R, true>(m, wc, sc);
+            Vs[role * P + ls] = heun_add<R, false>(m, wc, sc);
         }
         group_sync(grp);
         // E: S' = v / |v|
@@ -305,8 +304,7 @@ __global__ void __launch_bounds__(32 * 4 * kClusterMaxGroups) k_cluster_steps(co
             const R c0 = Cs[ls], c1 = Cs[P + ls], c2 = Cs[2 * P + ls];
             const R xc = role == 0 ? fma(p1, c2, -mul_rn(p2, c1))
                                    : (role == 1 ? fma(p2, c0, -mul_rn(p0, c2)) : fma(p0, c1, -mul_rn(p1, c0)));
-            const R dc = mul_rn(mgp, fma(lam, xc, cc));
-            Vs[role * P + ls] = fma(hdt, dc, qc);
+            Vs[role * P + ls] = heun_add<R, true>(m, fma(lam, xc, cc), qc);
         }
         group_sync(grp);
         // E: S = v / |v|, with the corrector kernel's non-finite check

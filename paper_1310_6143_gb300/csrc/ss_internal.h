@@ -59,11 +59,14 @@ struct alignas(16) MatDesc {
     R gp;         // gamma / (1 + lambda^2)
     R lambda;     // damping
     R dt;         // time step
+    R gdt, hgdt;  // -gp dt, -gp dt / 2 (FP64 update)
     R sig;        // sqrt(2 lambda kB / (gamma mu_s dt)); sigma = sig * sqrt(T)
     R mu;         // mu_s
     R ku;         // k_u
     int32_t sys;
-    int16_t has_neel, has_cubic;
+    int8_t has_neel, has_cubic;
+    int8_t axis_z;  // 1: the easy axis is exactly (0, 0, 1)
+    int8_t pad;
     R kf[6];      // (2 / mu_s) K, field tensor of the Neel term    (T)
     R K[6];       // Neel tensor (energy)
     R kc;         // cubic anisotropy k_c (energy (k_c/2) sum S^4)
