@@ -1501,8 +1501,9 @@ ss_status set_rows(ss_system *h, int32_t mode) {
 // step with 256 threads, 49.3 with 512; 256 grains of 5.2 M together: 256 and 248), everything
 // else in the latter.  FP64: 512 threads from four million spins on.
 // Spins per thread, up to 12: the count that leaves the busiest SM the least to do, its tiles times
-// the spins per thread (and about 0.3 spins' time for each tile's reduction).  The FP32-mixed
-// passes also need warps to hide their gathers: 16 a SM cost about 4 %, eight 30 % (FP64: eight 5 %).  fcc 64^3 in FP32-mixed form: 2 spins per thread leave the busiest SM 14
+// the spins per thread (and about 0.3 spins' time for each tile's reduction, 0.2 in FP64).  The
+// passes also need warps to hide their latencies: FP32-mixed, 16 a SM cost about 4 %, eight 30 %;
+// FP64, eight 15 %.  fcc 64^3 in FP32-mixed form: 2 spins per thread leave the busiest SM 14
 // tiles for 13.5 on average, 9 three for exactly three (66.2 -> 59.7 us per step).  From 24 tiles
 // of eight spins per thread a SM on there is little to round off, and eight are as fast as any.
 void default_shape(ss_system *h) {
@@ -1517,9 +1518,9 @@ void default_shape(ss_system *h) {
         int64_t tiles = 0;
         for (int64_t n : h->sys_n) tiles += (n + tile - 1) / tile;
         const int64_t per_sm = (tiles + sms - 1) / sms;
-        double cost = (double)per_sm * (slots + 0.3);
+        double cost = (double)per_sm * (slots + (mixed ? 0.3 : 0.2));
         const double warps = (double)per_sm * h->block / 32.0;
-        cost *= mixed ? 1.0 + 0.3 * std::pow(std::max(0.0, 24.0 - warps) / 16.0, 3.0) : (warps < 16.0 ? 1.05 : 1.0);
+        cost *= mixed ? 1.0 + 0.3 * std::pow(std::max(0.0, 24.0 - warps) / 16.0, 3.0) : (warps < 16.0 ? 1.15 : 1.0);
         if (cost < least) {
             least = cost;
             best = slots;
