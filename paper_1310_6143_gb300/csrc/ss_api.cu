@@ -110,6 +110,7 @@ struct ss_system {
     float *sched_f = nullptr;
     int64_t rec_cap = 0, sched_len = 0, sched_step0 = 0, sched_cap = 0;
     unsigned long long *ctl = nullptr;  // [0] step, [1] err|ticket, [2] barrier count|gen
+    double *report = nullptr;           // page-locked: what measurements and flag checks read back (kReport*)
     double2 *tab = nullptr;             // Box-Muller tables (build_bm_tables), then the
                                         // double-float tables (build_ff_tables)
     int32_t max_row = 0;                // longest CSR row
@@ -915,6 +916,12 @@ cudaError_t enqueue_cluster_steps(ss_system *h, int64_t n) {
         c.m = (int)std::min<int64_t>(chunk, n - k * chunk);
         return c;
     };
+    if (nk == 1) {  // nothing to overlap: in line, without the hand-overs between streams
+        cudaError_t e = launch_cluster_gauss<R>(a, args(0), h->stream);
+        if (e == cudaSuccess) e = launch_cluster_steps<R>(a, args(0), h->cl_ctas, h->max_row, h->stream);
+        if (e == cudaSuccess) e = launch_cluster_record<R>(a, args(0), h->block, h->stream);
+        return e;
+    }
     cudaEvent_t *eg = h->cl_ev, *ec = h->cl_ev + 2, *er = h->cl_ev + 4;
     cudaStream_t side = h->cl_side;
     cudaError_t e = cudaEventRecord(h->cl_ev[6], h->stream);  // parameters and state written before
@@ -1006,10 +1013,8 @@ cudaError_t ensure_graph(ss_system *h) {
     return cudaSuccess;
 }
 
-ss_status check_device_flags(ss_system *h) {
-    unsigned long long ctl[3];
-    SS_CUDA(h, cudaMemcpyAsync(ctl, h->ctl, sizeof(ctl), cudaMemcpyDeviceToHost, h->stream));
-    SS_CUDA(h, cudaStreamSynchronize(h->stream));
+// The control words read back after the handle's work: any device-side failure, and the step.
+ss_status apply_flags(ss_system *h, const unsigned long long ctl[3]) {
     const unsigned int err = (unsigned int)(ctl[1] & 0xffffffffull);
     h->step = (int64_t)ctl[0];
     if (err) {
@@ -1028,6 +1033,14 @@ ss_status check_device_flags(ss_system *h) {
         return fail(h, SS_ERR_NONFINITE, "a spin became non-finite (NaN/inf or zero length)");
     }
     return SS_OK;
+}
+
+ss_status check_device_flags(ss_system *h) {
+    unsigned long long own[3], *ctl = h->report ? reinterpret_cast<unsigned long long *>(h->report + kReportCtl) : own;
+    SS_CUDA(h, cudaMemcpyAsync(ctl, h->ctl, sizeof(own), cudaMemcpyDeviceToHost, h->stream));
+    SS_CUDA(h, cudaStreamSynchronize(h->stream));
+    std::memcpy(own, ctl, sizeof(own));
+    return apply_flags(h, own);
 }
 
 ss_status build_tiles(ss_system *h) {
@@ -1657,6 +1670,10 @@ ss_status create_impl(const ss_params *systems, int32_t count, ss_system **out, 
     if (st != SS_OK) return cleanup(st);
     st = h->precision == SS_FP32_MIXED ? init_random<float>(h, hs) : init_random<double>(h, hs);
     if (st != SS_OK) return cleanup(st);
+    if (cudaHostAlloc((void **)&h->report, kReportSize * sizeof(double), cudaHostAllocPortable) != cudaSuccess) {
+        cudaGetLastError();  // the control words and records are copied to pageable memory
+        h->report = nullptr;
+    }
     if (h->precision == SS_FP32_MIXED && !slab) {
         const size_t bytes = (size_t)packed_spins(h) * (3 * sizeof(float4) + sizeof(float2));
         if (dalloc(h, &h->packed, bytes) != cudaSuccess)
@@ -1674,13 +1691,17 @@ ss_status usable(ss_system *h) {
     return SS_OK;
 }
 
+// Whether the measurement reports to host memory itself.
+bool reports(const ss_system *h) { return h->report && h->nsys <= kMcInlineSystems; }
+
 template <typename R>
 ss_status measure(ss_system *h) {
     KArgs<R> a = make_args<R>(h);
     use_rows(h, a);
     if (h->rows) SS_CUDA(h, launch_rows_field<R>(a, a.sx, a.sy, a.sz, rows_grid(h), h->stream));
+    a.report = reports(h) ? h->report : nullptr;
     SS_CUDA(h, launch_measure<R>(a, h->block, step_grid(h), h->stream));
-    SS_CUDA(h, launch_finalize(h->sys, h->sys_tiles, h->nsys, h->partials, h->cur, h->stream));
+    if (!a.report) SS_CUDA(h, launch_finalize(h->sys, h->sys_tiles, h->nsys, h->partials, h->cur, h->stream));
     return SS_OK;
 }
 
@@ -1690,6 +1711,13 @@ ss_status current_record(ss_system *h, int32_t sys, double rec[kRecComps]) {
     if (sys < 0 || sys >= h->nsys) return fail(h, SS_ERR_INVALID_ARG, "system %d out of range", sys);
     st = h->precision == SS_FP32_MIXED ? measure<float>(h) : measure<double>(h);
     if (st != SS_OK) return st;
+    if (reports(h)) {
+        SS_CUDA(h, cudaStreamSynchronize(h->stream));
+        unsigned long long ctl[3];
+        std::memcpy(ctl, h->report + kReportCtl, sizeof(ctl));
+        std::memcpy(rec, h->report + kReportRec + sys * kRecComps, kRecComps * sizeof(double));
+        return apply_flags(h, ctl);
+    }
     SS_CUDA(h, cudaMemcpyAsync(rec, h->cur + (int64_t)sys * kRecComps, kRecComps * sizeof(double),
                                cudaMemcpyDeviceToHost, h->stream));
     return check_device_flags(h);
@@ -2232,6 +2260,7 @@ ss_status spin_system_destroy(ss_system *h) {
     if (!h) return SS_OK;
     if (h->stream) cudaStreamSynchronize(h->stream);
     drop_graph(h);
+    if (h->report) cudaFreeHost(h->report);
     for (auto &b : h->bufs) {
         cudaFree(b.p);
         g_live_bytes -= (int64_t)b.bytes;

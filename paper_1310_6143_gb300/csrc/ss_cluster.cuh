@@ -317,38 +317,36 @@ __global__ void __launch_bounds__(32 * 4 * kClusterMaxGroups) k_cluster_steps(co
 
 // The records of the chunk's steps (block s: step step0 + s) from the stored terms, tile by
 // tile with the predictor kernel's thread order and partial sums, then the record as the
-// corrector kernel finalises it.  BS must be the step kernels' block.
+// corrector kernel finalises it.  BS must be the step kernels' block.  A barrier per kTileChunk
+// tiles, as in predictor_pass: a system this small is one chunk, whose tiles' loads and FP64
+// butterflies then overlap.
 template <typename R, int BS>
 __global__ void __launch_bounds__(BS) k_cluster_record(const KArgs<R> a, const ClusterArgs<R> c) {
-    __shared__ double red[(BS / 32) * 8];
+    __shared__ double red[kTileChunk * (BS / 32) * 8];
     const int s = blockIdx.x;
     const uint64_t step = c.step0 + (uint64_t)s;
     const int64_t n = a.n;
     const R *T = c.T + (int64_t)s * 5 * n;
     double *part = c.partials + (int64_t)s * a.ntiles * kPartComps;
-    for (int64_t t = 0; t < a.ntiles; ++t) {
-        const TileDesc td = a.tiles[t];
-        TermAcc<R> ta;
-        ta.reset();
-        for (int k = threadIdx.x; k < td.count; k += BS) {
-            const int64_t i = td.start + k;
-            if constexpr (sizeof(R) == 4) {
+    for (int64_t t0 = 0; t0 < a.ntiles; t0 += kTileChunk) {
+        int nq = 0;
+        for (; nq < kTileChunk && t0 + nq < a.ntiles; ++nq) {
+            const TileDesc td = a.tiles[t0 + nq];
+            TermAcc<R> ta;
+            ta.reset();
+            for (int k = threadIdx.x; k < td.count; k += BS) {
+                const int64_t i = td.start + k;
                 R v[5];
 #pragma unroll
                 for (int q = 0; q < 5; ++q) v[q] = T[q * n + i];
                 ta.add(v);
-            } else {
-                double v[5];
-#pragma unroll
-                for (int q = 0; q < 5; ++q) v[q] = widen(T[q * n + i]);
-                ta.add(v);
             }
+            double acc[8];
+            ta.out(acc);
+            warp_partials<BS>(acc, red, nq);
         }
-        double acc[8];
-        ta.out(acc);
-        warp_partials<BS>(acc, red, 0);
         __syncthreads();
-        flush_partials<BS>(red, 1, part, t, 1);
+        flush_partials<BS>(red, nq, part, t0, 1);
         __syncthreads();
     }
     double *dst = a.rec + (int64_t)(step % (uint64_t)a.rec_cap) * a.nsys * kRecComps;

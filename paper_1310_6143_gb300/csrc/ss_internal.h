@@ -157,6 +157,8 @@ struct KArgs {
     double *rec;              // ring [rec_cap][nsys][kRecComps]
     int64_t rec_cap;
     double *cur;              // [nsys][kRecComps] on-demand measurement
+    double *report;           // host memory the measurement writes its records and the control words to
+                              // (kReport*), or nullptr (they are copied from cur)
     unsigned long long *step; // index of the next step
     const double *sqrtT_sched;
     const float *sqrtT_sched_f;  // the schedule rounded to float
@@ -200,8 +202,13 @@ struct McArgs {
     const int32_t *sys_slots; // [nsys + 1] first partial slot of each system
 };
 
-// Colour passes that end a step sum the record of at most this many systems.
+// Launches whose last block sums the record (a Monte Carlo step's last colour pass, the on-demand
+// measurement) do so for at most this many systems.
 constexpr int kMcInlineSystems = 8;
+
+// The host memory of KArgs.report, in doubles: the step counter, error and barrier words as they lie
+// in the control block, then the records of up to kMcInlineSystems systems.
+constexpr int kReportCtl = 0, kReportRec = 8, kReportSize = 8 + kMcInlineSystems * kRecComps;
 
 // Macrocell demagnetising field (Section "Demagnetising fields").
 struct DemagArgs {

@@ -1090,7 +1090,11 @@ __global__ void __launch_bounds__(BS) k_corrector_split(const KArgs<R> a, int nf
     }
 }
 
-// Tile partials of the current state (no integration): the on-demand measurement.
+// Tile partials of the current state (no integration): the on-demand measurement.  With a.report
+// the last block sums the records and writes them, with the control words, to host memory: a
+// measurement is then one launch and one wait, instead of two launches and two copies (a loop that
+// reads the magnetisation and the energy of sc 10^3 every 16 steps: 182 -> 137 us a round, with the
+// cluster step of a single chunk in line on the one stream and its record kernel's barrier per tile gone).
 template <typename R, int BS>
 __global__ void __launch_bounds__(BS) k_measure(const KArgs<R> a) {
     __shared__ double red[(BS / 32) * 8];
@@ -1124,6 +1128,26 @@ __global__ void __launch_bounds__(BS) k_measure(const KArgs<R> a) {
         ta.out(acc);
         const double r = block_sum8<BS>(acc, red);
         if (threadIdx.x < kPartComps) a.partials[t * kPartComps + threadIdx.x] = r;
+    }
+    if (!a.report) return;
+    __shared__ bool ends;
+    __threadfence();
+    __syncthreads();
+    if (threadIdx.x == 0) ends = atomicAdd(a.ticket, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!ends) return;
+    __threadfence();  // every other block's partials
+    for (int s = 0; s < a.nsys; ++s) {
+        double *dst = a.cur + (int64_t)s * kRecComps;
+        finalize_system<BS, true>(a.sys, a.sys_tiles, a.partials, s, dst, red);
+        if (threadIdx.x < kRecComps) a.report[kReportRec + s * kRecComps + threadIdx.x] = dst[threadIdx.x];
+    }
+    if (threadIdx.x == 0) {
+        *a.ticket = 0u;
+        __threadfence();
+        const volatile unsigned long long *ctl = a.step;  // the control block: step, error | ticket, barrier
+        unsigned long long *out = reinterpret_cast<unsigned long long *>(a.report + kReportCtl);
+        for (int k = 0; k < 3; ++k) out[k] = ctl[k];
     }
 }
 
