@@ -1543,13 +1543,14 @@ __device__ __forceinline__ void sib_a(R gp, R lam, R v0, R v1, R v2, R H0, R H1,
 // Threads per block of the passes of the alternative integrators.
 constexpr int kAltBlock = 256;
 
-// Resident blocks per SM the FP32-mixed first pass is compiled for (64 registers a thread; the
-// FP64 one for two, 128 registers).
-constexpr int kAltFirstBlocks = 4;
-// and the FP32-mixed second passes (40 registers): they wait for the neighbours' loads, so
-// resident warps count for more than a few spills (the semi-implicit
-// corrector on a 512 x 512 x 16 film: 82 us at the compiler's own 64 registers, 73 at 48, 68 at 40).
-constexpr int kAltSecondBlocks = 6;
+// Resident blocks per SM the FP32-mixed first pass is compiled for (80 registers a thread; the
+// FP64 one for two, 128 registers), and the FP32-mixed second passes (48 registers).  Both wait for
+// the neighbours' loads, against registers to hold them: with 64 and 40 registers the semi-implicit
+// step of a 512 x 512 x 16 film takes 207 us instead of 204, the midpoint step 371 instead of 357,
+// that of fcc 64^3 (rows of twelve) 148 instead of 130; a corrector left at the compiler's own 64
+// registers runs 82 us on the film, 68-73 with 40-48.
+constexpr int kAltFirstBlocks = 3;
+constexpr int kAltSecondBlocks = 5;
 
 // First pass of the alternative integrators: the step's thermal field (counters as the Heun
 // step), the part of the second pass's field that is fixed over the step,
@@ -1565,7 +1566,7 @@ constexpr int kAltSecondBlocks = 6;
 // Bound by issue.  In the FP32-mixed form the Gaussians come from the double-float transform
 // (the FP64 transform's values rounded to float, bit for bit, as in the Heun passes) and the
 // record terms are summed as float pairs, so the FP64 pipe runs no per-spin work; with the FP64
-// transform and the CSR this pass took 239 us on a 512 x 512 x 16 film.
+// transform and the CSR this pass took 239 us on a 512 x 512 x 16 film, now 140.
 template <typename R, int Mode, bool Sib>
 __device__ __forceinline__ void alt_first_pass(const KArgs<R> &a, const StepTabT<R> &tab, double *red, int sub,
                                                int len) {
