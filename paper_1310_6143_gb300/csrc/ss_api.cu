@@ -1196,6 +1196,9 @@ ss_status build_slices(ss_system *h, const std::vector<int32_t> &rp, const std::
     std::vector<int2> slice((size_t)nsl);
     std::vector<int64_t> off(1, 0);
     std::vector<uint32_t> sell, words;
+    int64_t most = 0;  // if no two slices are alike (the reserved pages cost nothing until they are written)
+    for (int64_t i = 0; i < n; ++i) most = std::max<int64_t>(most, rp[i + 1] - rp[i]);
+    sell.reserve((size_t)(32 * nsl * most));
     std::unordered_multimap<uint64_t, int32_t> form_of;  // hash of a slice's words -> form (contents compared)
     for (int64_t b = 0; b < period; ++b) {
         for (int64_t s = c.first(b); s < c.first(b + 1); ++s) {
@@ -1500,6 +1503,11 @@ ss_status set_rows(ss_system *h, int32_t mode) {
             SS_CUDA(h, cudaMemsetAsync(h->x4, 0, 128 * (size_t)h->nslice * rs, h->stream));
         }
     }
+    // the classes' padding in the float4 spins is gathered with J = 0 and has to be finite, whatever
+    // runs without row passes left there
+    if (on && !h->rows && h->packed && h->nslice > 0)
+        SS_CUDA(h, cudaMemsetAsync(h->packed, 0, (size_t)packed_spins(h) * (3 * sizeof(float4) + sizeof(float2)),
+                                   h->stream));
     h->rows_req = mode;
     if (on != h->rows) drop_graph(h);
     h->rows = on;
@@ -1727,30 +1735,51 @@ template <typename R>
 ss_status time_kernels_impl(ss_system *h, int32_t nsteps, double out_ms[4]) {
     KArgs<R> a = make_args<R>(h);
     use_rows(h, a);
-    const bool split = split_step(h);
-    const int gp = split ? split_grid(h, 1) : step_grid(h), gc = split ? split_grid(h, 2) : corrector_grid(h);
+    const bool split = split_step(h), packed = packed_run(h, nsteps);  // (as the steps of a run that long)
+    const int gp = split ? split_grid(h, 1) : packed ? packed_grid(h, 0) : step_grid(h);
+    const int gc = split ? split_grid(h, 2) : packed ? packed_grid(h, 1) : corrector_grid(h);
     const int gg = split ? split_grid(h, 0) : 0, gr = h->rows ? rows_grid(h) : 0;
     // per step: [Gaussian pass] ev[3k+1] predictor ev[3k+2] corrector ev[3k+3]
     std::vector<cudaEvent_t> ev(3 * (size_t)nsteps + 1);
     for (auto &e : ev) SS_CUDA(h, cudaEventCreate(&e));
+    auto rows = [&](const R *X, const R *Y, const R *Z, float4 *V) {  // the field of S or S' of long rows
+        if (!packed) return launch_rows_field<R>(a, X, Y, Z, gr, h->stream);
+        KArgs<R> r = a;
+        r.x4 = reinterpret_cast<R *>(V);
+        return launch_rows_field<R>(r, nullptr, nullptr, nullptr, gr, h->stream);
+    };
+    auto predictor = [&]() -> cudaError_t {
+        if constexpr (sizeof(R) == 4) {
+            if (packed) return launch_predictor4<R>(a, h->block, gp, h->stream);
+        }
+        return launch_predictor<R>(a, h->block, gp, h->stream);
+    };
+    auto corrector = [&]() -> cudaError_t {
+        if constexpr (sizeof(R) == 4) {
+            if (packed) return launch_corrector4<R>(a, h->block, gc, h->nfin, h->stream);
+        }
+        return launch_corrector<R>(a, h->block, gc, h->nfin, h->stream);
+    };
+    if (packed) SS_CUDA(h, packed_state(h, true));
     SS_CUDA(h, cudaEventRecord(ev[0], h->stream));
     for (int32_t k = 0; k < nsteps; ++k) {
         if (split && k == 0) SS_CUDA(h, launch_gstep_sync<R>(a, h->stream));
         if (split) SS_CUDA(h, launch_gauss<R>(a, h->block, gg, h->stream, 0));
         SS_CUDA(h, cudaEventRecord(ev[3 * k + 1], h->stream));
-        if (h->rows) SS_CUDA(h, launch_rows_field<R>(a, a.sx, a.sy, a.sz, gr, h->stream));
+        if (h->rows) SS_CUDA(h, rows(a.sx, a.sy, a.sz, a.s4));
         if (split)
             SS_CUDA(h, launch_predictor_split<R>(a, h->block, gp, h->stream));
         else
-            SS_CUDA(h, launch_predictor<R>(a, h->block, gp, h->stream));
+            SS_CUDA(h, predictor());
         SS_CUDA(h, cudaEventRecord(ev[3 * k + 2], h->stream));
-        if (h->rows) SS_CUDA(h, launch_rows_field<R>(a, a.px, a.py, a.pz, gr, h->stream));
+        if (h->rows) SS_CUDA(h, rows(a.px, a.py, a.pz, a.p4));
         if (split)
             SS_CUDA(h, launch_corrector_split<R>(a, h->block, gc, h->nfin, h->stream));
         else
-            SS_CUDA(h, launch_corrector<R>(a, h->block, gc, h->nfin, h->stream));
+            SS_CUDA(h, corrector());
         SS_CUDA(h, cudaEventRecord(ev[3 * k + 3], h->stream));
     }
+    if (packed) SS_CUDA(h, packed_state(h, false));
     SS_CUDA(h, cudaEventSynchronize(ev.back()));
     double tg = 0.0, tp = 0.0, tc = 0.0;
     for (int32_t k = 0; k < nsteps; ++k) {
