@@ -533,6 +533,12 @@ KArgs<R> make_args(const ss_system *h) {
     a.ell_w = h->ell_w;
     a.mat_uniform = h->nmat == 1 ? 1 : 0;
     std::memcpy(&a.mat0, h->mat0, sizeof(MatDesc<R>));
+    if (a.mat_uniform) {
+        a.key0 = h->hsys[0].key0;
+        a.key1 = h->hsys[0].key1;
+        a.ctr2 = h->hsys[0].ctr2;
+        a.pshift = (int32_t)(h->hsys[0].pbase - h->hsys[0].offset);
+    }
     a.Jt = static_cast<const R *>(h->Jt);
     a.Jtidx = h->Jtidx;
     a.J_tensor = h->J_tensor ? 1 : 0;

@@ -103,7 +103,10 @@ struct KArgs {
     const R *ell_J;           // 8 | entry of ell_J), ell_w of them, padded with J = 0; or nullptr
     int ell_w;
     MatDesc<R> mat0;          // the only material when mat_uniform is set
-    int mat_uniform;          // 1: every spin has material 0 (mat is not read)
+    int mat_uniform;          // 1: every spin has material 0 (mat is not read); the handle is then one
+                              // system, with these Philox words:
+    uint32_t key0, key1, ctr2;  // its key and third counter word,
+    int32_t pshift;             // and spin i draws with word i + pshift
     const R *Jt;              // [9 ndict] distinct exchange tensors / mu_s,i, row by row
     const int32_t *Jtidx;     // [nnz] tensor of each bond (J_tensor = 1)
     int J_tensor;             // 1: the exchange sum uses Jt[Jtidx[k]] instead of J

@@ -639,6 +639,26 @@ __device__ __forceinline__ void flush_partials(const double *red, int nq, double
     }
 }
 
+// What the FP32-mixed kernels of 64 registers (512-thread blocks) do to keep a tile's spins' loads in
+// registers instead of spilling: 32-bit spin indices, and with a single material -- then a single
+// system -- its Philox words from the kernel arguments.  The film's passes spill 24 and 4 bytes instead
+// of 52 and 44 (16 steps: 10.00 -> 9.50 ms), the grains' 68 and 48 of 112 and 64 (4.10 -> 4.04 ms); with
+// 80 registers it made the compiler spill more (fcc 64^3: 3.97 -> 4.08 ms for 64 steps).
+template <typename R, int BS>
+constexpr bool kTight = sizeof(R) == 4 && BS >= 512;
+
+// The Philox words of a tile's draws: spin i's counter word is i + shift.
+struct DrawKey {
+    uint32_t key0, key1, ctr2, shift;
+};
+template <bool Args, typename R>
+__device__ __forceinline__ DrawKey draw_key(const KArgs<R> &a, const SysDesc &sd) {
+    if constexpr (Args)
+        return DrawKey{a.key0, a.key1, a.ctr2, (uint32_t)a.pshift};
+    else
+        return DrawKey{sd.key0, sd.key1, sd.ctr2, (uint32_t)(sd.pbase - sd.offset)};
+}
+
 // Where a Heun pass gathers its spins.
 template <typename R, bool Coherent, bool V4>
 __device__ __forceinline__ auto heun_src(const KArgs<R> &a, const R *X, const R *Y, const R *Z, const float4 *V) {
@@ -665,8 +685,7 @@ __device__ __forceinline__ void predictor_tile(const KArgs<R> &a, const TileDesc
     constexpr int BM = base_mode(Mode);
     const SysDesc &sd = a.sys[td.sys];
     const R sqrtT = sqrtT_of_step(a, step, sd);
-    const uint32_t key0 = sd.key0, key1 = sd.key1, ctr2 = sd.ctr2;
-    const int64_t off = sd.offset - sd.pbase;  // Philox spin index i - off
+    const DrawKey dk = draw_key<kTight<R, BS> && Mode == kUniform>(a, sd);
     const R ha0 = sys_H(sd, 0, R()), ha1 = sys_H(sd, 1, R()), ha2 = sys_H(sd, 2, R());
     const auto src = heun_src<R, Coherent, V4>(a, a.sx, a.sy, a.sz, a.s4);
     TermAcc<R> ta;
@@ -676,7 +695,7 @@ __device__ __forceinline__ void predictor_tile(const KArgs<R> &a, const TileDesc
     int rot = (threadIdx.x >> 5) % a.slots;
     int next_form = (int)threadIdx.x < td.count ? form_of(a, td.start + threadIdx.x) : 0;
     for (int k = threadIdx.x; k < td.count; k += BS, rot = rot + 1 == a.slots ? 0 : rot + 1) {
-        const int64_t i = td.start + k;
+        const std::conditional_t<kTight<R, BS>, int32_t, int64_t> i = td.start + k;
         const int form = next_form;  // read a slot ahead: the chain form -> offsets -> spins starts at the offsets
         if (k + BS < td.count) next_form = form_of(a, i + BS);
         const MatDesc<R> &m = mat_at<Mode>(a, i);
@@ -701,7 +720,7 @@ __device__ __forceinline__ void predictor_tile(const KArgs<R> &a, const TileDesc
             const R sig = m.sig * sqrtT;
             if constexpr (!Split) {
                 if (!given) {
-                    const Philox4 w = philox4x32_10((uint32_t)(i - off), (uint32_t)step, ctr2, 0u, key0, key1);
+                    const Philox4 w = philox4x32_10((uint32_t)i + dk.shift, (uint32_t)step, dk.ctr2, 0u, dk.key0, dk.key1);
                     thermal_gaussians(a, *tab, w, g0, g1, g2);
                 }
             }
@@ -759,14 +778,13 @@ __device__ __forceinline__ void corrector_tile(const KArgs<R> &a, const TileDesc
     // Gaussians of step + 1 for the slots the next predictor will not draw (FP32-mixed):
     // this puts transform work next to the corrector's memory traffic.
     const R sqrtT_next = tab ? sqrtT_of_step(a, step + 1, sd) : (R)0;
-    const uint32_t key0 = sd.key0, key1 = sd.key1, ctr2 = sd.ctr2;
-    const int64_t off = sd.offset - sd.pbase;  // Philox spin index i - off
+    const DrawKey dk = draw_key<kTight<R, BS> && Mode == kUniform>(a, sd);
     const R ha0 = sys_H(sd, 0, R()), ha1 = sys_H(sd, 1, R()), ha2 = sys_H(sd, 2, R());
     const auto src = heun_src<R, Coherent, V4>(a, a.px, a.py, a.pz, a.p4);
     int rot = (threadIdx.x >> 5) % a.slots;  // the predictor's rotated slot index
     int next_form = (int)threadIdx.x < td.count ? form_of(a, td.start + threadIdx.x) : 0;
     for (int k = threadIdx.x; k < td.count; k += BS, rot = rot + 1 == a.slots ? 0 : rot + 1) {
-        const int64_t i = td.start + k;
+        const std::conditional_t<kTight<R, BS>, int32_t, int64_t> i = td.start + k;
         const int form = next_form;  // a slot ahead, as the predictor
         if (k + BS < td.count) next_form = form_of(a, i + BS);
         const MatDesc<R> &m = mat_at<Mode>(a, i);
@@ -825,7 +843,7 @@ __device__ __forceinline__ void corrector_tile(const KArgs<R> &a, const TileDesc
             a.sz[i] = mul_rn(v2, inv);
         }
         if (!Split && rot >= a.pre_slot && sqrtT_next > (R)0) {
-            const Philox4 w = philox4x32_10((uint32_t)(i - off), (uint32_t)(step + 1), ctr2, 0u, key0, key1);
+            const Philox4 w = philox4x32_10((uint32_t)i + dk.shift, (uint32_t)(step + 1), dk.ctr2, 0u, dk.key0, dk.key1);
             R g0, g1, g2;
             thermal_gaussians(a, *tab, w, g0, g1, g2);
             a.gx[i] = g0;
