@@ -1297,8 +1297,11 @@ __global__ void __launch_bounds__(BS) k_persistent(const KArgs<R> a, int nfin, l
 // systems are independent).  Every spin a block reads was written by the same block, after
 // a block barrier; loads bypass the non-coherent L1.  Each step's record is summed in the
 // block directly.  The last block to finish advances the step counter.
+//
+// The FP32-mixed kernel keeps 24 warps a SM (80 registers) in blocks of up to 256 threads; left to
+// itself the compiler takes 128 (1,024 systems of sc 10^3: 52 us per step, with the bound 45).
 template <typename R, int BS, int Mode = kGeneral>
-__global__ void __launch_bounds__(BS) k_system_blocks(const KArgs<R> a, long long nsteps) {
+__global__ void __launch_bounds__(BS, sizeof(R) == 8 || BS >= 512 ? 0 : heun_blocks(BS)) k_system_blocks(const KArgs<R> a, long long nsteps) {
     __shared__ StepTabT<R> tab;
     __shared__ double red[(BS / 32) * 8];
     stage_step_tables(a, tab);
