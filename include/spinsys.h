@@ -259,8 +259,8 @@ ss_status get_mc_stats(ss_system *h, int32_t sys, int64_t out[2]);
  * fixed-point iterations from the Euler predictor; nothing is renormalised (the rule keeps
  * |S| when converged; the residual of the iteration shows in |S| - 1).  Shares the step
  * counter, record ring, temperatures and demagnetising field (set_demag: updated at the same
- * steps, held over each step) with llg_heun_step; runs iterations + 3 launches per step (the
- * first also sums the step's record).  SS_ERR_INVALID_ARG for n < 0 or iterations out of
+ * steps, held over each step) with llg_heun_step; runs iterations + 1 launches per step (the
+ * first iteration also sums the step's record, the last advances the step counter).  SS_ERR_INVALID_ARG for n < 0 or iterations out of
  * range. */
 ss_status llg_midpoint_step(ss_system *h, int64_t n, int32_t iterations);
 
@@ -272,9 +272,9 @@ ss_status llg_midpoint_step(ss_system *h, int64_t n, int32_t iterations);
  * x A(Sb), Sb = (S_n + S')/2, each in closed form (a rotation of S_n: |S| is kept without
  * renormalisation); H includes the step's thermal field, drawn once per step from the same
  * Philox counters as llg_heun_step and held over the step.  Shares the step counter, record
- * ring, temperatures and demagnetising field (as llg_midpoint_step) with llg_heun_step; 4
- * launches per step (the predictor also sums the step's record), captured in CUDA graphs for
- * runs of whole graphs.  SS_ERR_INVALID_ARG for n < 0. */
+ * ring, temperatures and demagnetising field (as llg_midpoint_step) with llg_heun_step; 2
+ * launches per step (the corrector also sums the step's record and advances the step counter),
+ * captured in CUDA graphs for runs of whole graphs.  SS_ERR_INVALID_ARG for n < 0. */
 ss_status llg_semi_implicit_step(ss_system *h, int64_t n);
 
 /* Copy all spins (concatenated over systems) to out3n [3n], AoS, FP64 (synchronous): the
@@ -335,10 +335,12 @@ ss_status spin_system_set_launch(ss_system *h, int32_t block, int32_t tile);
  * section runs), 1 a thread per row (the step kernels sum their own rows), 2 a warp per row.  With a warp per row, each Heun pass is preceded by a pass that sums the exchange
  * field of every spin into a buffer of 3n values.  For scalar J with at most 255 distinct
  * J_ij / mu_s,i and fewer than 2^24 spins (checked at creation, when the rows average 16 or
- * more bonds) the bonds are stored as packed 32-bit words (neighbour index and dictionary
- * entry, 4 bytes per bond) in slices of 32 consecutive rows, bond k of the slice's rows
- * interleaved and each slice padded to its longest row with zero bonds; lane l of a warp
- * sums row l of its slice in CSR order from H_app, exactly as a thread per row does, so the
+ * more bonds) the bonds are stored as packed 32-bit words (neighbour and dictionary entry, 4
+ * bytes per bond) in slices of 32 rows a period apart (the period, 1 to 8, chosen so that a
+ * bond's neighbours lie together in the pass's copy of the spins), bond k of the slice's rows
+ * interleaved, each slice padded to its longest row with zero bonds and slices with the same
+ * words stored once; lane l of a warp sums row l of its slice in CSR order from H_app, exactly
+ * as a thread per row does, so the
  * results are identical to mode 1 (ss_info.exchange_rows = 3).  Otherwise (tensors, more
  * values) each warp sums 32 consecutive rows one by one, its lanes striding over the row's
  * bonds (exchange_rows = 2): only the summation order differs.  The midpoint and
