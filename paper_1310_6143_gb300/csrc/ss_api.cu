@@ -14,6 +14,8 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <new>
+#include <stdexcept>
 #include <string>
 #include <unordered_map>
 #include <vector>
@@ -186,7 +188,7 @@ struct ss_system {
     bool rows = false;           // a warp per row in force
     uint32_t *sell = nullptr;    // packed bonds of the distinct slices of 32 rows (k_rows_sell)
     int64_t *sell_off = nullptr; // [distinct slices + 1] word offset of each
-    int2 *slice = nullptr;       // [nslice] (distinct slice, first row)
+    SliceRef *slice = nullptr;   // [nslice]
     int64_t nslice = 0;
     int period = 1;              // distance of a slice's rows
     void *Jd = nullptr;          // the dictionary of J_ij / mu_s,i (with 0 for the padding)
@@ -496,19 +498,6 @@ ss_status build_patterns(ss_system *h, const std::vector<int32_t> &rp, const std
     return SS_OK;
 }
 
-// The classes of a period: spins i = b, b + period, ... of each b, padded to whole slices.
-struct Classes {
-    int64_t n;
-    int period, rest, hi, lo;
-    Classes(int64_t n_, int period_) : n(n_), period(period_), rest((int)(n_ % period_)) {
-        lo = (int)((n / period + 31) / 32);
-        hi = (int)((n / period + 1 + 31) / 32);
-    }
-    int64_t first(int64_t b) const { return b <= rest ? b * hi : (int64_t)rest * hi + (b - rest) * lo; }
-    int64_t slices() const { return first(period); }
-    int64_t pos(int64_t i) const { return 32 * first(i % period) + i / period; }  // as x4_pos on the device
-};
-
 // Spins of a float4 array: with sliced long rows the classes' padding as well.
 int64_t packed_spins(const ss_system *h) { return std::max<int64_t>(h->n, 32 * h->nslice); }
 
@@ -549,13 +538,7 @@ KArgs<R> make_args(const ss_system *h) {
     a.sell_off = h->sell_off;
     a.slice = h->slice;
     a.nslice = h->nslice;
-    {
-        const Classes c(h->n, h->period);
-        a.period = c.period;
-        a.period_rest = c.rest;
-        a.period_hi = c.hi;
-        a.period_lo = c.lo;
-    }
+    a.cls = Classes::of(h->n, h->period);
     a.x4 = static_cast<R *>(h->x4);
     a.Jd = static_cast<const R *>(h->Jd);
     a.nJd = h->nJd;
@@ -1127,133 +1110,20 @@ void fill_material(MatDesc<R> &m, const MatKey &k, const ss_params *p) {
     m.has_cubic = k.v[11] != 0.0 ? 1 : 0;
 }
 
-// The distinct J_ij / mu_s,i of the bonds (at most 255, and 0 for padding) and each bond's entry.
-template <typename R>
-bool bond_dictionary(const std::vector<R> &J, int64_t nnz, std::vector<R> &dict, std::vector<uint8_t> &bid, int &zero) {
-    using Bits = typename std::conditional<sizeof(R) == 8, uint64_t, uint32_t>::type;
-    constexpr int kSlots = 1024;
-    std::vector<Bits> key(kSlots);
-    std::vector<int> id(kSlots, -1);
-    Bits last = 0;
-    bid.resize((size_t)nnz);
-    zero = -1;
-    for (int64_t k = 0; k < nnz; ++k) {
-        Bits b;
-        std::memcpy(&b, &J[k], sizeof(R));
-        if (k > 0 && b == last) {  // (bonds of a row mostly repeat)
-            bid[(size_t)k] = bid[(size_t)k - 1];
-            continue;
-        }
-        last = b;
-        uint32_t hsh = (uint32_t)(((uint64_t)b * 0x9E3779B97F4A7C15ull) >> 54);  // 10 bits
-        while (id[hsh] >= 0 && key[hsh] != b) hsh = (hsh + 1) & (kSlots - 1);
-        if (id[hsh] < 0) {
-            if (dict.size() == 255) return false;
-            key[hsh] = b;
-            id[hsh] = (int)dict.size();
-            if (b == 0) zero = id[hsh];
-            dict.push_back(J[k]);
-        }
-        bid[(size_t)k] = (uint8_t)id[hsh];
-    }
-    if (zero < 0) {
-        zero = (int)dict.size();
-        dict.push_back((R)0);
-    }
-    return true;
-}
-
-// The slices of k_rows_sell.  The period is the one of a few whose slices' bonds touch the fewest
-// 128-byte lines of the spins' copy (a sample of the rows; a larger one has to be a tenth better),
-// as long as the positions fit a bond word.
+// The slices of k_rows_sell on the device.
 ss_status build_slices(ss_system *h, const std::vector<int32_t> &rp, const std::vector<int32_t> &col,
                        const std::vector<uint8_t> &bid, int zero) {
-    const int64_t n = h->n;
-    int period = 1;
-    int64_t least = INT64_MAX;
-    for (int p : {1, 2, 3, 4, 6, 8}) {
-        const Classes c(n, p);
-        if (32 * c.slices() >= (int64_t(1) << 24) || p > n) continue;
-        int64_t lines = 0;
-        std::vector<int64_t> seen;
-        for (int q = 0; q < 8; ++q) {  // slices spread over the rows, some of their bonds
-            const int64_t i0 = (n - 1) * q / 8;
-            int32_t len = INT32_MAX;
-            for (int l = 0; l < 32 && i0 + (int64_t)l * p < n; ++l) len = std::min(len, rp[i0 + (int64_t)l * p + 1] - rp[i0 + (int64_t)l * p]);
-            for (int32_t k = 0; k < len; k += 1 + len / 16) {
-                seen.clear();
-                for (int l = 0; l < 32 && i0 + (int64_t)l * p < n; ++l) seen.push_back(c.pos(col[rp[i0 + (int64_t)l * p] + k]) >> 3);
-                std::sort(seen.begin(), seen.end());
-                lines += std::unique(seen.begin(), seen.end()) - seen.begin();
-            }
-        }
-        if (lines < least - least / 10) {
-            least = lines;
-            period = p;
-        }
-    }
-    const Classes c(n, period);
-    const int64_t nsl = c.slices();
-    std::vector<int32_t> pos((size_t)n);
-    for (int64_t b = 0; b < period; ++b) {
-        int32_t at = (int32_t)(32 * c.first(b));
-        for (int64_t i = b; i < n; i += period) pos[(size_t)i] = at++;
-    }
-    std::vector<int2> slice((size_t)nsl);
-    std::vector<int64_t> off(1, 0);
-    std::vector<uint32_t> sell, words;
-    int64_t most = 0;  // if no two slices are alike (the reserved pages cost nothing until they are written)
-    for (int64_t i = 0; i < n; ++i) most = std::max<int64_t>(most, rp[i + 1] - rp[i]);
-    sell.reserve((size_t)(32 * nsl * most));
-    std::unordered_multimap<uint64_t, int32_t> form_of;  // hash of a slice's words -> form (contents compared)
-    for (int64_t b = 0; b < period; ++b) {
-        for (int64_t s = c.first(b); s < c.first(b + 1); ++s) {
-            const int64_t row0 = b + (int64_t)period * 32 * (s - c.first(b));
-            int32_t w = 0;
-            for (int64_t i = row0; i < std::min<int64_t>(n, row0 + 32 * (int64_t)period); i += period) w = std::max(w, rp[i + 1] - rp[i]);
-            words.resize(32 * (size_t)w);
-            const int32_t base = (int32_t)(32 * s);
-            for (int l = 0; l < 32; ++l) {
-                const int64_t i = row0 + (int64_t)l * period;
-                const int32_t len = i < n ? rp[i + 1] - rp[i] : 0;
-                const uint32_t pad = ((uint32_t)l << 8) | (uint32_t)zero;
-                uint32_t *out = words.data() + l;
-                const int32_t *cj = i < n ? col.data() + rp[i] : nullptr;
-                const uint8_t *bj = i < n ? bid.data() + rp[i] : nullptr;
-                for (int32_t k = 0; k < len; ++k) out[32 * (size_t)k] = ((uint32_t)(pos[(size_t)cj[k]] - base) << 8) | bj[k];
-                for (int32_t k = len; k < w; ++k) out[32 * (size_t)k] = pad;
-            }
-            uint64_t hsh = (uint64_t)w, mul = 0x9E3779B97F4A7C15ull;  // of a sample: contents are compared below
-            for (size_t q = 0; q < words.size(); q += 29) {
-                hsh += (words[q] ^ 0x5bd1e995u) * mul;
-                mul += 0xBF58476D1CE4E5BAull;
-            }
-            hsh ^= hsh >> 31;
-            int32_t form = -1;
-            const auto range = form_of.equal_range(hsh);
-            for (auto it = range.first; it != range.second && form < 0; ++it) {
-                const int64_t o = off[(size_t)it->second], len = off[(size_t)it->second + 1] - o;
-                if (len == (int64_t)words.size() && std::equal(words.begin(), words.end(), sell.begin() + o)) form = it->second;
-            }
-            if (form < 0) {
-                form = (int32_t)off.size() - 1;
-                form_of.emplace(hsh, form);
-                sell.insert(sell.end(), words.begin(), words.end());
-                off.push_back((int64_t)sell.size());
-            }
-            slice[(size_t)s] = make_int2(form, (int)row0);
-        }
-    }
-    if (sell.empty()) sell.push_back(0);
-    SS_CUDA(h, dalloc(h, (void **)&h->sell, sell.size() * sizeof(uint32_t)));
-    SS_CUDA(h, dalloc(h, (void **)&h->sell_off, off.size() * sizeof(int64_t)));
-    SS_CUDA(h, dalloc(h, (void **)&h->slice, slice.size() * sizeof(int2)));
-    SS_CUDA(h, cudaMemcpyAsync(h->sell, sell.data(), sell.size() * sizeof(uint32_t), cudaMemcpyHostToDevice, h->stream));
-    SS_CUDA(h, cudaMemcpyAsync(h->sell_off, off.data(), off.size() * sizeof(int64_t), cudaMemcpyHostToDevice, h->stream));
-    SS_CUDA(h, cudaMemcpyAsync(h->slice, slice.data(), slice.size() * sizeof(int2), cudaMemcpyHostToDevice, h->stream));
+    Slices s;
+    pack_slices(h->n, rp.data(), col.data(), bid.data(), zero, s);
+    SS_CUDA(h, dalloc(h, (void **)&h->sell, s.words.size() * sizeof(uint32_t)));
+    SS_CUDA(h, dalloc(h, (void **)&h->sell_off, s.off.size() * sizeof(int64_t)));
+    SS_CUDA(h, dalloc(h, (void **)&h->slice, s.slice.size() * sizeof(SliceRef)));
+    SS_CUDA(h, cudaMemcpyAsync(h->sell, s.words.data(), s.words.size() * sizeof(uint32_t), cudaMemcpyHostToDevice, h->stream));
+    SS_CUDA(h, cudaMemcpyAsync(h->sell_off, s.off.data(), s.off.size() * sizeof(int64_t), cudaMemcpyHostToDevice, h->stream));
+    SS_CUDA(h, cudaMemcpyAsync(h->slice, s.slice.data(), s.slice.size() * sizeof(SliceRef), cudaMemcpyHostToDevice, h->stream));
     SS_CUDA(h, cudaStreamSynchronize(h->stream));  // the host vectors go out of scope
-    h->nslice = nsl;
-    h->period = period;
+    h->nslice = (int64_t)s.slice.size();
+    h->period = s.period;
     return SS_OK;
 }
 
@@ -1403,10 +1273,9 @@ ss_status upload_system(ss_system *h, const std::vector<HostSys> &hs) {
                                    h->stream));
         SS_CUDA(h, cudaStreamSynchronize(h->stream));  // the host vectors go out of scope
     }
-    // Packed bonds for rows long enough to go a warp per row: col (< 2^24) and one byte naming
-    // the bond's J_ij / mu_s,i in a dictionary of at most 255 values plus 0, stored in slices
-    // of 32 rows (bond k of the slice's row l at 32 k + l), each padded to its longest row with
-    // J = 0 bonds.
+    // Packed bonds for rows long enough to go a warp per row (pack_slices): the neighbour's position
+    // (< 2^24) and one byte naming the bond's J_ij / mu_s,i in a dictionary of at most 255 values
+    // plus 0.
     if (!tensor && nnz >= kSellMin * n && n < (int64_t(1) << 24)) {
         std::vector<R> dict;
         std::vector<uint8_t> bid;
@@ -1568,6 +1437,26 @@ struct SlabInit {
     const std::vector<uint8_t> *edge;  // [n_own] owned spins with a halo neighbour
 };
 
+// A handle under construction, destroyed unless it is released (h = nullptr).
+struct Owner {
+    ss_system *h;
+    ~Owner() {
+        if (h) spin_system_destroy(h);
+    }
+};
+
+// The creating calls: a host allocation that fails is reported like any other failure.
+template <typename F>
+ss_status guarded(F create) {
+    try {
+        return create();
+    } catch (const std::bad_alloc &) {
+        return fail(nullptr, SS_ERR_OOM, "host allocation failed");
+    } catch (const std::length_error &) {
+        return fail(nullptr, SS_ERR_OOM, "host allocation failed");
+    }
+}
+
 ss_status create_impl(const ss_params *systems, int32_t count, ss_system **out, const SlabInit *slab = nullptr) {
     if (!out) return fail(nullptr, SS_ERR_INVALID_ARG, "out is NULL");
     *out = nullptr;
@@ -1590,6 +1479,7 @@ ss_status create_impl(const ss_params *systems, int32_t count, ss_system **out, 
 
     ss_system *h = new (std::nothrow) ss_system();
     if (!h) return fail(nullptr, SS_ERR_OOM, "host allocation failed");
+    Owner owner{h};
     h->precision = systems[0].precision;
     h->n = n;
     h->nnz = nnz;
@@ -1600,7 +1490,6 @@ ss_status create_impl(const ss_params *systems, int32_t count, ss_system **out, 
     if (e != cudaSuccess) {
         ss_status st = fail(nullptr, e == cudaErrorNoDevice ? SS_ERR_UNSUPPORTED : SS_ERR_CUDA, "CUDA: %s",
                             cudaGetErrorString(e));
-        delete h;
         return st;
     }
     h->stream = h->own_stream;
@@ -1644,9 +1533,7 @@ ss_status create_impl(const ss_params *systems, int32_t count, ss_system **out, 
         d.msum = ms;
     }
     auto cleanup = [&](ss_status st) {
-        std::string msg = h->err;
-        spin_system_destroy(h);
-        g_create_error = msg;
+        g_create_error = h->err;
         return st;
     };
     ss_status st;
@@ -1695,6 +1582,7 @@ ss_status create_impl(const ss_params *systems, int32_t count, ss_system **out, 
         else if (h->nslice > 0 && (e = cudaMemsetAsync(h->packed, 0, bytes, h->stream)) != cudaSuccess)
             return cleanup(cuda_fail(h, e, "cudaMemsetAsync"));  // (the classes' padding has to be finite)
     }
+    owner.h = nullptr;
     *out = h;
     return SS_OK;
 }
@@ -2285,10 +2173,12 @@ cudaError_t enqueue_mc(ss_system *h, int64_t nsteps) {
 
 extern "C" {
 
-ss_status spin_system_create(const ss_params *p, ss_system **out) { return create_impl(p, 1, out); }
+ss_status spin_system_create(const ss_params *p, ss_system **out) {
+    return guarded([&] { return create_impl(p, 1, out); });
+}
 
 ss_status spin_batch_create(const ss_params *systems, int32_t count, ss_system **out) {
-    return create_impl(systems, count, out);
+    return guarded([&] { return create_impl(systems, count, out); });
 }
 
 ss_status spin_system_destroy(ss_system *h) {
@@ -2874,7 +2764,7 @@ ss_status spin_system_set_draw_ahead(ss_system *h, int32_t eighths) {
 // and halo spins, the halo passed between processors twice per time step)
 // ----------------------------------------------------------------------------------
 
-ss_status spin_slab_create(const ss_params *p, int32_t nslabs, int32_t slab, ss_system **out) {
+static ss_status slab_create(const ss_params *p, int32_t nslabs, int32_t slab, ss_system **out) {
     if (!out) return fail(nullptr, SS_ERR_INVALID_ARG, "out is NULL");
     *out = nullptr;
     if (!p) return fail(nullptr, SS_ERR_INVALID_ARG, "params is NULL");
@@ -2949,6 +2839,7 @@ ss_status spin_slab_create(const ss_params *p, int32_t nslabs, int32_t slab, ss_
     ss_system *h = nullptr;
     st = create_impl(&q, 1, &h, &init);
     if (st != SS_OK) return st;
+    Owner owner{h};
     h->slab_lo = lo;
     h->slab_hi = hi;
     h->nslabs = nslabs;
@@ -2961,8 +2852,13 @@ ss_status spin_slab_create(const ss_params *p, int32_t nslabs, int32_t slab, ss_
         h->slab_runs.push_back(own + (int64_t)r);
         r = e;
     }
+    owner.h = nullptr;
     *out = h;
     return SS_OK;
+}
+
+ss_status spin_slab_create(const ss_params *p, int32_t nslabs, int32_t slab, ss_system **out) {
+    return guarded([&] { return slab_create(p, nslabs, slab, out); });
 }
 
 ss_status spin_slab_info(ss_system *h, ss_slab_info *o) {

@@ -4,6 +4,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "ss_slices.h"
+
 namespace ss {
 
 // Table I of the paper.
@@ -118,11 +120,9 @@ struct KArgs {
                               // row l at sell[sell_off[form] + 32 k + l]: (x4 position of the neighbour -
                               // that of the slice's first row, modulo 2^24) << 8 | entry of Jd; or nullptr
     const int64_t *sell_off;  // [forms + 1]
-    const int2 *slice;        // [nslice] (form, first row) of each slice; row l is first + l * period
+    const SliceRef *slice;    // [nslice]; row l of a slice is row + l * cls.period
     int64_t nslice;
-    int period;               // the rows of a slice are this far apart
-    int period_rest;          // n mod period, and the slices of a class of ceil(n / period) and of
-    int period_hi, period_lo; // floor(n / period) rows (x4_pos)
+    Classes cls;              // where spin i lies in x4 (cls.pos)
     R *x4;                    // [4 * 32 nslice] the spins read by the sliced pass, (x, y, z, 0) each, slice by
                               // slice
     const R *Jd;              // [nJd <= 256] distinct J_ij / mu_s,i of the packed bonds (and 0)

@@ -169,9 +169,6 @@ struct Aos {
     }
 };
 
-template <typename R>
-__device__ __forceinline__ int64_t x4_pos(const KArgs<R> &a, int64_t i);
-
 // The row form of spin i (0 when the handle reads the CSR).
 template <typename R>
 __device__ __forceinline__ int form_of(const KArgs<R> &a, int64_t i) {
@@ -699,7 +696,7 @@ __device__ __forceinline__ void predictor_tile(const KArgs<R> &a, const TileDesc
         const int form = next_form;  // read a slot ahead: the chain form -> offsets -> spins starts at the offsets
         if (k + BS < td.count) next_form = form_of(a, i + BS);
         const MatDesc<R> &m = mat_at<Mode>(a, i);
-        const int64_t i4 = V4 && Mode == kRows ? x4_pos(a, i) : i;  // the row passes gather from s4 and p4
+        const int64_t i4 = V4 && Mode == kRows ? a.cls.pos(i) : i;  // the row passes gather from s4 and p4
         R s0, s1, s2;
         src.get(i4, s0, s1, s2);
         const bool given = sqrtT > (R)0 && (Split || rot >= pre_slot);  // drawn beforehand (k_gauss, or the
@@ -788,7 +785,7 @@ __device__ __forceinline__ void corrector_tile(const KArgs<R> &a, const TileDesc
         const int form = next_form;  // a slot ahead, as the predictor
         if (k + BS < td.count) next_form = form_of(a, i + BS);
         const MatDesc<R> &m = mat_at<Mode>(a, i);
-        const int64_t i4 = V4 && Mode == kRows ? x4_pos(a, i) : i;
+        const int64_t i4 = V4 && Mode == kRows ? a.cls.pos(i) : i;
         R s0, s1, s2;
         src.get(i4, s0, s1, s2);
         R q0, q1, q2, t0 = 0, t1 = 0, t2 = 0;  // the half step and the thermal field
@@ -941,11 +938,11 @@ __device__ __forceinline__ void predictor_pass(const KArgs<R> &a, uint64_t step,
 // order the row passes gather from).
 static __global__ void __launch_bounds__(256) k_pack_state(const KArgs<float> a) {
     for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < a.n; i += (int64_t)gridDim.x * 256)
-        a.s4[a.ex ? x4_pos(a, i) : i] = make_float4(a.sx[i], a.sy[i], a.sz[i], 0.0f);
+        a.s4[a.ex ? a.cls.pos(i) : i] = make_float4(a.sx[i], a.sy[i], a.sz[i], 0.0f);
 }
 static __global__ void __launch_bounds__(256) k_unpack_state(const KArgs<float> a) {
     for (int64_t i = (int64_t)blockIdx.x * 256 + threadIdx.x; i < a.n; i += (int64_t)gridDim.x * 256) {
-        const int64_t at = a.ex ? x4_pos(a, i) : i;
+        const int64_t at = a.ex ? a.cls.pos(i) : i;
         const float4 s = a.s4[at], p = a.p4[at];
         a.sx[i] = s.x;
         a.sy[i] = s.y;
@@ -1358,20 +1355,10 @@ __global__ void __launch_bounds__(BS, sizeof(R) == 8 || BS >= 512 ? 0 : heun_blo
 // the gathers' L1 misses.  U bonds in flight a warp: 2 1.65, 3 1.36, 4 1.22, 8 1.32, 16 1.53 ms per four steps
 // (more evict each other's lines); words loaded past the L1 1.71, two slices to a warp 2.0 ms.
 //
-// Where spin i lies in the copy: class i mod period, then i / period, classes padded to whole slices.
-template <typename R>
-__device__ __forceinline__ int64_t x4_pos(const KArgs<R> &a, int64_t i) {
-    if (a.period == 1) return i;
-    const uint32_t c = (uint32_t)i / (uint32_t)a.period, b = (uint32_t)i - c * (uint32_t)a.period;
-    const int rest = a.period_rest, over = (int)b - rest;
-    const int first = over <= 0 ? (int)b * a.period_hi : rest * a.period_hi + over * a.period_lo;
-    return 32 * (int64_t)first + c;
-}
-
 template <typename R>
 __global__ void k_pack4(const KArgs<R> a, const R *X, const R *Y, const R *Z) {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < a.n; i += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t at = x4_pos(a, i);
+        const int64_t at = a.cls.pos(i);
         if constexpr (sizeof(R) == 4) {
             reinterpret_cast<float4 *>(a.x4)[at] = make_float4(X[i], Y[i], Z[i], 0.f);
         } else {
@@ -1413,8 +1400,8 @@ __global__ void __launch_bounds__(kSellBlock) k_rows_sell(const KArgs<R> a) {
     const int64_t nwarps = ((int64_t)gridDim.x * kSellBlock) >> 5;
     const int64_t npos = 32 * a.nslice;
     for (int64_t s = warp; s < a.nslice; s += nwarps) {
-        const int2 sl = __ldg(a.slice + s);
-        const int64_t row = sl.y + (int64_t)lane * a.period;
+        const int2 sl = __ldg(reinterpret_cast<const int2 *>(a.slice) + s);  // (form, first row)
+        const int64_t row = sl.y + (int64_t)lane * a.cls.period;
         const uint32_t base = (uint32_t)(32 * s);
         const int64_t o = __ldg(a.sell_off + sl.x);
         const int w = (int)((__ldg(a.sell_off + sl.x + 1) - o) >> 5);

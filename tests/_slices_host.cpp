@@ -1,0 +1,46 @@
+// The host code that packs long rows into slices, as plain C functions for tests/test_slices_host.py.
+#include "ss_slices.h"
+
+#include <new>
+
+using namespace ss;
+
+extern "C" {
+
+// Packs the rows; sizes[] = (period, slices, distinct slices, words), nothing is copied out.
+// Returns 0, or 1 when the host memory does not suffice.
+int slices_pack(int64_t n, const int32_t *rp, const int32_t *col, const uint8_t *bid, int zero, Slices **out,
+                int64_t sizes[4]) {
+    *out = nullptr;
+    Slices *s = new Slices;
+    try {
+        pack_slices(n, rp, col, bid, zero, *s);
+    } catch (const std::bad_alloc &) {
+        delete s;
+        return 1;
+    }
+    sizes[0] = s->period;
+    sizes[1] = (int64_t)s->slice.size();
+    sizes[2] = (int64_t)s->off.size() - 1;
+    sizes[3] = (int64_t)s->words.size();
+    *out = s;
+    return 0;
+}
+
+void slices_copy(const Slices *s, int32_t *slice, int64_t *off, uint32_t *words) {
+    std::memcpy(slice, s->slice.data(), s->slice.size() * sizeof(SliceRef));
+    std::memcpy(off, s->off.data(), s->off.size() * sizeof(int64_t));
+    std::memcpy(words, s->words.data(), s->words.size() * sizeof(uint32_t));
+}
+
+void slices_free(Slices *s) { delete s; }
+
+void slices_positions(int64_t n, int period, int64_t *pos) {
+    const Classes c = Classes::of(n, period);
+    for (int64_t i = 0; i < n; ++i) pos[i] = c.pos(i);
+}
+
+uint64_t slices_hash(const uint32_t *words, int64_t count) {
+    return slice_hash(std::vector<uint32_t>(words, words + count));
+}
+}
