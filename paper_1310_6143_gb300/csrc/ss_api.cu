@@ -1135,15 +1135,9 @@ ss_status build_ell(ss_system *h, const std::vector<R> &J) {
     const int64_t n = h->n, nnz = h->nnz;
     if (h->npat > 0 || h->J_tensor || nnz <= 0 || h->max_row > kPatRow || n >= (int64_t(1) << 24)) return SS_OK;
     const int W = h->max_row <= kShortRow ? kShortRow : kPatRow;
-    std::vector<R> dict(1, (R)0);  // entry 0: the padding
-    size_t last = 0;
-    for (int64_t k = 0; k < nnz; ++k) {
-        if (std::memcmp(&J[k], &dict[last], sizeof(R)) == 0) continue;  // (bonds of a row mostly repeat)
-        for (last = 0; last < dict.size() && std::memcmp(&J[k], &dict[last], sizeof(R)) != 0;) ++last;
-        if (last < dict.size()) continue;
-        if (dict.size() == 256) return SS_OK;
-        dict.push_back(J[k]);
-    }
+    std::vector<R> dict;
+    int zero = -1;
+    if (!bond_dictionary<R>(J, nnz, dict, zero, nullptr)) return SS_OK;
     void *J_dev = nullptr;
     uint32_t *ell = nullptr;
     if (dalloc(h, (void **)&ell, (size_t)W * n * sizeof(uint32_t)) != cudaSuccess ||
@@ -1154,7 +1148,7 @@ ss_status build_ell(ss_system *h, const std::vector<R> &J) {
     }
     SS_CUDA(h, cudaMemcpyAsync(J_dev, dict.data(), dict.size() * sizeof(R), cudaMemcpyHostToDevice, h->stream));
     SS_CUDA(h, launch_build_ell<R>(h->row_ptr, h->col, static_cast<const R *>(h->J), static_cast<const R *>(J_dev),
-                                   (int)dict.size(), n, W, ell, h->stream));
+                                   (int)dict.size(), zero, n, W, ell, h->stream));
     SS_CUDA(h, cudaStreamSynchronize(h->stream));  // the host vectors go out of scope
     h->ell = ell;
     h->ell_J = J_dev;
@@ -1280,7 +1274,7 @@ ss_status upload_system(ss_system *h, const std::vector<HostSys> &hs) {
         std::vector<R> dict;
         std::vector<uint8_t> bid;
         int zero = -1;
-        if (bond_dictionary<R>(J, nnz, dict, bid, zero)) {
+        if (bond_dictionary<R>(J, nnz, dict, zero, &bid)) {
             const ss_status ps = build_slices(h, rp, col, bid, zero);
             if (ps != SS_OK) return ps;
             SS_CUDA(h, dalloc(h, &h->Jd, dict.size() * sizeof(R)));

@@ -32,12 +32,12 @@ cudaError_t launch_finalize_ring(const SysDesc *sys, const int32_t *sys_tiles, i
 }
 
 template <typename R>
-__global__ void k_build_ell(const int32_t *row_ptr, const int32_t *col, const R *J, const R *dict, int ndict, int64_t n,
-                            int W, uint32_t *ell) {
+__global__ void k_build_ell(const int32_t *row_ptr, const int32_t *col, const R *J, const R *dict, int ndict, int zero,
+                            int64_t n, int W, uint32_t *ell) {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         const int32_t b = row_ptr[i], len = row_ptr[i + 1] - b;
         for (int32_t k = 0; k < W; ++k) {
-            uint32_t w = (uint32_t)i << 8;  // padding: the spin itself with J = 0
+            uint32_t w = ((uint32_t)i << 8) | (uint32_t)zero;  // padding: the spin itself with J = 0
             if (k < len) {
                 int e = 0;
                 while (e + 1 < ndict && !(dict[e] == J[b + k])) ++e;
@@ -50,15 +50,15 @@ __global__ void k_build_ell(const int32_t *row_ptr, const int32_t *col, const R 
 
 template <typename R>
 cudaError_t launch_build_ell(const int32_t *row_ptr, const int32_t *col, const R *J, const R *dict, int ndict,
-                             int64_t n, int W, uint32_t *ell, cudaStream_t s) {
+                             int zero, int64_t n, int W, uint32_t *ell, cudaStream_t s) {
     const int64_t g = (n + 255) / 256;
-    k_build_ell<R><<<(int)(g < 65536 ? g : 65536), 256, 0, s>>>(row_ptr, col, J, dict, ndict, n, W, ell);
+    k_build_ell<R><<<(int)(g < 65536 ? g : 65536), 256, 0, s>>>(row_ptr, col, J, dict, ndict, zero, n, W, ell);
     return cudaGetLastError();
 }
 template cudaError_t launch_build_ell<float>(const int32_t *, const int32_t *, const float *, const float *, int,
-                                             int64_t, int, uint32_t *, cudaStream_t);
+                                             int, int64_t, int, uint32_t *, cudaStream_t);
 template cudaError_t launch_build_ell<double>(const int32_t *, const int32_t *, const double *, const double *, int,
-                                              int64_t, int, uint32_t *, cudaStream_t);
+                                              int, int64_t, int, uint32_t *, cudaStream_t);
 
 __global__ void k_debug_philox(uint4 ctr0, uint2 key, long long count, uint32_t *out) {
     for (long long k = blockIdx.x * (long long)blockDim.x + threadIdx.x; k < count;

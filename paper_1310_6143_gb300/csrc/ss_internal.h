@@ -234,10 +234,10 @@ constexpr unsigned int kErrBounds = 4u;   // checked builds: an index out of its
 void set_global_error(const char *msg);
 
 // The columns of packed bonds (KArgs.ell, W words per row) of a CSR on the device; every J is in
-// the dictionary, whose entry 0 is the padding's 0.
+// the dictionary, whose entry `zero` is the padding's 0.
 template <typename R>
 cudaError_t launch_build_ell(const int32_t *row_ptr, const int32_t *col, const R *J, const R *dict, int ndict,
-                             int64_t n, int W, uint32_t *ell, cudaStream_t s);
+                             int zero, int64_t n, int W, uint32_t *ell, cudaStream_t s);
 
 // Launchers (ss_kernels_f32.cu / ss_kernels_f64.cu).
 template <typename R> cudaError_t launch_predictor(const KArgs<R> &a, int block, int grid, cudaStream_t s);

@@ -46,34 +46,36 @@ struct alignas(8) SliceRef {
     int32_t form, row;
 };
 
-// The distinct J_ij / mu_s,i of the bonds (at most 255, and 0 for padding) and each bond's entry.
+// The distinct J_ij / mu_s,i of the bonds (at most 255 beside 0, which is always there, for padding),
+// the entry of 0, and each bond's entry (if asked for).  False with more.
 template <typename R>
-bool bond_dictionary(const std::vector<R> &J, int64_t nnz, std::vector<R> &dict, std::vector<uint8_t> &bid, int &zero) {
+bool bond_dictionary(const std::vector<R> &J, int64_t nnz, std::vector<R> &dict, int &zero, std::vector<uint8_t> *bid) {
     using Bits = typename std::conditional<sizeof(R) == 8, uint64_t, uint32_t>::type;
     constexpr int kSlots = 1024;
     std::vector<Bits> key(kSlots);
     std::vector<int> id(kSlots, -1);
     Bits last = 0;
-    bid.resize((size_t)nnz);
+    dict.clear();
+    if (bid) bid->resize((size_t)nnz);
     zero = -1;
     for (int64_t k = 0; k < nnz; ++k) {
         Bits b;
         std::memcpy(&b, &J[k], sizeof(R));
         if (k > 0 && b == last) {  // (bonds of a row mostly repeat)
-            bid[(size_t)k] = bid[(size_t)k - 1];
+            if (bid) (*bid)[(size_t)k] = (*bid)[(size_t)k - 1];
             continue;
         }
         last = b;
         uint32_t hsh = (uint32_t)(((uint64_t)b * 0x9E3779B97F4A7C15ull) >> 54);  // 10 bits
         while (id[hsh] >= 0 && key[hsh] != b) hsh = (hsh + 1) & (kSlots - 1);
         if (id[hsh] < 0) {
-            if (dict.size() == 255) return false;
+            if (b != 0 && dict.size() - (zero >= 0 ? 1 : 0) == 255) return false;
             key[hsh] = b;
             id[hsh] = (int)dict.size();
             if (b == 0) zero = id[hsh];
             dict.push_back(J[k]);
         }
-        bid[(size_t)k] = (uint8_t)id[hsh];
+        if (bid) (*bid)[(size_t)k] = (uint8_t)id[hsh];
     }
     if (zero < 0) {
         zero = (int)dict.size();

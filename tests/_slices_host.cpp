@@ -43,4 +43,14 @@ void slices_positions(int64_t n, int period, int64_t *pos) {
 uint64_t slices_hash(const uint32_t *words, int64_t count) {
     return slice_hash(std::vector<uint32_t>(words, words + count));
 }
+
+// Entries of the dictionary, or -1 with too many; zero and each bond's entry.
+int slices_dictionary(const float *J, int64_t nnz, float *dict, int *zero, uint8_t *bid) {
+    std::vector<float> d;
+    std::vector<uint8_t> b;
+    if (!bond_dictionary<float>(std::vector<float>(J, J + nnz), nnz, d, *zero, bid ? &b : nullptr)) return -1;
+    std::memcpy(dict, d.data(), d.size() * sizeof(float));
+    if (bid) std::memcpy(bid, b.data(), b.size());
+    return (int)d.size();
+}
 }

@@ -144,6 +144,34 @@ def test_dilute_impurities_pack_in_linear_time(host):
     assert len(off) - 1 > 40_000
 
 
+def _dictionary(lib, J):
+    d, zero, bid = np.zeros(256, np.float32), ctypes.c_int(), np.zeros(len(J), np.uint8)
+    k = lib.slices_dictionary(_p(J), ctypes.c_int64(len(J)), _p(d), ctypes.byref(zero), _p(bid))
+    return (None if k < 0 else d[:k]), zero.value, bid
+
+
+@pytest.mark.parametrize("values,with_zero", [(1, False), (1, True), (254, True), (255, False), (255, True), (256, False)])
+def test_dictionary_of_bond_values(host, values, with_zero):
+    rng = np.random.default_rng(values)
+    v = np.concatenate([1e-3 * np.arange(1, values + 1), [0.0] * with_zero]).astype(np.float32)
+    J = np.concatenate([v, rng.choice(v, 5000)])
+    d, zero, bid = _dictionary(host, J)
+    if values > 255:
+        assert d is None
+        return
+    assert len(d) == values + 1 and d[zero] == 0.0
+    np.testing.assert_array_equal(d[bid], J)
+
+
+def test_dictionary_of_many_values_in_linear_time(host):
+    # 200 values in no order, as disordered exchange has them: 20 M bonds at a few ns each
+    J = np.random.default_rng(3).integers(1, 201, 20_000_000).astype(np.float32)
+    t0 = time.perf_counter()
+    d, zero, bid = _dictionary(host, J)
+    assert time.perf_counter() - t0 < 1.0
+    assert len(d) == 201
+
+
 def test_create_reports_host_memory_that_runs_out():
     # the table of 2^31 - 1 systems does not fit 1 GB: an error code, not the end of the process
     code = ("import ctypes, resource\n"
