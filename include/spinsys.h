@@ -208,7 +208,10 @@ ss_status set_temperature_schedule(ss_system *h, const double *T_per_step, int64
  * S <- norm(S + dt/2 (dS(S, H) + dS(S', H'))) with the same thermal field in H and H'.
  * Each step records the moment and energy of the state at its start (Eq. spinhamiltonian)
  * into the per-step record ring.  SS_ERR_INVALID_ARG for n < 0; a non-finite spin raised
- * on the device is reported as SS_ERR_NONFINITE by the next synchronising call. */
+ * on the device is reported as SS_ERR_NONFINITE by the next synchronising call.
+ * The first FP32-mixed run of four or more steps by kernels or graphs allocates 56 bytes per
+ * spin to work in.  Without that memory the run gives the same results, slower; a later call
+ * on the handle that needs the memory takes it back. */
 ss_status llg_heun_step(ss_system *h, int64_t n);
 
 /* Advance every system by n >= 0 Monte Carlo steps (asynchronous; Section "Monte Carlo
@@ -454,9 +457,12 @@ ss_status ss_debug_fp64_rate(int32_t mode, double *inst_per_s);
  * after `after` (>= 0) more successful device allocations by the handles of this process,
  * every device allocation fails as if the device were out of memory, so the calls that
  * allocate (create, set_demag, the first mc_step, ...) return SS_ERR_OOM; a negative value
- * switches the injection off.  ss_debug_live_bytes: the device bytes currently held by all
- * handles of this process (a failed create holds none). */
+ * switches the injection off.  ss_debug_limit_bytes: device allocations that would take what
+ * all handles of this process hold above `limit` bytes fail in the same way (negative: off).
+ * ss_debug_live_bytes: the device bytes currently held by all handles of this process (a
+ * failed create holds none). */
 ss_status ss_debug_fail_allocations(int64_t after);
+ss_status ss_debug_limit_bytes(int64_t limit);
 int64_t ss_debug_live_bytes(void);
 
 /* ---------------------------------------------------------------------------------

@@ -30,7 +30,7 @@ EXPORTS = (
     "spin_system_set_barrier_test", "spin_system_sync", "spin_system_time_kernels", "ss_debug_philox", "ss_debug_gaussians",
     "llg_heun_step_noalloc", "spin_system_set_draw_ahead", "spin_system_set_row_patterns", "spin_system_set_gaussian_pass", "spin_system_time_passes", "ss_debug_fp64_rate", "mc_step", "get_mc_stats", "set_demag", "llg_midpoint_step",
     "spin_system_set_exchange_rows", "spin_system_time_rows", "llg_semi_implicit_step",
-    "ss_debug_fail_allocations", "ss_debug_live_bytes",
+    "ss_debug_fail_allocations", "ss_debug_limit_bytes", "ss_debug_live_bytes",
     "get_demag_field",
     "spin_slab_create", "spin_slab_info", "spin_slab_halo_runs", "get_state_device", "spin_system_heun_pass",
     "ss_last_error", "ss_status_string",
@@ -138,6 +138,7 @@ def load(path: str | None = None) -> ctypes.CDLL:
         "llg_midpoint_step": [P, I64, I32],
         "llg_semi_implicit_step": [P, I64],
         "ss_debug_fail_allocations": [I64],
+        "ss_debug_limit_bytes": [I64],
         "get_mc_stats": [P, I32, P],
         "set_demag": [P, D, D, I32],
         "get_demag_field": [P, P],

@@ -93,8 +93,10 @@ struct ss_system {
     int mat_bytes = 4;
     void *J = nullptr, *mats = nullptr;
     void *state[12] = {};  // sx sy sz px py pz qx qy qz hx hy hz
-    void *packed = nullptr;  // float4 S, S' and half step + field x, float2 field y, z (FP32-mixed runs of steps;
-                             // nullptr: not available, the steps work on the arrays of `state`)
+    void *packed = nullptr;  // float4 S, S' and half step + field x, float2 field y, z (FP32-mixed runs of steps,
+                             // see ensure_packed; nullptr: the steps work on the arrays of `state`)
+    bool packed_off = false; // no memory for it, or given back
+    bool pinned = false;     // work of the handle was captured by a caller: its buffers stay
     void *ahead[3] = {};   // Gaussians drawn ahead by the corrector (FP32-mixed only)
     int pre_slot = 1 << 30;
     int ahead_q = 5;       // eighths of each tile drawn ahead by the corrector
@@ -207,6 +209,7 @@ struct ss_system {
     int mcgraph_steps = 0;
     bool mcgraph_failed = false;
     int graph_steps = 0;
+    bool graph_packed = false;          // the captured steps work on the float4 spins
     cudaGraphExec_t pgraph = nullptr;  // captured persistent launch (barrier reset + kernel)
     long long pgraph_steps = 0;
     bool pgraph_failed = false;
@@ -255,10 +258,14 @@ ss_status cuda_fail(ss_system *h, cudaError_t e, const char *what) {
 // allocations left before every allocation fails; and the bytes held by all handles.
 std::atomic<int64_t> g_fail_after{-1};
 std::atomic<int64_t> g_live_bytes{0};
+// ss_debug_limit_bytes: allocations that would take the bytes above it fail; < 0 off.
+std::atomic<int64_t> g_byte_limit{-1};
 
-cudaError_t dalloc(ss_system *h, void **p, size_t bytes) {
+cudaError_t try_alloc(ss_system *h, void **p, size_t bytes) {
     *p = nullptr;
     if (bytes == 0) bytes = 16;
+    const int64_t limit = g_byte_limit.load();
+    if (limit >= 0 && g_live_bytes.load() + (int64_t)bytes > limit) return cudaErrorMemoryAllocation;
     int64_t left = g_fail_after.load();
     while (left >= 0) {
         if (left == 0) return cudaErrorMemoryAllocation;
@@ -282,6 +289,37 @@ void dfree(ss_system *h, void *p) {
             return;
         }
     }
+}
+
+void drop_graph(ss_system *h);
+
+// Gives back one of the buffers the handle can do without -- the float4 spins, then the columns of
+// packed bonds -- and with it the captured launches that name it.
+bool release_optional(ss_system *h) {
+    if (h->pinned || (!h->packed && !h->ell)) return false;
+    cudaStreamSynchronize(h->stream);
+    drop_graph(h);
+    if (h->packed) {
+        dfree(h, h->packed);
+        h->packed = nullptr;
+        h->packed_off = true;
+    } else {
+        dfree(h, h->ell);
+        dfree(h, h->ell_J);
+        h->ell = nullptr;
+        h->ell_J = nullptr;
+    }
+    return true;
+}
+
+// Memory that a call cannot do without: what fitted without the optional buffers still fits.
+cudaError_t dalloc(ss_system *h, void **p, size_t bytes) {
+    cudaError_t e = try_alloc(h, p, bytes);
+    while (e == cudaErrorMemoryAllocation && release_optional(h)) {
+        cudaGetLastError();
+        e = try_alloc(h, p, bytes);
+    }
+    return e;
 }
 
 size_t real_size(const ss_system *h) { return h->precision == SS_FP32_MIXED ? 4 : 8; }
@@ -687,8 +725,34 @@ constexpr int64_t kPackedMin = 4;
 // Whether a run of n steps in the graph or plain-launch mode works on float4 spins: FP32-mixed,
 // not a slab (its halo refresh reads S'), not the split step (the Gaussians come in arrays), and
 // with long rows only the packed-bond pass, which reads float4 spins itself.
-bool packed_run(const ss_system *h, int64_t n) {
-    return h->packed && n >= kPackedMin && !split_step(h) && (!h->rows || h->sell);
+bool wants_packed(const ss_system *h, int64_t n) {
+    return h->precision == SS_FP32_MIXED && h->slab_own < 0 && n >= kPackedMin && !split_step(h) && (!h->rows || h->sell);
+}
+bool packed_run(const ss_system *h, int64_t n) { return h->packed && wants_packed(h, n); }
+
+size_t packed_bytes(const ss_system *h) { return (size_t)packed_spins(h) * (3 * sizeof(float4) + sizeof(float2)); }
+
+// The float4 spins, allocated by the first run that takes them (handles that only do Monte Carlo,
+// alternative integrators, single steps or the cluster, persistent and system-block steps never hold
+// their 56 bytes per spin; allocating them takes 0.2 ms).  Without the memory the steps work on the
+// arrays.  Allowed while a stream is captured: nothing is enqueued on it here.
+void ensure_packed(ss_system *h) {
+    if (h->packed || h->packed_off) return;
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    cudaError_t e = try_alloc(h, &h->packed, packed_bytes(h));
+    if (e == cudaSuccess && h->nslice > 0) {  // (the classes' padding has to be finite)
+        const cudaStream_t s = h->pinned ? h->own_stream : h->stream;
+        e = cudaMemsetAsync(h->packed, 0, packed_bytes(h), s);
+        if (e == cudaSuccess && s != h->stream) e = cudaStreamSynchronize(s);
+        if (e != cudaSuccess) dfree(h, h->packed);
+    }
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        h->packed = nullptr;
+        h->packed_off = true;
+    }
 }
 
 int packed_grid(const ss_system *h, int which) {
@@ -980,8 +1044,10 @@ int graph_len(const ss_system *h) {
 }
 
 cudaError_t ensure_graph(ss_system *h) {
-    if (h->graph) return cudaSuccess;
     const int g = graph_len(h);
+    if (wants_packed(h, g)) ensure_packed(h);
+    if (h->graph && h->graph_packed != packed_run(h, g)) drop_graph(h);
+    if (h->graph) return cudaSuccess;
     cudaGraph_t graph = nullptr;
     cudaError_t e = cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal);
     if (e != cudaSuccess) return e;
@@ -999,6 +1065,7 @@ cudaError_t ensure_graph(ss_system *h) {
         return e;
     }
     h->graph_steps = g;
+    h->graph_packed = packed_run(h, g);
     return cudaSuccess;
 }
 
@@ -1140,8 +1207,8 @@ ss_status build_ell(ss_system *h, const std::vector<R> &J) {
     if (!bond_dictionary<R>(J, nnz, dict, zero, nullptr)) return SS_OK;
     void *J_dev = nullptr;
     uint32_t *ell = nullptr;
-    if (dalloc(h, (void **)&ell, (size_t)W * n * sizeof(uint32_t)) != cudaSuccess ||
-        dalloc(h, &J_dev, dict.size() * sizeof(R)) != cudaSuccess) {
+    if (try_alloc(h, (void **)&ell, (size_t)W * n * sizeof(uint32_t)) != cudaSuccess ||
+        try_alloc(h, &J_dev, dict.size() * sizeof(R)) != cudaSuccess) {
         cudaGetLastError();
         if (ell) dfree(h, ell);
         return SS_OK;
@@ -1375,8 +1442,7 @@ ss_status set_rows(ss_system *h, int32_t mode) {
     // the classes' padding in the float4 spins is gathered with J = 0 and has to be finite, whatever
     // runs without row passes left there
     if (on && !h->rows && h->packed && h->nslice > 0)
-        SS_CUDA(h, cudaMemsetAsync(h->packed, 0, (size_t)packed_spins(h) * (3 * sizeof(float4) + sizeof(float2)),
-                                   h->stream));
+        SS_CUDA(h, cudaMemsetAsync(h->packed, 0, packed_bytes(h), h->stream));
     h->rows_req = mode;
     if (on != h->rows) drop_graph(h);
     h->rows = on;
@@ -1569,13 +1635,6 @@ ss_status create_impl(const ss_params *systems, int32_t count, ss_system **out, 
         cudaGetLastError();  // the control words and records are copied to pageable memory
         h->report = nullptr;
     }
-    if (h->precision == SS_FP32_MIXED && !slab) {
-        const size_t bytes = (size_t)packed_spins(h) * (3 * sizeof(float4) + sizeof(float2));
-        if (dalloc(h, &h->packed, bytes) != cudaSuccess)
-            cudaGetLastError();  // not enough memory: the steps work on the arrays of `state`
-        else if (h->nslice > 0 && (e = cudaMemsetAsync(h->packed, 0, bytes, h->stream)) != cudaSuccess)
-            return cleanup(cuda_fail(h, e, "cudaMemsetAsync"));  // (the classes' padding has to be finite)
-    }
     owner.h = nullptr;
     *out = h;
     return SS_OK;
@@ -1584,6 +1643,11 @@ ss_status create_impl(const ss_params *systems, int32_t count, ss_system **out, 
 ss_status usable(ss_system *h) {
     if (!h) return fail(nullptr, SS_ERR_INVALID_ARG, "handle is NULL");
     if (h->bad) return fail(h, SS_ERR_STATE, "handle unusable after an earlier CUDA error: %s", h->err.c_str());
+    if (h->stream != h->own_stream && !h->pinned) {  // (the private stream is captured by the handle alone)
+        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(h->stream, &cs) != cudaSuccess) cudaGetLastError();
+        h->pinned = cs != cudaStreamCaptureStatusNone;
+    }
     return SS_OK;
 }
 
@@ -1621,6 +1685,7 @@ ss_status current_record(ss_system *h, int32_t sys, double rec[kRecComps]) {
 
 template <typename R>
 ss_status time_kernels_impl(ss_system *h, int32_t nsteps, double out_ms[4]) {
+    if (wants_packed(h, nsteps)) ensure_packed(h);
     KArgs<R> a = make_args<R>(h);
     use_rows(h, a);
     const bool split = split_step(h), packed = packed_run(h, nsteps);  // (as the steps of a run that long)
@@ -2342,6 +2407,7 @@ static ss_status advance_steps(ss_system *h, int64_t n) {
     if (mode == SS_EXEC_AUTO && h->n <= kClusterAutoMax && h->nsys == 1 && !cluster_ready(h))
         mode = SS_EXEC_CLUSTER;
     if (mode == SS_EXEC_AUTO) mode = n >= graph_len(h) ? SS_EXEC_GRAPH : SS_EXEC_KERNELS;
+    if ((mode == SS_EXEC_GRAPH || mode == SS_EXEC_KERNELS) && wants_packed(h, n)) ensure_packed(h);
     if (mode == SS_EXEC_GRAPH && !h->graph_failed) {
         e = ensure_graph(h);
         if (e != cudaSuccess) {
@@ -3126,6 +3192,11 @@ ss_status spin_system_set_barrier_test(ss_system *h, int32_t extra, int64_t time
 
 ss_status ss_debug_fail_allocations(int64_t after) {
     g_fail_after.store(after < 0 ? -1 : after);
+    return SS_OK;
+}
+
+ss_status ss_debug_limit_bytes(int64_t limit) {
+    g_byte_limit.store(limit < 0 ? -1 : limit);
     return SS_OK;
 }
 
