@@ -398,8 +398,9 @@ ss_status spin_system_set_draw_ahead(ss_system *h, int32_t eighths);
  * steps each, keep the fastest, and write it to *out_info.  The spins and the step
  * counter are restored afterwards, so the trajectory is unchanged.  With the environment
  * variable SPINSYS_AUTOTUNE_CACHE naming a file, a workload tuned before on the same device
- * (same precision, spins, bonds, systems, largest system, exchange-row mode and kernel
- * variant) takes its stored choice without trial runs, and a new result is appended. */
+ * (same precision, spins, bonds, systems, largest system, exchange-row mode, kernel variant and
+ * storage of the rows) by this version's kernels takes its stored choice without trial runs, and a
+ * new result is appended. */
 ss_status spin_system_autotune(ss_system *h, int32_t trial_steps, ss_info *out_info);
 
 /* The handle's sizes and current launch settings into *out (caller-owned).  `exec` is the mode

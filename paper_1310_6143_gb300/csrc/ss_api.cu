@@ -3042,15 +3042,19 @@ ss_status spin_system_time_rows(ss_system *h, int32_t launches, double *out_ms) 
 }
 
 // The autotune cache (SPINSYS_AUTOTUNE_CACHE): one line per tuned workload, "key<TAB>exec block
-// tile draw-ahead", the key naming the device and what the launch shape depends on.
+// tile draw-ahead gaussian-pass", the key naming the device and what the launch shape depends on.  Its
+// version goes up when the kernels change so that shapes timed on the old ones say nothing about them
+// (v3: float4 runs, columns of packed bonds).
 static std::string autotune_key(const ss_system *h) {
     cudaDeviceProp prop{};
     if (cudaGetDeviceProperties(&prop, h->device) != cudaSuccess) cudaGetLastError();
     int64_t nmax = 0;
     for (int64_t v : h->sys_n) nmax = std::max(nmax, v);
+    // how a thread reads its row: forms (two-byte indices), columns of packed bonds, or the CSR
+    const char *store = !h->use_pat ? "csr" : h->npat > 0 ? (h->pat_wide ? "forms2" : "forms") : h->ell ? "columns" : "csr";
     char buf[512];
-    std::snprintf(buf, sizeof(buf), "v2|%s|%d|%lld|%lld|%d|%lld|%d|%d", prop.name, h->precision, (long long)h->n,
-                  (long long)h->nnz, h->nsys, (long long)nmax, h->rows ? (h->sell ? 3 : 2) : 1, step_mode(h));
+    std::snprintf(buf, sizeof(buf), "v3|%s|%d|%lld|%lld|%d|%lld|%d|%d|%s", prop.name, h->precision, (long long)h->n,
+                  (long long)h->nnz, h->nsys, (long long)nmax, h->rows ? (h->sell ? 3 : 2) : 1, step_mode(h), store);
     for (char *c = buf; *c; ++c)
         if (*c == '\t' || *c == '\n') *c = ' ';
     return buf;
