@@ -395,7 +395,8 @@ ss_status spin_system_set_gaussian_pass(ss_system *h, int32_t mode);
 ss_status spin_system_set_draw_ahead(ss_system *h, int32_t eighths);
 
 /* Time the candidate (exec, block, tile, draw-ahead, Gaussian pass) choices on this handle over `trial_steps`
- * steps each, keep the fastest, and write it to *out_info.  The spins and the step
+ * steps each (FP32-mixed: at least four, the length from which runs take float4 spins; their packing
+ * before and after a run is not timed), keep the fastest, and write it to *out_info.  The spins and the step
  * counter are restored afterwards, so the trajectory is unchanged.  With the environment
  * variable SPINSYS_AUTOTUNE_CACHE naming a file, a workload tuned before on the same device
  * (same precision, spins, bonds, systems, largest system, exchange-row mode, kernel variant and

@@ -2373,7 +2373,8 @@ ss_status set_temperature_schedule(ss_system *h, const double *T_per_step, int64
     return SS_OK;
 }
 
-static ss_status advance_steps(ss_system *h, int64_t n);
+// (from, to: recorded around the steps themselves, without the packing and unpacking of a run)
+static ss_status advance_steps(ss_system *h, int64_t n, cudaEvent_t from = nullptr, cudaEvent_t to = nullptr);
 
 ss_status llg_heun_step(ss_system *h, int64_t n) {
     ss_status st = usable(h);
@@ -2399,7 +2400,7 @@ ss_status llg_heun_step(ss_system *h, int64_t n) {
     return SS_OK;
 }
 
-static ss_status advance_steps(ss_system *h, int64_t n) {
+static ss_status advance_steps(ss_system *h, int64_t n, cudaEvent_t from, cudaEvent_t to) {
     cudaError_t e = cudaSuccess;
     int mode = h->exec;
     // automatic: the cluster step for a small single system that it takes (on GB300 a few
@@ -2420,6 +2421,7 @@ static ss_status advance_steps(ss_system *h, int64_t n) {
     }
     const bool packed = (mode == SS_EXEC_GRAPH || mode == SS_EXEC_KERNELS) && packed_run(h, n);
     if (packed && (e = packed_state(h, true)) != cudaSuccess) return cuda_fail(h, e, "step launch");
+    if (from && (e = cudaEventRecord(from, h->stream)) != cudaSuccess) return cuda_fail(h, e, "cudaEventRecord");
     if (mode == SS_EXEC_GRAPH) {
         int64_t left = n;
         while (left >= h->graph_steps) {
@@ -2453,6 +2455,7 @@ static ss_status advance_steps(ss_system *h, int64_t n) {
     } else {
         e = enqueue_kernels(h, n, packed);
     }
+    if (e == cudaSuccess && to) e = cudaEventRecord(to, h->stream);
     if (e == cudaSuccess && packed) e = packed_state(h, false);
     if (e != cudaSuccess) return cuda_fail(h, e, "step launch");
     h->step += n;
@@ -3135,6 +3138,19 @@ ss_status spin_system_autotune(ss_system *h, int32_t trial_steps, ss_info *out_i
     cudaEvent_t e0, e1;
     SS_CUDA(h, cudaEventCreate(&e0));
     SS_CUDA(h, cudaEventCreate(&e1));
+    // What longer runs launch: over float4 spins where they take them, whose packing and unpacking
+    // (once a run, however long) would count only against the candidates that do it.
+    const int64_t trial = mixed ? std::max<int64_t>(trial_steps, kPackedMin) : trial_steps;
+    auto timed_run = [&] {
+        if (!h->demag_on) return advance_steps(h, trial, e0, e1);
+        cudaEventRecord(e0, h->stream);
+        const ss_status s = llg_heun_step(h, trial);
+        cudaEventRecord(e1, h->stream);
+        return s;
+    };
+    // (a candidate that does not fit beside the float4 spins is left out)
+    const bool pinned = h->pinned;
+    h->pinned = true;
     float best = 1e30f;
     Cand bestc{h->exec, h->block, h->tile, h->ahead_q, h->gauss_mode};
     for (const Cand &c : cands) {
@@ -3142,14 +3158,12 @@ ss_status spin_system_autotune(ss_system *h, int32_t trial_steps, ss_info *out_i
         if (spin_system_set_gaussian_pass(h, c.gauss) != SS_OK) { h->bad = false; continue; }
         if (spin_system_set_launch(h, c.block, c.tile) != SS_OK) continue;
         if (spin_system_set_exec(h, (ss_exec)c.exec) != SS_OK) continue;
-        if (llg_heun_step(h, std::min(trial_steps, 4)) != SS_OK) { h->bad = false; continue; }
+        if (llg_heun_step(h, std::min<int64_t>(trial, 4)) != SS_OK) { h->bad = false; continue; }
         // the shorter of two timed runs: one run of a few steps of a small system is noisy
         float ms = 1e30f;
         bool ok = true;
         for (int r = 0; r < 2 && ok; ++r) {
-            cudaEventRecord(e0, h->stream);
-            if (llg_heun_step(h, trial_steps) != SS_OK) { h->bad = false; ok = false; break; }
-            cudaEventRecord(e1, h->stream);
+            if (timed_run() != SS_OK) { h->bad = false; ok = false; break; }
             if (cudaEventSynchronize(e1) != cudaSuccess) { cudaGetLastError(); ok = false; break; }
             float t = 0.f;
             cudaEventElapsedTime(&t, e0, e1);
@@ -3161,6 +3175,7 @@ ss_status spin_system_autotune(ss_system *h, int32_t trial_steps, ss_info *out_i
             bestc = c;
         }
     }
+    h->pinned = pinned;
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     h->ahead_q = bestc.ahead;

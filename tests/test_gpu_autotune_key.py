@@ -41,3 +41,19 @@ def test_entries_of_older_kernels_are_not_taken(cache):
         info = s.autotune(4)
     assert (info["block"], info["tile"]) != (512, 8192)
     assert len(cache.read_text().splitlines()) == 2
+
+
+def test_trials_launch_what_runs_launch():
+    # however few steps are asked for: the trials run over the float4 spins that runs take
+    from paper_1310_6143_gb300.system import SpinSystem
+
+    with SpinSystem(L.film(24, 20, 17), **KW) as s:
+        held, ref = s.info()["device_bytes"], s.spins()
+        s.autotune(1)
+        assert (s.spins() == ref).all() and s.step_index == 0
+        s.set_gaussian_pass(0)
+        s.set_launch(256, 256)
+        now = s.info()["device_bytes"]
+        s.set_exec("kernels")
+        s.step(8)
+        assert s.info()["device_bytes"] == now > held + 56 * s.n
