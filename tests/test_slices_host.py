@@ -81,6 +81,17 @@ def test_words_give_the_rows_back(host, n, basis):
     assert seen.all()
 
 
+@pytest.mark.parametrize("vacancies", [0, 1, 2, 3])
+def test_lattice_sizes_off_the_period(host, vacancies):
+    # the lattices that tests/test_gpu_uneven_rows.py steps: period 4, classes of 225 and 224 rows
+    from test_gpu_uneven_rows import fcc_with_vacancies
+
+    lat = fcc_with_vacancies(vacancies)
+    period, sl, off, words = _pack(host, lat.row_ptr.astype(np.int32), lat.col.astype(np.int32),
+                                   np.zeros(lat.nnz, np.uint8), 1)
+    assert period == 4 and lat.n == 900 - vacancies and len(sl) == 32 - vacancies
+
+
 @pytest.mark.parametrize("period", [1, 2, 3, 4, 6, 8])
 def test_positions_are_distinct_and_in_range(host, period):
     for n in list(range(period, 300)) + [4093, 4096, 4099]:
