@@ -22,6 +22,7 @@
 
 #include "../../include/spinsys.h"
 #include "ss_internal.h"
+#include "ss_shape.h"
 
 using namespace ss;
 
@@ -1652,7 +1653,7 @@ ss_status usable(ss_system *h) {
 }
 
 // Whether the measurement reports to host memory itself.
-bool reports(const ss_system *h) { return h->report && h->nsys <= kMcInlineSystems; }
+bool reports(const ss_system *h) { return h->report && h->nsys <= kReportSystems; }
 
 template <typename R>
 ss_status measure(ss_system *h) {
@@ -1948,23 +1949,13 @@ ss_status mc_prepare(ss_system *h) {
                                h->stream));
     if (ncol <= 2 && n > 0) {
         // tiles of at most `tile` trials within one system, per colour class; partial slots system by
-        // system (class 0's tiles of the system, then class 1's).  Classes of fewer than 256 trials
-        // per SM take 64 (k_mc_colour_rec), others whole 256-thread rounds, as many as leave the
-        // busiest SM the least to do (as default_shape).
-        const int64_t sms = std::max(h->sm_count, 1), most = h->mc_cstart[1];
-        h->mc_small = most < 256 * sms;
-        int64_t kMcTile = 64;
-        if (!h->mc_small) {
-            double least = 1e300;
-            for (int r = 1; r <= 10; ++r) {
-                const int64_t tiles = (most + 256 * r - 1) / (256 * r);
-                const double cost = (double)((tiles + sms - 1) / sms) * (r + 0.3);
-                if (cost < least) {
-                    least = cost;
-                    kMcTile = 256 * r;
-                }
-            }
-        }
+        // system (class 0's tiles of the system, then class 1's)
+        std::vector<int64_t> trials[2];  // of each system in the class
+        for (int c = 0; c < 2; ++c) trials[c].assign((size_t)h->nsys, 0);
+        for (int s = 0; s < h->nsys; ++s)
+            for (int64_t i = h->sys_offset[s]; i < h->sys_offset[s] + h->sys_n[s]; ++i) ++trials[colour[i]][(size_t)s];
+        const int64_t tile = mc_tile(h->precision == SS_FP32_MIXED, h->sm_count, h->nsys <= kMcInlineSystems, trials);
+        h->mc_small = tile < 256;
         std::vector<TileDesc> tl[2];
         std::vector<int32_t> sl[2];
         std::vector<int32_t> sys_slots((size_t)h->nsys + 1, 0);
@@ -1977,10 +1968,10 @@ ss_status mc_prepare(ss_system *h) {
                 const int32_t *b0 = order.data() + h->mc_cstart[c], *b1 = order.data() + h->mc_cstart[c + 1];
                 const int64_t r0 = std::lower_bound(b0, b1, (int32_t)lo) - order.data();
                 const int64_t r1 = std::lower_bound(b0, b1, (int32_t)std::min<int64_t>(hi, INT32_MAX)) - order.data();
-                for (int64_t q = r0; q < r1; q += kMcTile) {
+                for (int64_t q = r0; q < r1; q += tile) {
                     TileDesc t;
                     t.start = q;
-                    t.count = (int32_t)std::min<int64_t>(kMcTile, r1 - q);
+                    t.count = (int32_t)std::min<int64_t>(tile, r1 - q);
                     t.sys = s;
                     tl[c].push_back(t);
                     sl[c].push_back(next++);

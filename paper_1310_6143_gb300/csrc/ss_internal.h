@@ -205,13 +205,19 @@ struct McArgs {
     const int32_t *sys_slots; // [nsys + 1] first partial slot of each system
 };
 
-// Launches whose last block sums the record (a Monte Carlo step's last colour pass, the on-demand
-// measurement) do so for at most this many systems.
-constexpr int kMcInlineSystems = 8;
+// A Monte Carlo step's last colour pass sums the record of at most this many systems in its last
+// block, one after the other; for more, a launch of a block per system does it.  us per step, in
+// the pass / by a launch: 2 x sc 20^3 25.3 / 27.3, 3 x 28.5 / 28.4, 4 x 31.2 / 28.2, 8 x 40.3 / 29.5
+// (FP32-mixed; FP64 2 x 31.4 / 33.5, 3 x 33.5 / 33.7, 8 x 52.0 / 41.8).
+constexpr int kMcInlineSystems = 2;
+
+// The on-demand measurement sums and reports the records of at most this many systems in its last
+// block (one launch and a wait, against two launches, two copies and a wait).
+constexpr int kReportSystems = 8;
 
 // The host memory of KArgs.report, in doubles: the step counter, error and barrier words as they lie
-// in the control block, then the records of up to kMcInlineSystems systems.
-constexpr int kReportCtl = 0, kReportRec = 8, kReportSize = 8 + kMcInlineSystems * kRecComps;
+// in the control block, then the records of up to kReportSystems systems.
+constexpr int kReportCtl = 0, kReportRec = 8, kReportSize = 8 + kReportSystems * kRecComps;
 
 // Macrocell demagnetising field (Section "Demagnetising fields").
 struct DemagArgs {

@@ -2230,9 +2230,9 @@ __global__ void __launch_bounds__(BS) k_mc_colour_warp1(const KArgs<R> a, const 
 // kMcInlineSystems systems and advances the step counter, which as launches of their own took
 // 17 + 4 of 274 us on a 512 x 512 x 16 film and 8 + 4 of 54 on sc 28^3 in FP64 (ncu).
 //
-// Small classes take 64-thread blocks that read the transform's tables where they lie: a trial is a
-// chain of some 90 FP64 instructions, which an SM sub-partition issues one in 64 cycles, so the
-// trials are spread over every SM, and 64 trials do not repay copying 40 KB of tables.
+// Tiles of 64 trials (mc_tile) take 64-thread blocks that read the transform's tables where they lie:
+// a trial is a chain of some 90 FP64 instructions, which an SM sub-partition issues one in 64 cycles,
+// so the trials are spread over every SM, and 64 trials do not repay copying 40 KB of tables.
 template <typename R, int BS, int Mode, bool First, bool Staged>
 __global__ void __launch_bounds__(BS, (sizeof(R) == 4 ? 1024 : 512) / BS) k_mc_colour_rec(const KArgs<R> a, const McArgs m) {
     __shared__ double red[(BS / 32) * 8];

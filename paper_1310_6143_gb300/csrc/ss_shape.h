@@ -1,0 +1,65 @@
+// Rules that pick launch shapes from sizes, in plain C++ so that they can be checked without a GPU.
+#pragma once
+#include <stdint.h>
+
+#include <algorithm>
+#include <cmath>
+#include <numeric>
+#include <vector>
+
+namespace ss {
+
+// Trials per tile of the colour passes that sum the record (at most two classes): 64, in blocks of as
+// many threads, or r rounds of 256-thread blocks, r to 10 -- whichever a model of the pass, fitted to
+// 46 lattices and batches on GB300, finds cheapest.  A tile lies within one system, so the tiles are
+// counted system by system: a rule that took the class as one run gave 40 systems of 20^3 four tiles
+// of 1,280 and 160 trials each, two on the busiest SM (FP64 202 us per step; now 106), 9 of 40^3
+// FP32-mixed 75 us (now 51).  The model, in rounds of a 256-thread block at full residency
+// (2.8 us FP32-mixed, 17.5 us FP64), of the k tiles on the busiest SM:
+//  - FP32-mixed, r rounds: four blocks are resident on an SM.  Each group of four tiles takes r + 0.8
+//    (0.8: the record's reduction); one, two or three left over wait for latency, and take 2, 1.25 and
+//    1.12 each of what a tile of a full group takes.
+//  - FP64, r rounds: (r + 0.2) k, an eighth more for a lone tile's eight warps.
+//  - 64 trials, whose blocks read the transform's tables where they lie: 2.5 + 0.31 k FP32-mixed,
+//    0.38 + 0.265 k FP64; and, where the pass sums the record itself, 3.75 ns a slot.  Always
+//    for classes of fewer than 256 trials per SM; not for a system of more than 2,048 slots, which one
+//    block sums.
+// Its choice is within 4 % of the fastest on all 46, 0.3 % on average.
+inline int64_t mc_tile(bool mixed, int sm_count, bool sums_record, const std::vector<int64_t> (&trials)[2]) {
+    const int64_t sms = std::max(sm_count, 1);
+    auto total = [](const std::vector<int64_t> &t) { return std::accumulate(t.begin(), t.end(), int64_t(0)); };
+    auto busiest = [&](int64_t tile, const std::vector<int64_t> &t) {
+        int64_t tiles = 0;
+        for (int64_t n : t) tiles += (n + tile - 1) / tile;
+        return (double)((tiles + sms - 1) / sms);
+    };
+    if (std::max(total(trials[0]), total(trials[1])) < 256 * sms) return 64;
+    int64_t best = 256, slots = 0, longest = 0;
+    double least = 1e300;
+    for (size_t s = 0; s < trials[0].size(); ++s) {
+        const int64_t k = (trials[0][s] + 63) / 64 + (trials[1][s] + 63) / 64;
+        slots += k;
+        longest = std::max(longest, k);
+    }
+    if (longest <= 2048) {
+        least = sums_record ? (double)slots * (3.75e-3 / (mixed ? 2.8 : 17.5)) : 0.0;
+        for (const auto &t : trials)
+            if (total(t) > 0) least += mixed ? 2.5 + 0.31 * busiest(64, t) : 0.38 + 0.265 * busiest(64, t);
+        best = 64;
+    }
+    for (int r = 1; r <= 10; ++r) {
+        double cost = 0.0;
+        for (const auto &t : trials) {
+            const double k = busiest(256 * r, t), over = std::fmod(k, 4.0);
+            cost += mixed ? (r + 0.8) * (k - over + over * (over == 1.0 ? 2.0 : over == 2.0 ? 1.25 : 1.12))
+                          : (r + 0.2) * k * (k == 1.0 ? 1.13 : 1.0);
+        }
+        if (cost < least) {
+            least = cost;
+            best = 256 * r;
+        }
+    }
+    return best;
+}
+
+}  // namespace ss

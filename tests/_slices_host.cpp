@@ -1,4 +1,6 @@
-// The host code that packs long rows into slices, as plain C functions for tests/test_slices_host.py.
+// Host code of the library that needs no GPU, as plain C functions for tests/test_slices_host.py and
+// tests/test_shape_host.py.
+#include "ss_shape.h"
 #include "ss_slices.h"
 
 #include <new>
@@ -52,5 +54,10 @@ int slices_dictionary(const float *J, int64_t nnz, float *dict, int *zero, uint8
     std::memcpy(dict, d.data(), d.size() * sizeof(float));
     if (bid) std::memcpy(bid, b.data(), b.size());
     return (int)d.size();
+}
+
+int64_t shape_mc_tile(int mixed, int sms, int sums_record, int nsys, const int64_t *class0, const int64_t *class1) {
+    const std::vector<int64_t> t[2] = {std::vector<int64_t>(class0, class0 + nsys), std::vector<int64_t>(class1, class1 + nsys)};
+    return mc_tile(mixed != 0, sms, sums_record != 0, t);
 }
 }

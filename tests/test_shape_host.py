@@ -1,0 +1,60 @@
+"""Launch shapes picked from sizes, on the host: tiles are counted within the systems of a batch, so that
+the busiest SM has little more than its share."""
+import ctypes
+import os
+import subprocess
+
+import numpy as np
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+SMS = 152
+
+
+@pytest.fixture(scope="module")
+def host(tmp_path_factory):
+    so = str(tmp_path_factory.mktemp("shape") / "shape.so")
+    subprocess.run(["g++", "-std=c++17", "-O2", "-fPIC", "-shared", "-I",
+                    os.path.join(ROOT, "paper_1310_6143_gb300", "csrc"),
+                    os.path.join(ROOT, "tests", "_slices_host.cpp"), "-o", so], check=True)
+    lib = ctypes.CDLL(so)
+    lib.shape_mc_tile.restype = ctypes.c_int64
+    return lib
+
+
+def _mc_tile(lib, mixed, sizes):
+    c = [np.array([(n + 1 - k) // 2 for n in sizes], np.int64) for k in (0, 1)]
+    return lib.shape_mc_tile(int(mixed), SMS, int(len(sizes) <= 2), len(sizes),
+                             *(a.ctypes.data_as(ctypes.c_void_p) for a in c)), c[0]
+
+
+def _share(tile, trials):
+    """Trials of the busiest SM's tiles, against an even share of the class."""
+    tiles = np.sum(-(-trials // tile))
+    return -(-tiles // SMS) * tile / (trials.sum() / SMS)
+
+
+BATCHES = [[20 ** 3] * 40, [30 ** 3] * 40, [40 ** 3] * 9, [40 ** 3] * 8, [12 ** 3] * 100, [8 ** 3] * 400, [80 ** 3], [100 ** 3],
+           [512 * 512 * 16], [64 ** 3], [48 ** 3, 48 ** 3, 2000]]
+
+
+@pytest.mark.parametrize("mixed", [True, False])
+@pytest.mark.parametrize("sizes", BATCHES, ids=lambda s: f"{len(s)}x{s[0]}")
+def test_monte_carlo_tiles_of_batches(host, sizes, mixed):
+    tile, trials = _mc_tile(host, mixed, sizes)
+    assert tile == 64 or (tile % 256 == 0 and 256 <= tile <= 2560)
+    assert _share(tile, trials) < 1.3
+
+
+@pytest.mark.parametrize("mixed", [True, False])
+def test_monte_carlo_tiles_of_drawn_batches(host, mixed):
+    rng = np.random.default_rng(7)
+    for _ in range(300):
+        sizes = rng.integers(2000, 200_000, rng.integers(1, 60)).tolist()
+        tile, trials = _mc_tile(host, mixed, sizes)
+        if trials.sum() < 256 * SMS:
+            assert tile == 64
+        else:
+            # a ragged tile per system and a last round per SM in tiles of 256, and 0.3 for the
+            # reductions that longer tiles save
+            assert _share(tile, trials) < 1.3 + 256 * (SMS + len(sizes)) / trials.sum()
