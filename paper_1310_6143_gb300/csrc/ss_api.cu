@@ -701,6 +701,11 @@ int corrector_grid(const ss_system *h) {
     return (int)std::max<int64_t>(1, std::min<int64_t>(h->ntiles, g));
 }
 
+// The blocks that sum the record, on top of a launch of `grid` others over the tiles.
+int record_blocks(const ss_system *h, int grid) {
+    return ss::record_blocks(h->precision == SS_FP32_MIXED, h->nsys, h->nfin, grid, h->tile / h->block, h->sm_count);
+}
+
 // The split FP32-mixed step (a Gaussian pass before the Heun passes) is used by the graph and
 // plain-launch modes of FP32-mixed handles that sum a thread per exchange row.
 bool split_step(const ss_system *h) {
@@ -775,7 +780,7 @@ cudaError_t enqueue_packed_step(const ss_system *h, const KArgs<R> &a, int gp, i
         r.x4 = reinterpret_cast<R *>(a.p4);
         e = launch_rows_field<R>(r, nullptr, nullptr, nullptr, gr, h->stream);
     }
-    if (e == cudaSuccess) e = launch_corrector4<R>(a, h->block, gc, h->nfin, h->stream);
+    if (e == cudaSuccess) e = launch_corrector4<R>(a, h->block, gc, record_blocks(h, gc), h->stream);
     return e;
 }
 
@@ -816,7 +821,7 @@ cudaError_t enqueue_steps_kernels(ss_system *h, int64_t n, bool packed) {
             for (int64_t k = 0; k < n && e == cudaSuccess; ++k) {
                 e = launch_gauss<R>(a, h->block, gg, h->stream, 0);
                 if (e == cudaSuccess) e = launch_predictor_split<R>(a, h->block, gp, h->stream);
-                if (e == cudaSuccess) e = launch_corrector_split<R>(a, h->block, gc, h->nfin, h->stream);
+                if (e == cudaSuccess) e = launch_corrector_split<R>(a, h->block, gc, record_blocks(h, gc), h->stream);
             }
             return e;
         }
@@ -839,7 +844,7 @@ cudaError_t enqueue_steps_kernels(ss_system *h, int64_t n, bool packed) {
             }
             if (e == cudaSuccess && k >= 1) e = cudaStreamWaitEvent(h->stream, h->ev_gauss, 0);
             if (e == cudaSuccess) e = launch_predictor_split<R>(a, h->block, gp, h->stream);
-            if (e == cudaSuccess) e = launch_corrector_split<R>(a, h->block, gc, h->nfin, h->stream);
+            if (e == cudaSuccess) e = launch_corrector_split<R>(a, h->block, gc, record_blocks(h, gc), h->stream);
             if (e == cudaSuccess) e = cudaEventRecord(h->ev_corr, h->stream);
         }
         // join the side stream (needed when it ran nothing after the fork)
@@ -853,7 +858,7 @@ cudaError_t enqueue_steps_kernels(ss_system *h, int64_t n, bool packed) {
         if (e == cudaSuccess) e = launch_predictor<R>(a, h->block, gp, h->stream);
         if (e != cudaSuccess) return e;
         if (h->rows) e = launch_rows_field<R>(a, a.px, a.py, a.pz, gr, h->stream);
-        if (e == cudaSuccess) e = launch_corrector<R>(a, h->block, gc, h->nfin, h->stream);
+        if (e == cudaSuccess) e = launch_corrector<R>(a, h->block, gc, record_blocks(h, gc), h->stream);
         if (e != cudaSuccess) return e;
     }
     return cudaSuccess;
@@ -1710,9 +1715,9 @@ ss_status time_kernels_impl(ss_system *h, int32_t nsteps, double out_ms[4]) {
     };
     auto corrector = [&]() -> cudaError_t {
         if constexpr (sizeof(R) == 4) {
-            if (packed) return launch_corrector4<R>(a, h->block, gc, h->nfin, h->stream);
+            if (packed) return launch_corrector4<R>(a, h->block, gc, record_blocks(h, gc), h->stream);
         }
-        return launch_corrector<R>(a, h->block, gc, h->nfin, h->stream);
+        return launch_corrector<R>(a, h->block, gc, record_blocks(h, gc), h->stream);
     };
     if (packed) SS_CUDA(h, packed_state(h, true));
     SS_CUDA(h, cudaEventRecord(ev[0], h->stream));
@@ -1728,7 +1733,7 @@ ss_status time_kernels_impl(ss_system *h, int32_t nsteps, double out_ms[4]) {
         SS_CUDA(h, cudaEventRecord(ev[3 * k + 2], h->stream));
         if (h->rows) SS_CUDA(h, rows(a.px, a.py, a.pz, a.p4));
         if (split)
-            SS_CUDA(h, launch_corrector_split<R>(a, h->block, gc, h->nfin, h->stream));
+            SS_CUDA(h, launch_corrector_split<R>(a, h->block, gc, record_blocks(h, gc), h->stream));
         else
             SS_CUDA(h, corrector());
         SS_CUDA(h, cudaEventRecord(ev[3 * k + 3], h->stream));
@@ -2060,7 +2065,7 @@ AltGrids alt_grids(const ss_system *h, int which) {
     g.len = (h->tile + g.sub - 1) / g.sub;
     g.first = (int)std::max<int64_t>(1, std::min<int64_t>(h->ntiles * g.sub, wave));
     g.second = one_wave(h, grid, alt_pass_blocks_per_sm<R>(which, mode));
-    g.nfin = h->nfin;
+    g.nfin = ss::record_blocks(sizeof(R) == 4, h->nsys, h->nfin, g.second, h->n / (256 * (int64_t)g.second), h->sm_count);
     g.rows = h->rows ? rows_grid(h) : 0;
     return g;
 }

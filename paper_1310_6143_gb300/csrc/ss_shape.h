@@ -62,4 +62,17 @@ inline int64_t mc_tile(bool mixed, int sm_count, bool sums_record, const std::ve
     return best;
 }
 
+// The blocks that sum the record of nsys systems on top of `grid` blocks with the launch's own work
+// of `rounds` spins a thread: at most `most`, and no more than fill the last round of blocks on the
+// SMs.  Blocks are handed out to the SMs in an order that is no plain round: with 40 of them on top
+// of 440 corrector blocks (40 x sc 30^3 in FP64, three to an SM) ten SMs got four of the 440, 212 us
+// instead of 160; with the 16 that fill the third round no SM does.  One block sums a system in
+// about the time an SM takes for a spin a thread (FP64: a quarter of it), so it is given at most as
+// many as that allows, or eight; where the round has less room, `most` are taken.
+inline int record_blocks(bool mixed, int64_t nsys, int most, int64_t grid, int64_t rounds, int sm_count) {
+    const int64_t sms = std::max(sm_count, 1), room = (sms - grid % sms) % sms;
+    const int64_t each = std::max<int64_t>(8, (mixed ? 1 : 4) * rounds * ((grid + sms - 1) / sms));
+    return room >= most || each * room < nsys ? most : (int)room;
+}
+
 }  // namespace ss

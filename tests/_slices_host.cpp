@@ -60,4 +60,8 @@ int64_t shape_mc_tile(int mixed, int sms, int sums_record, int nsys, const int64
     const std::vector<int64_t> t[2] = {std::vector<int64_t>(class0, class0 + nsys), std::vector<int64_t>(class1, class1 + nsys)};
     return mc_tile(mixed != 0, sms, sums_record != 0, t);
 }
+
+int shape_record_blocks(int mixed, int64_t nsys, int most, int64_t grid, int64_t rounds, int sms) {
+    return record_blocks(mixed != 0, nsys, most, grid, rounds, sms);
+}
 }

@@ -58,3 +58,21 @@ def test_monte_carlo_tiles_of_drawn_batches(host, mixed):
             # a ragged tile per system and a last round per SM in tiles of 256, and 0.3 for the
             # reductions that longer tiles save
             assert _share(tile, trials) < 1.3 + 256 * (SMS + len(sizes)) / trials.sum()
+
+
+@pytest.mark.parametrize("mixed", [True, False])
+def test_record_blocks_stay_in_the_last_round(host, mixed):
+    def blocks(nsys, grid, rounds):
+        return host.shape_record_blocks(int(mixed), ctypes.c_int64(nsys), min(nsys, 64), ctypes.c_int64(grid),
+                                        ctypes.c_int64(rounds), SMS)
+
+    for nsys in (1, 2, 5, 40, 64, 300, 1200):
+        for grid in list(range(1, 460)) + [608, 1216]:
+            for rounds in (1, 9):
+                k, most, room = blocks(nsys, grid, rounds), min(nsys, 64), -grid % SMS
+                if room < most and nsys <= room * max(8, (1 if mixed else 4) * rounds * -(-grid // SMS)):
+                    assert k == room  # the launch takes the rounds that its own blocks take
+                else:
+                    assert k == most  # room for all, or for too few
+    assert blocks(40, 440, 10) == 16 and blocks(60, 299, 9) == 5 and blocks(60, 275, 10) == 29
+    assert blocks(100, 300, 11) == (64 if mixed else 4)
