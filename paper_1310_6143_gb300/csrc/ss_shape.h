@@ -9,29 +9,42 @@
 
 namespace ss {
 
+// Tiles on the SM with most of them, when at most `resident` blocks per SM take the tiles in turn, block
+// b those at b, b + blocks, ...  Where the tiles are no multiple of the blocks, the low blocks have
+// one more.  The SMs do not get their blocks in plain rounds: four of the 152 are handed out a third
+// faster (measured with kernels that note their SM), so of a grid of several blocks per SM the
+// first 117, not 152, lie on distinct SMs, and 0.77 of the SMs take up a round of the rest.
+inline int64_t busiest_sm(int64_t tiles, int sm_count, int resident) {
+    const int64_t sms = std::max(sm_count, 1), blocks = resident * sms;
+    if (tiles < blocks) return (tiles + sms - 1) / sms;
+    const int64_t rest = tiles % blocks, most = (int64_t)std::ceil((double)rest / (0.77 * (double)sms));
+    return resident * (tiles / blocks) + std::min<int64_t>(resident, most);
+}
+
 // Trials per tile of the colour passes that sum the record (at most two classes): 64, in blocks of as
 // many threads, or r rounds of 256-thread blocks, r to 10 -- whichever a model of the pass, fitted to
-// 46 lattices and batches on GB300, finds cheapest.  A tile lies within one system, so the tiles are
+// 59 lattices and batches on GB300, finds cheapest.  A tile lies within one system, so the tiles are
 // counted system by system: a rule that took the class as one run gave 40 systems of 20^3 four tiles
 // of 1,280 and 160 trials each, two on the busiest SM (FP64 202 us per step; now 106), 9 of 40^3
 // FP32-mixed 75 us (now 51).  The model, in rounds of a 256-thread block at full residency
 // (2.8 us FP32-mixed, 17.5 us FP64), of the k tiles on the busiest SM:
-//  - FP32-mixed, r rounds: four blocks are resident on an SM.  Each group of four tiles takes r + 0.8
-//    (0.8: the record's reduction); one, two or three left over wait for latency, and take 2, 1.25 and
-//    1.12 each of what a tile of a full group takes.
-//  - FP64, r rounds: (r + 0.2) k, an eighth more for a lone tile's eight warps.
-//  - 64 trials, whose blocks read the transform's tables where they lie: 2.5 + 0.31 k FP32-mixed,
-//    0.38 + 0.265 k FP64; and, where the pass sums the record itself, 3.75 ns a slot.  Always
-//    for classes of fewer than 256 trials per SM; not for a system of more than 2,048 slots, which one
-//    block sums.
-// Its choice is within 4 % of the fastest on all 46, 0.3 % on average.
+//  - FP32-mixed, r rounds: four blocks are resident on an SM.  Each group of four tiles takes r + 0.9
+//    (0.9: the record's reduction); one, two or three left over wait for latency, and take 1.8, 1.25
+//    and 1.06 each of what a tile of a full group takes.
+//  - FP64, r rounds: two blocks are resident; (r + 0.2) k, an eighth more for a lone tile's eight warps.
+//  - 64 trials, whose blocks read the transform's tables where they lie and are handed out as SMs get
+//    free: 2.5 + 0.31 k FP32-mixed, 0.38 + 0.265 k FP64; and, where the pass sums the record itself,
+//    3.75 ns a slot.  Always for classes of fewer than 256 trials per SM; not for a system of more
+//    than 2,048 slots, which one block sums.
+// Its choice is within 4 % of the fastest on all 59 (FP64 1.4 %), 0.3 % on average.  Counted in plain
+// rounds of SMs, sc 128^3 in FP64 got nine rounds: 656 us per step, seven 521.
 inline int64_t mc_tile(bool mixed, int sm_count, bool sums_record, const std::vector<int64_t> (&trials)[2]) {
     const int64_t sms = std::max(sm_count, 1);
     auto total = [](const std::vector<int64_t> &t) { return std::accumulate(t.begin(), t.end(), int64_t(0)); };
-    auto busiest = [&](int64_t tile, const std::vector<int64_t> &t) {
-        int64_t tiles = 0;
-        for (int64_t n : t) tiles += (n + tile - 1) / tile;
-        return (double)((tiles + sms - 1) / sms);
+    auto tiles = [](int64_t tile, const std::vector<int64_t> &t) {
+        int64_t k = 0;
+        for (int64_t n : t) k += (n + tile - 1) / tile;
+        return k;
     };
     if (std::max(total(trials[0]), total(trials[1])) < 256 * sms) return 64;
     int64_t best = 256, slots = 0, longest = 0;
@@ -44,14 +57,17 @@ inline int64_t mc_tile(bool mixed, int sm_count, bool sums_record, const std::ve
     if (longest <= 2048) {
         least = sums_record ? (double)slots * (3.75e-3 / (mixed ? 2.8 : 17.5)) : 0.0;
         for (const auto &t : trials)
-            if (total(t) > 0) least += mixed ? 2.5 + 0.31 * busiest(64, t) : 0.38 + 0.265 * busiest(64, t);
+            if (total(t) > 0) {
+                const double k = (double)((tiles(64, t) + sms - 1) / sms);
+                least += mixed ? 2.5 + 0.31 * k : 0.38 + 0.265 * k;
+            }
         best = 64;
     }
     for (int r = 1; r <= 10; ++r) {
         double cost = 0.0;
         for (const auto &t : trials) {
-            const double k = busiest(256 * r, t), over = std::fmod(k, 4.0);
-            cost += mixed ? (r + 0.8) * (k - over + over * (over == 1.0 ? 2.0 : over == 2.0 ? 1.25 : 1.12))
+            const double k = (double)busiest_sm(tiles(256 * r, t), sm_count, mixed ? 4 : 2), over = std::fmod(k, 4.0);
+            cost += mixed ? (r + 0.9) * (k - over + over * (over == 1.0 ? 1.8 : over == 2.0 ? 1.25 : 1.06))
                           : (r + 0.2) * k * (k == 1.0 ? 1.13 : 1.0);
         }
         if (cost < least) {

@@ -64,4 +64,6 @@ int64_t shape_mc_tile(int mixed, int sms, int sums_record, int nsys, const int64
 int shape_record_blocks(int mixed, int64_t nsys, int most, int64_t grid, int64_t rounds, int sms) {
     return record_blocks(mixed != 0, nsys, most, grid, rounds, sms);
 }
+
+int64_t shape_busiest_sm(int64_t tiles, int sms, int resident) { return busiest_sm(tiles, sms, resident); }
 }

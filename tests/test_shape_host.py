@@ -18,7 +18,7 @@ def host(tmp_path_factory):
                     os.path.join(ROOT, "paper_1310_6143_gb300", "csrc"),
                     os.path.join(ROOT, "tests", "_slices_host.cpp"), "-o", so], check=True)
     lib = ctypes.CDLL(so)
-    lib.shape_mc_tile.restype = ctypes.c_int64
+    lib.shape_mc_tile.restype = lib.shape_busiest_sm.restype = ctypes.c_int64
     return lib
 
 
@@ -58,6 +58,26 @@ def test_monte_carlo_tiles_of_drawn_batches(host, mixed):
             # a ragged tile per system and a last round per SM in tiles of 256, and 0.3 for the
             # reductions that longer tiles save
             assert _share(tile, trials) < 1.3 + 256 * (SMS + len(sizes)) / trials.sum()
+
+
+@pytest.mark.parametrize("sizes,worst", [([128 ** 3], 2304), ([120 ** 3], 2048)])
+def test_monte_carlo_tiles_that_leave_half_a_wave_over(host, sizes, worst):
+    # 456 tiles of 2,304 and 422 of 2,048 are three and 2.8 for each of 152 SMs, but four on some
+    # of them: two blocks are resident, and of the 152 or 118 that take a second tile some share an SM
+    tile, _ = _mc_tile(host, False, sizes)
+    assert tile != worst
+
+
+def test_tiles_of_the_busiest_sm(host):
+    def busiest(tiles, resident):
+        return host.shape_busiest_sm(ctypes.c_int64(tiles), SMS, resident)
+
+    for resident in (1, 2, 3, 4):
+        for tiles in range(1, 5000, 7):
+            k, mean = busiest(tiles, resident), tiles / SMS
+            assert mean <= k < mean + 1 + resident
+            assert k == -(-tiles // SMS) or tiles > resident * SMS
+    assert [busiest(t, 2) for t in (152, 303, 304, 304 + 117, 304 + 118, 456, 608)] == [1, 2, 2, 3, 4, 4, 4]
 
 
 @pytest.mark.parametrize("mixed", [True, False])
