@@ -1461,38 +1461,12 @@ ss_status set_rows(ss_system *h, int32_t mode) {
 // 512-thread blocks and for more registers in smaller ones (heun_blocks); rows of at most six
 // bonds are faster in the former from about two million spins on (film of 1.05 M: 47.8 us per
 // step with 256 threads, 49.3 with 512; 256 grains of 5.2 M together: 256 and 248), everything
-// else in the latter.  FP64: 512 threads from four million spins on.
-// Spins per thread, up to 12: the count that leaves the busiest SM the least to do, its tiles times
-// the spins per thread (and about 0.3 spins' time for each tile's reduction, 0.2 in FP64).  The
-// passes also need warps to hide their latencies: FP32-mixed, 16 a SM cost about 4 %, eight 30 %;
-// FP64, eight 15 %.  fcc 64^3 in FP32-mixed form: 2 spins per thread leave the busiest SM 14
-// tiles for 13.5 on average, 9 three for exactly three (66.2 -> 59.7 us per step).  From 24 tiles
-// of eight spins per thread a SM on there is little to round off, and eight are as fast as any.
+// else in the latter.  FP64: 512 threads from four million spins on.  Spins per thread: heun_slots.
 void default_shape(ss_system *h) {
     const bool mixed = h->precision == SS_FP32_MIXED;
     const bool wide = h->n >= (int64_t(1) << (mixed ? 21 : 22)) && (!mixed || h->max_row <= kShortRow);
     h->block = wide ? 512 : 256;
-    const int64_t sms = std::max(h->sm_count, 1);
-    int best = 8;
-    double least = 1e300;
-    for (int slots = 1; slots <= 12; ++slots) {
-        const int64_t tile = (int64_t)slots * h->block;
-        int64_t tiles = 0;
-        for (int64_t n : h->sys_n) tiles += (n + tile - 1) / tile;
-        const int64_t per_sm = (tiles + sms - 1) / sms;
-        double cost = (double)per_sm * (slots + (mixed ? 0.3 : 0.2));
-        const double warps = (double)per_sm * h->block / 32.0;
-        cost *= mixed ? 1.0 + 0.3 * std::pow(std::max(0.0, 24.0 - warps) / 16.0, 3.0) : (warps < 16.0 ? 1.15 : 1.0);
-        if (cost < least) {
-            least = cost;
-            best = slots;
-        }
-        if (slots == 8 && tiles >= 24 * sms) {
-            best = 8;
-            break;
-        }
-    }
-    h->tile = best * h->block;
+    h->tile = h->block * heun_slots(mixed, h->block, h->sm_count, h->sys_n);
     h->ahead_q = 5;
 }
 

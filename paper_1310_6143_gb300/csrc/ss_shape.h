@@ -78,6 +78,34 @@ inline int64_t mc_tile(bool mixed, int sm_count, bool sums_record, const std::ve
     return best;
 }
 
+// Spins per thread of the Heun passes' tiles, up to 12: the count that leaves the busiest SM the least
+// to do, its tiles times the spins per thread (and 0.5 spins' time for each tile's reduction, 0.2 in
+// FP64).  An SM holds two FP32-mixed blocks of 512 threads or three of 256, one FP64 block.  The
+// passes also need warps to hide their latencies: FP32-mixed, 16 a SM cost about 4 %, eight 30 %;
+// FP64, eight 15 %.  Over 41 lattices and batches and 1024 x 1024 films of 8 to 20 layers the FP32-mixed
+// choice is within 2.3 % of the fastest, 0.3 % on average.  Counted in plain rounds of SMs, and with eight
+// taken from 24 tiles a SM on, it was up to 8.7 % off: the film of 8 layers took 12 spins a thread,
+// 315 us per step (9: 290), that of 16 eight, 585 us (9: 570).  fcc 64^3: 2 spins per thread
+// 66.2 us, 9 59.7.
+inline int heun_slots(bool mixed, int block, int sm_count, const std::vector<int64_t> &sizes) {
+    const int resident = !mixed ? 1 : block >= 512 ? 2 : 3;
+    int best = 1;
+    double least = 1e300;
+    for (int slots = 1; slots <= 12; ++slots) {
+        const int64_t tile = (int64_t)slots * block;
+        int64_t tiles = 0;
+        for (int64_t n : sizes) tiles += (n + tile - 1) / tile;
+        const double k = (double)busiest_sm(tiles, sm_count, resident), warps = k * block / 32.0;
+        double cost = k * (slots + (mixed ? 0.5 : 0.2));
+        cost *= mixed ? 1.0 + 0.3 * std::pow(std::max(0.0, 24.0 - warps) / 16.0, 3.0) : (warps < 16.0 ? 1.15 : 1.0);
+        if (cost < least) {
+            least = cost;
+            best = slots;
+        }
+    }
+    return best;
+}
+
 // The blocks that sum the record of nsys systems on top of `grid` blocks with the launch's own work
 // of `rounds` spins a thread: at most `most`, and no more than fill the last round of blocks on the
 // SMs.  Blocks are handed out to the SMs in an order that is no plain round: with 40 of them on top

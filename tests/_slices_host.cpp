@@ -66,4 +66,8 @@ int shape_record_blocks(int mixed, int64_t nsys, int most, int64_t grid, int64_t
 }
 
 int64_t shape_busiest_sm(int64_t tiles, int sms, int resident) { return busiest_sm(tiles, sms, resident); }
+
+int shape_heun_slots(int mixed, int block, int sms, int nsys, const int64_t *sizes) {
+    return heun_slots(mixed != 0, block, sms, std::vector<int64_t>(sizes, sizes + nsys));
+}
 }

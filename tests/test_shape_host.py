@@ -96,3 +96,16 @@ def test_record_blocks_stay_in_the_last_round(host, mixed):
                     assert k == most  # room for all, or for too few
     assert blocks(40, 440, 10) == 16 and blocks(60, 299, 9) == 5 and blocks(60, 275, 10) == 29
     assert blocks(100, 300, 11) == (64 if mixed else 4)
+
+
+# us per step of FP32-mixed runs of 1024 x 1024 films by layers and spins per thread (512-thread blocks, GB300)
+FILMS = {8: {6: 298, 7: 301, 8: 299, 9: 290, 10: 314, 11: 294, 12: 315}, 10: {6: 371, 7: 375, 8: 384, 9: 376, 10: 365, 11: 364, 12: 380},
+         13: {6: 485, 7: 486, 8: 472, 9: 473, 10: 475, 11: 463, 12: 460}, 14: {6: 518, 7: 513, 8: 511, 9: 512, 10: 523, 11: 516, 12: 504},
+         15: {6: 545, 7: 559, 8: 553, 9: 536, 10: 529, 11: 535, 12: 559}, 16: {6: 585, 7: 595, 8: 585, 9: 570, 10: 576, 11: 573, 12: 571}}
+
+
+@pytest.mark.parametrize("layers", sorted(FILMS))
+def test_spins_per_thread_of_large_films(host, layers):
+    n = np.array([1024 * 1024 * layers], np.int64)
+    slots = host.shape_heun_slots(1, 512, SMS, 1, n.ctypes.data_as(ctypes.c_void_p))
+    assert FILMS[layers][slots] <= 1.025 * min(FILMS[layers].values())
