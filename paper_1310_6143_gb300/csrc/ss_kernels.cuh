@@ -1559,6 +1559,12 @@ constexpr int kAltBlock = 256;
 // registers runs 82 us on the film, 68-73 with 40-48.
 constexpr int kAltFirstBlocks = 3;
 constexpr int kAltSecondBlocks = 5;
+// FP64 second passes: the compiler's own registers (64 to 128, two to four blocks), but three blocks with tensor
+// bonds or cubic anisotropy, whose forms would take 150 registers and leave one (fcc 30^3 with
+// Dzyaloshinskii-Moriya bonds, midpoint step: 236 us with one, 225 with three; fcc 40^3 495 and 476).
+// In the others three cost the core-shell sphere 3 % and sc 100^3 2 %.
+template <typename R, int Mode>
+constexpr int kAltSecond = sizeof(R) == 4 ? kAltSecondBlocks : Mode == kGeneral ? 3 : 1;
 
 // First pass of the alternative integrators: the step's thermal field (counters as the Heun
 // step), the part of the second pass's field that is fixed over the step,
@@ -1580,7 +1586,11 @@ __device__ __forceinline__ void alt_first_pass(const KArgs<R> &a, const StepTabT
                                                int len) {
     constexpr int BM = base_mode(Mode);
     const uint64_t step = *a.step;
-    for (int64_t u = blockIdx.x; u < a.ntiles * sub; u += gridDim.x) {
+    // FP64: the units left over when they are no multiple of the blocks go to the last blocks.  Of the
+    // first, some share an SM (see busiest_sm), which then has two units more than most, and this pass
+    // is bound by the FP64 pipe: fcc 30^3 95 -> 86 us a semi-implicit step, sc 48^3 85 -> 77, fcc 30^3 with
+    // tensor bonds 143 -> 127.  FP32-mixed passes gain nothing from it.
+    for (int64_t u = sizeof(R) == 8 ? gridDim.x - 1 - blockIdx.x : blockIdx.x; u < a.ntiles * sub; u += gridDim.x) {
         const int64_t t = u / sub;
         const int k0 = (int)(u - t * sub) * len;
         const TileDesc td = a.tiles[t];
@@ -1693,7 +1703,7 @@ __global__ void __launch_bounds__(kAltBlock, sizeof(R) == 4 ? kAltFirstBlocks : 
 // writes Y over S (Last: and flags non-finite spins, and advances the step counter).  Blocks
 // [0, nfin) sum the step's record instead (the first iteration; nfin = 0 otherwise).
 template <typename R, int Mode, bool Last>
-__global__ void __launch_bounds__(kAltBlock, sizeof(R) == 4 ? kAltSecondBlocks : 1)
+__global__ void __launch_bounds__(kAltBlock, kAltSecond<R, Mode>)
     k_mid_iter(const KArgs<R> a, const R *xx, const R *xy, const R *xz, R *yx, R *yy, R *yz, int nfin, int sub) {
     constexpr int BM = base_mode(Mode);
     if ((int)blockIdx.x < nfin) {
@@ -1730,7 +1740,7 @@ __global__ void __launch_bounds__(kAltBlock, sizeof(R) == 4 ? kAltSecondBlocks :
 // on-site terms of Sb; the new spin overwrites S (a thread reads S only at its own spin).  Blocks
 // [0, nfin) sum the step's record; the last block advances the step counter.
 template <typename R, int Mode>
-__global__ void __launch_bounds__(kAltBlock, sizeof(R) == 4 ? kAltSecondBlocks : 1)
+__global__ void __launch_bounds__(kAltBlock, kAltSecond<R, Mode>)
     k_sib_corr(const KArgs<R> a, int nfin, int sub) {
     constexpr int BM = base_mode(Mode);
     if ((int)blockIdx.x < nfin) {
