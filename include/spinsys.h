@@ -209,9 +209,10 @@ ss_status set_temperature_schedule(ss_system *h, const double *T_per_step, int64
  * Each step records the moment and energy of the state at its start (Eq. spinhamiltonian)
  * into the per-step record ring.  SS_ERR_INVALID_ARG for n < 0; a non-finite spin raised
  * on the device is reported as SS_ERR_NONFINITE by the next synchronising call.
- * The first FP32-mixed run of four or more steps by kernels or graphs allocates 56 bytes per
- * spin to work in.  Without that memory the run gives the same results, slower; a later call
- * on the handle that needs the memory takes it back. */
+ * The first FP32-mixed run by kernels or graphs that is long enough to gain from it (4 to 32
+ * steps, by size; rows with row forms or packed slices) allocates 56 bytes per spin to work in.
+ * Without that memory the run gives the same results, slower; a later call on the handle that
+ * needs the memory takes it back. */
 ss_status llg_heun_step(ss_system *h, int64_t n);
 
 /* Advance every system by n >= 0 Monte Carlo steps (asynchronous; Section "Monte Carlo
@@ -395,8 +396,8 @@ ss_status spin_system_set_gaussian_pass(ss_system *h, int32_t mode);
 ss_status spin_system_set_draw_ahead(ss_system *h, int32_t eighths);
 
 /* Time the candidate (exec, block, tile, draw-ahead, Gaussian pass) choices on this handle over `trial_steps`
- * steps each (FP32-mixed: at least four, the length from which runs take float4 spins; their packing
- * before and after a run is not timed), keep the fastest, and write it to *out_info.  The spins and the step
+ * steps each (FP32-mixed: at least the length from which runs take float4 spins, 4 to 32; their
+ * packing before and after a run is not timed), keep the fastest, and write it to *out_info.  The spins and the step
  * counter are restored afterwards, so the trajectory is unchanged.  With the environment
  * variable SPINSYS_AUTOTUNE_CACHE naming a file, a workload tuned before on the same device
  * (same precision, spins, bonds, systems, largest system, exchange-row mode, kernel variant and

@@ -723,23 +723,32 @@ int split_grid(const ss_system *h, int which) {
     return (int)std::max<int64_t>(1, std::min<int64_t>(h->ntiles, g));
 }
 
-// Runs of at least this many steps work on float4 spins: packing and unpacking the state moves
-// 84 bytes per spin (0.24 ms on the 1024 x 1024 x 16 film), and a step over float4 spins saves
-// about 0.07 ms there.
-constexpr int64_t kPackedMin = 4;
-
-// Whether a run of n steps in the graph or plain-launch mode works on float4 spins: FP32-mixed,
-// not a slab (its halo refresh reads S'), not the split step (the Gaussians come in arrays), and
-// with long rows only the packed-bond pass, which reads float4 spins itself.
-bool wants_packed(const ss_system *h, int64_t n) {
-    return h->precision == SS_FP32_MIXED && h->slab_own < 0 && n >= kPackedMin && !split_step(h) && (!h->rows || h->sell);
+// The least number of steps for which a run in the graph or plain-launch mode works on float4 spins
+// (FP32-mixed; not a slab, whose halo refresh reads S'; not the split step, whose Gaussians come in
+// arrays).  Packing and unpacking the state takes two launches and moves 84 bytes per spin: 6 us on a
+// small system, 0.21 ms on the 1024 x 1024 x 16 film, where a step saves 80 of 660 us.  Measured
+// as runs of 4 to 64 steps against the same on the arrays:
+//  - long rows, whose packed-bond pass then needs no copy of the spins: every run gains (2,048 spins of
+//    140 bonds 12 % at four steps);
+//  - row forms, from 2^21 spins (film 512 x 512 x 16 11 %, sc 128^3 12 %): even at three steps; from 2^17
+//    (2 to 5 %): at five to eight; from 10,000 (between 2 % loss and 3 % gain): at 30; below (up to 6 %
+//    gain): at ten or so;
+//  - columns and CSR rows: never (core-shell spheres of 15 to 36 nm 1 to 7 % slower, a random graph of a
+//    million spins 16 %): their neighbours lie in no order, and a gather of 16 bytes a spin misses more.
+constexpr int64_t kPackedNever = INT64_MAX;
+int64_t packed_min(const ss_system *h) {
+    if (h->precision != SS_FP32_MIXED || h->slab_own >= 0 || split_step(h)) return kPackedNever;
+    if (h->rows) return h->sell ? 4 : kPackedNever;
+    if (!h->use_pat || h->npat == 0) return kPackedNever;
+    return h->n >= (int64_t(1) << 21) ? 4 : h->n >= (int64_t(1) << 17) ? 8 : h->n >= 10000 ? 32 : 12;
 }
+bool wants_packed(const ss_system *h, int64_t n) { return n >= packed_min(h); }
 bool packed_run(const ss_system *h, int64_t n) { return h->packed && wants_packed(h, n); }
 
 size_t packed_bytes(const ss_system *h) { return (size_t)packed_spins(h) * (3 * sizeof(float4) + sizeof(float2)); }
 
 // The float4 spins, allocated by the first run that takes them (handles that only do Monte Carlo,
-// alternative integrators, single steps or the cluster, persistent and system-block steps never hold
+// alternative integrators, short runs or the cluster, persistent and system-block steps never hold
 // their 56 bytes per spin; allocating them takes 0.2 ms).  Without the memory the steps work on the
 // arrays.  Allowed while a stream is captured: nothing is enqueued on it here.
 void ensure_packed(ss_system *h) {
@@ -1445,10 +1454,6 @@ ss_status set_rows(ss_system *h, int32_t mode) {
             SS_CUDA(h, cudaMemsetAsync(h->x4, 0, 128 * (size_t)h->nslice * rs, h->stream));
         }
     }
-    // the classes' padding in the float4 spins is gathered with J = 0 and has to be finite, whatever
-    // runs without row passes left there
-    if (on && !h->rows && h->packed && h->nslice > 0)
-        SS_CUDA(h, cudaMemsetAsync(h->packed, 0, packed_bytes(h), h->stream));
     h->rows_req = mode;
     if (on != h->rows) drop_graph(h);
     h->rows = on;
@@ -3110,7 +3115,8 @@ ss_status spin_system_autotune(ss_system *h, int32_t trial_steps, ss_info *out_i
     SS_CUDA(h, cudaEventCreate(&e1));
     // What longer runs launch: over float4 spins where they take them, whose packing and unpacking
     // (once a run, however long) would count only against the candidates that do it.
-    const int64_t trial = mixed ? std::max<int64_t>(trial_steps, kPackedMin) : trial_steps;
+    const int64_t least = packed_min(h) == kPackedNever ? 1 : packed_min(h);
+    const int64_t trial = std::max<int64_t>(trial_steps, least);
     auto timed_run = [&] {
         if (!h->demag_on) return advance_steps(h, trial, e0, e1);
         cudaEventRecord(e0, h->stream);
@@ -3128,7 +3134,7 @@ ss_status spin_system_autotune(ss_system *h, int32_t trial_steps, ss_info *out_i
         if (spin_system_set_gaussian_pass(h, c.gauss) != SS_OK) { h->bad = false; continue; }
         if (spin_system_set_launch(h, c.block, c.tile) != SS_OK) continue;
         if (spin_system_set_exec(h, (ss_exec)c.exec) != SS_OK) continue;
-        if (llg_heun_step(h, std::min<int64_t>(trial, 4)) != SS_OK) { h->bad = false; continue; }
+        if (llg_heun_step(h, std::min<int64_t>(trial, std::max<int64_t>(least, 4))) != SS_OK) { h->bad = false; continue; }
         // the shorter of two timed runs: one run of a few steps of a small system is noisy
         float ms = 1e30f;
         bool ok = true;

@@ -55,5 +55,5 @@ def test_trials_launch_what_runs_launch():
         s.set_launch(256, 256)
         now = s.info()["device_bytes"]
         s.set_exec("kernels")
-        s.step(8)
+        s.step(12)
         assert s.info()["device_bytes"] == now > held + 56 * s.n

@@ -38,20 +38,23 @@ def test_held_by_runs_only(env):
         s.mc_step(2)
         s.semi_implicit_step(5)
         s.midpoint_step(4)
-        s.step(3)
+        s.step(11)  # 8,160 spins with row forms: runs of 12 steps and more
         s.set_exec("system_blocks")
-        s.step(5)
+        s.step(12)
         s.set_exec("persistent")
-        s.step(5)
-        assert s.info()["device_bytes"] == held
+        s.step(12)
         s.set_exec("kernels")
-        s.step(4)
+        s.set_row_patterns(False)
+        s.step(12)
+        s.set_row_patterns(True)
+        assert s.info()["device_bytes"] == held
+        s.step(12)
         assert s.info()["device_bytes"] == held + 56 * s.n
         s.step(8)
         assert s.info()["device_bytes"] == held + 56 * s.n
 
 
-@pytest.mark.parametrize("mode,runs", [("kernels", [5, 6]), ("graph", [2, 70]), ("auto", [3, 130])])
+@pytest.mark.parametrize("mode,runs", [("kernels", [14, 15]), ("graph", [2, 70]), ("auto", [3, 130])])
 def test_runs_without_the_memory(env, mode, runs):
     lib, SS = env
     out = []
@@ -111,8 +114,8 @@ def test_first_run_inside_a_callers_capture(env):
 
     lib, SS = env
     with SS(_film(), **KW) as s:
-        s.step(20)  # (loads the kernels, too)
-        ref = s.spins(), s.record(0, 20)
+        s.step(30)  # (loads the kernels, too)
+        ref = s.spins(), s.record(0, 30)
     stream = torch.cuda.Stream()
     with SS(_film(), **KW) as s:
         s.set_stream(stream)
@@ -120,13 +123,14 @@ def test_first_run_inside_a_callers_capture(env):
         torch.cuda.synchronize()
         graph = torch.cuda.CUDAGraph()
         with torch.cuda.graph(graph, stream=stream):
-            s.step(5)
+            s.step(15)
         with torch.cuda.stream(stream):
-            for _ in range(4):
+            for _ in range(2):
                 graph.replay()
         held = s.info()["device_bytes"]
+        assert held >= 56 * s.n
         np.testing.assert_array_equal(s.spins(), ref[0])
-        np.testing.assert_array_equal(s.record(0, 20), ref[1])
+        np.testing.assert_array_equal(s.record(0, 30), ref[1])
         # memory that runs out later: the caller's graph names the buffer, so it stays
         lib.ss_debug_limit_bytes(lib.ss_debug_live_bytes())
         from paper_1310_6143_gb300._binding import SpinSysError
@@ -136,3 +140,27 @@ def test_first_run_inside_a_callers_capture(env):
         lib.ss_debug_limit_bytes(-1)
         assert s.info()["device_bytes"] == held
         torch.cuda.synchronize()
+
+
+@pytest.mark.parametrize("lats", ["film", "batch", "tensor", "wide"])
+def test_longer_runs_equal_single_steps(env, lats):
+    # the lengths from which float4 spins are taken: 12 steps below 10,000 spins, 32 above
+    lib, SS = env
+    systems = {"film": lambda: L.film(13, 11, 17), "wide": lambda: L.film(41, 30, 9),
+               "batch": lambda: [L.simple_cubic(3, 3, 115), L.simple_cubic(11, 31, 3), L.dimer(), L.film(9, 8, 7)],
+               "tensor": lambda: L.with_dm(L.fcc(5, 4, 6, with_pos=True), D=1e-21)}[lats]()
+    steps = 34 if lats == "wide" else 14
+    ref = None
+    for block, slots, runs in ((256, 1, [1] * steps), (256, 1, [steps]), (256, 3, [1, steps - 1]), (512, 1, [steps - 2, 2]),
+                               (128, 5, [steps])):
+        with SS(systems, **KW) as s:
+            s.set_exec("kernels")
+            s.set_launch(block, block * slots)
+            held = s.info()["device_bytes"]
+            for k in runs:
+                s.step(k)
+            assert s.info()["device_bytes"] - held == (56 * s.n if len(runs) < steps else 0)
+            out = [s.spins()] + [v.cpu().numpy() for v in s.state_device(1)]
+        ref = ref or out
+        for x, y in zip(out, ref):
+            np.testing.assert_array_equal(x, y)
