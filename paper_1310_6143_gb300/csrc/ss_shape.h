@@ -23,20 +23,21 @@ inline int64_t busiest_sm(int64_t tiles, int sm_count, int resident) {
 
 // Trials per tile of the colour passes that sum the record (at most two classes): 64, in blocks of as
 // many threads, or r rounds of 256-thread blocks, r to 10 -- whichever a model of the pass, fitted to
-// 59 lattices and batches on GB300, finds cheapest.  A tile lies within one system, so the tiles are
+// 53 lattices and batches on GB300, finds cheapest.  A tile lies within one system, so the tiles are
 // counted system by system: a rule that took the class as one run gave 40 systems of 20^3 four tiles
 // of 1,280 and 160 trials each, two on the busiest SM (FP64 202 us per step; now 106), 9 of 40^3
 // FP32-mixed 75 us (now 51).  The model, in rounds of a 256-thread block at full residency
 // (2.8 us FP32-mixed, 17.5 us FP64), of the k tiles on the busiest SM:
-//  - FP32-mixed, r rounds: four blocks are resident on an SM.  Each group of four tiles takes r + 0.9
-//    (0.9: the record's reduction); one, two or three left over wait for latency, and take 1.8, 1.25
-//    and 1.06 each of what a tile of a full group takes.
+//  - FP32-mixed, r rounds: four blocks are resident on an SM.  Each whole round of four tiles takes
+//    4 (r + 0.85) (0.85: the record's reduction).  One to four left over, on the busiest SM, wait for
+//    latency: as the only tiles they take 2, 2.4, 3.25 and 3.85 of r + 0.85, behind whole rounds, which
+//    end unevenly, 2.35, 2.55, 3.8 and 5.2.
 //  - FP64, r rounds: two blocks are resident; (r + 0.2) k, an eighth more for a lone tile's eight warps.
 //  - 64 trials, whose blocks read the transform's tables where they lie and are handed out as SMs get
 //    free: 2.5 + 0.31 k FP32-mixed, 0.38 + 0.265 k FP64; and, where the pass sums the record itself,
 //    3.75 ns a slot.  Always for classes of fewer than 256 trials per SM; not for a system of more
-//    than 2,048 slots, which one block sums.
-// Its choice is within 4 % of the fastest on all 59 (FP64 1.4 %), 0.3 % on average.  Counted in plain
+//    than 2,048 slots, which one block sums, nor beyond the k for which they were ever fastest.
+// Its choice is within 4.1 % of the fastest on all 53 (FP64 1.5 %), 0.4 % on average (0.1 %).  Counted in plain
 // rounds of SMs, sc 128^3 in FP64 got nine rounds: 656 us per step, seven 521.
 inline int64_t mc_tile(bool mixed, int sm_count, bool sums_record, const std::vector<int64_t> (&trials)[2]) {
     const int64_t sms = std::max(sm_count, 1);
@@ -54,7 +55,8 @@ inline int64_t mc_tile(bool mixed, int sm_count, bool sums_record, const std::ve
         slots += k;
         longest = std::max(longest, k);
     }
-    if (longest <= 2048) {
+    const int64_t k64 = (std::max(tiles(64, trials[0]), tiles(64, trials[1])) + sms - 1) / sms;
+    if (longest <= 2048 && k64 <= (mixed ? 24 : 72)) {
         least = sums_record ? (double)slots * (3.75e-3 / (mixed ? 2.8 : 17.5)) : 0.0;
         for (const auto &t : trials)
             if (total(t) > 0) {
@@ -66,9 +68,14 @@ inline int64_t mc_tile(bool mixed, int sm_count, bool sums_record, const std::ve
     for (int r = 1; r <= 10; ++r) {
         double cost = 0.0;
         for (const auto &t : trials) {
-            const double k = (double)busiest_sm(tiles(256 * r, t), sm_count, mixed ? 4 : 2), over = std::fmod(k, 4.0);
-            cost += mixed ? (r + 0.9) * (k - over + over * (over == 1.0 ? 1.8 : over == 2.0 ? 1.25 : 1.06))
-                          : (r + 0.2) * k * (k == 1.0 ? 1.13 : 1.0);
+            const int64_t n = tiles(256 * r, t), k = busiest_sm(n, sm_count, mixed ? 4 : 2);
+            if (mixed) {
+                constexpr double only[5] = {0.0, 2.0, 2.4, 3.25, 3.85}, behind[5] = {0.0, 2.35, 2.55, 3.8, 5.2};
+                const int64_t whole = n / (4 * sms);
+                cost += (r + 0.85) * (4.0 * (double)whole + (whole ? behind : only)[k - 4 * whole]);
+            } else {
+                cost += (r + 0.2) * (double)k * (k == 1 ? 1.13 : 1.0);
+            }
         }
         if (cost < least) {
             least = cost;
