@@ -4,8 +4,8 @@ Default workload: the 1024 x 1024 x 16 simple-cubic thin film (16,777,216 spins,
 periodic, free z surfaces, J = 6.0e-21 J, mu_s = 1.5 muB, k_u = 1.0e-24 J || z,
 alpha = 0.02, dt = 1e-16 s) under the 100 fs Gaussian temperature pulse (1200 K peak on a
 300 K base, centred at 1 ps), FP32-mixed precision.  A step is one full Heun step of the
-whole film: thermal field, predictor, corrector, renormalisation and the FP64 moment and
-energy reductions.  The state (~0.8 GB of working arrays) is far larger than L2, so no
+whole film: thermal field, predictor, corrector, renormalisation and the moment and energy
+reductions (FP64; FP32-mixed sums each thread's terms of a tile in float pairs first).  The state (~0.8 GB of working arrays) is far larger than L2, so no
 flush is needed between steps.
 
 Also reported: the same film in plain FP64, and the 256-grain batched ensemble in one
@@ -56,15 +56,15 @@ def step_bytes_per_spin(real_bytes, nnz_per_spin):
     return 2 * pass_bytes_per_spin(real_bytes, nnz_per_spin)
 
 
-# Bytes the implemented layout of arrays moves per spin-step (FP32-mixed runs of several steps keep
-# S, S' and Q as float4 and move 16 more): S, S', the half step Q and the stored
-# thermal field (24 words), the Gaussians drawn ahead (written and read back for a fraction
+# Bytes the implemented layout moves per spin-step: S, S', the half step Q and the stored
+# thermal field (24 words of arrays; float4=True: runs over float4 spins, whose S and S' are read and
+# written as four words each, 28), the Gaussians drawn ahead (written and read back for a fraction
 # f of the spins), the neighbour rows once per pass -- one byte per spin with row patterns,
 # else the CSR columns and row offset (and J unless every bond has the same J_ij/mu_s,i) --
 # and the material index once per pass unless the handle has a single material.
-def layout_bytes_per_spin(real_bytes, nnz_per_spin, f_ahead, j_uniform, patterns=False, one_material=False):
+def layout_bytes_per_spin(real_bytes, nnz_per_spin, f_ahead, j_uniform, patterns=False, one_material=False, float4=False):
     rows = 2.0 if patterns else 2 * (nnz_per_spin * 4 + 4) + (0 if j_uniform else 2 * nnz_per_spin * real_bytes)
-    return 24 * real_bytes + 6 * real_bytes * f_ahead + rows + (0 if one_material else 8)
+    return (28 if float4 else 24) * real_bytes + 6 * real_bytes * f_ahead + rows + (0 if one_material else 8)
 
 
 # The FP64 form's step kernels run every operation on the FP64 pipe (2 instructions per cycle
@@ -76,8 +76,8 @@ FP64_FORM_PREDICTOR_FP64_PER_SPIN = 93.0
 # DRAM bytes per launch of the default film shape (block, tile, draw-ahead eighths), read from
 # one ncu capture of the FP32-mixed kernels (profiles/k_predictor_film1024x1024x16_fp32.md,
 # profiles/k_corrector_film1024x1024x16_fp32.md), not measured in this run.
-DEFAULT_FILM_SHAPE = (512, 4096, 5)
-KERNEL_DRAM_BYTES = {"k_predictor": 1.039e9, "k_corrector": 1.074e9}
+DEFAULT_FILM_SHAPE = (512, 6144, 5)
+KERNEL_DRAM_BYTES = {"k_predictor": 1.069e9, "k_corrector": 1.099e9}
 SMS = 152
 NO_AUTOTUNE = False
 EXEC_NAMES = {0: "auto", 1: "kernels", 2: "graph", 3: "persistent", 4: "system_blocks", 5: "cluster"}
@@ -706,7 +706,8 @@ def main():
     f_ahead = ((info32["draw_ahead"] * spt) // 8) / spt if args.precision == "fp32" else 0.0
     j_rows = lat.J / np.repeat(lat.mu_s, np.diff(lat.row_ptr))
     lay_b = layout_bytes_per_spin(rb, nnz_per, f_ahead, bool(np.all(j_rows == j_rows[0])),
-                                  patterns=info32.get("row_patterns", 0) > 0, one_material=info32["num_materials"] == 1)
+                                  patterns=info32.get("row_patterns", 0) > 0, one_material=info32["num_materials"] == 1,
+                                  float4=args.precision == "fp32" and args.steps >= 4 and info32.get("gaussian_pass", 0) == 0)
     default_shape = (info32["block"], info32["tile"], info32["draw_ahead"]) == DEFAULT_FILM_SHAPE
     sm_ghz = (clk32.get("sm_mhz") or float(peaks.get("sm_max_mhz", 2070.0))) / 1e3
     out = {
@@ -718,7 +719,7 @@ def main():
                                f"step {PULSE_PEAK_STEP}); timed steps {win32['first_step']}..."
                                f"{win32['first_step'] + win32['steps'] - 1} of the schedule, centred on the pulse "
                                f"(T {win32['T_min_K']:.0f}-{win32['T_max_K']:.0f} K), entered from the warm-up state",
-                   "precision": "fp32-mixed (FP64-exact thermal transform and FP64 reductions)"
+                   "precision": "fp32-mixed (FP64-exact thermal transform; record sums in float pairs per thread, FP64 beyond)"
                    if args.precision == "fp32" else "fp64",
                    "spins": lat.n, "nnz": lat.nnz, "timed_window": win32,
                    "exec": EXEC_NAMES[info32["exec"]] if info32["exec"] else "auto (captured graphs of step launches)",

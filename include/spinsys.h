@@ -71,8 +71,9 @@ typedef enum {
 
 typedef enum {
     SS_FP64 = 0,      /* every step in FP64                                          */
-    SS_FP32_MIXED = 1 /* FP32 storage, field and LLG arithmetic; FP64 Philox-to-Gaussian
-                         transform and FP64 moment/energy sums                        */
+    SS_FP32_MIXED = 1 /* FP32 storage, field and LLG arithmetic; the FP64 Philox-to-Gaussian
+                         transform's values; moment/energy terms summed in float pairs
+                         (2^-48) by each thread of a tile, in FP64 beyond               */
 } ss_precision;
 
 /* ss_params.flags */

@@ -1464,8 +1464,8 @@ ss_status set_rows(ss_system *h, int32_t mode) {
 
 // The default launch shape.  Block: the FP32-mixed kernels are compiled for more resident warps in
 // 512-thread blocks and for more registers in smaller ones (heun_blocks); rows of at most six
-// bonds are faster in the former from about two million spins on (film of 1.05 M: 47.8 us per
-// step with 256 threads, 49.3 with 512; 256 grains of 5.2 M together: 256 and 248), everything
+// bonds are faster in the former from about two million spins on (film of 1.05 M: 52.8 us per step of a
+// 32-step run with 256 threads, 52.2 with 512; 256 grains of 5.2 M together: 255 and 244), everything
 // else in the latter.  FP64: 512 threads from four million spins on.  Spins per thread: heun_slots.
 void default_shape(ss_system *h) {
     const bool mixed = h->precision == SS_FP32_MIXED;

@@ -14,7 +14,8 @@
 //     H'_i from S' with the same H_th,i; dS'_i = LLG(S'_i, H'_i)
 //     S_i <- normalise(Q_i + dt/2 dS'_i)   (= S_i + dt/2 (dS_i + dS'_i), then renormalised)
 //
-// Data layout: spins as structure-of-arrays (three arrays per vector); the neighbour list
+// Data layout: spins as structure-of-arrays (three arrays per vector; longer FP32-mixed runs keep them as
+// float4, see k_predictor); the neighbour list
 // in CSR (int32 offsets and columns, J in the working type); one material index per spin.
 // Work is split into tiles (contiguous spins of one system); each tile yields one FP64
 // partial of the reductions, summed per system in a fixed order, so the record is
@@ -956,17 +957,17 @@ static __global__ void __launch_bounds__(256) k_unpack_state(const KArgs<float> 
 // Resident blocks per SM the FP32-mixed Heun passes are compiled for: two of 512 threads (64
 // registers) or 24 warps in smaller blocks (80 registers).  Both passes wait for the gathers, so
 // resident warps and loads in flight per thread trade against each other: rows of six bonds are
-// faster at 64 registers (the 1024 x 1024 x 16 film 0.620 against 0.673 ms per step, 256 grains
-// 248 against 256 us), rows of twelve at 80 (fcc 64^3 59.7 against 65.1 us, the 20 nm core-shell
-// sphere 36 against 40 us).  default_shape picks the block.
+// faster at 64 registers (runs of 32 steps of the 1024 x 1024 x 16 film 570 against 666 us per step, of
+// 256 grains 244 against 255), the 20 nm core-shell sphere's rows at 80 (41.6 against 43.7 us), and
+// fcc 64^3 takes either (65.7 and 66.0 us).  default_shape picks the block.
 __host__ __device__ constexpr int heun_blocks(int bs) { return bs >= 512 ? 2 : 768 / bs; }
 
 // The Heun predictor.  V4 (FP32-mixed runs of several steps): the spins come as one float4 each.
 // Three arrays cost a gather three loads and three addresses, which is what the 64 or 80
 // registers then hold instead of neighbours in flight; a float4 costs one of each.  S' goes out
 // as a float4, and the half step and the thermal field, which only their own spin reads back, as
-// a float4 and a float2.  134 bytes of traffic per spin and step against 110, but the passes move
-// less than 40 % of what HBM gives: the film 0.692 -> 0.620 ms per step.
+// a float4 and a float2.  128 bytes of traffic per spin and step against 112, but the passes move
+// about half of what HBM gives: the 1024 x 1024 x 16 film 0.645 (single steps, on the arrays) -> 0.564 ms.
 //
 // FP64: one resident block per SM is enough for the FP64 pipe, and the minimum-blocks bound
 // lets the compiler keep the transform in registers (without it the FP64 form spills at 64).
@@ -1352,7 +1353,8 @@ __global__ void __launch_bounds__(BS, sizeof(R) == 8 || BS >= 512 ? 0 : heun_blo
 // slices with the same words -- on a lattice, all those in the same position along the short axis
 // and away from the others' ends -- share them, which then come from the L2 instead of HBM (fcc
 // 32^3 to 4a: 556 -> 44 MB of words).  One FP32 pass there: 286 -> about 140 us, still waiting for
-// the gathers' L1 misses.  U bonds in flight a warp: 2 1.65, 3 1.36, 4 1.22, 8 1.32, 16 1.53 ms per four steps
+// the gathers: half of their sectors miss the L1 (48 %, 1.16 GB from the L2), issue 30 %.  U bonds in
+// flight a warp: 2 1.65, 3 1.36, 4 1.22, 8 1.32, 16 1.53 ms per four steps
 // (more evict each other's lines); words loaded past the L1 1.71, two slices to a warp 2.0 ms.
 //
 template <typename R>

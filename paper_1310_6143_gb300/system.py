@@ -44,7 +44,7 @@ class SpinSystem:
     ``lattices`` is a SpinLattice or a sequence of them (a batch of independent systems).
     ``alpha``, ``dt``, ``T``, ``H``, ``seed``, ``sys_id`` and ``S0`` may be given per
     system as sequences.  ``precision`` is "fp64" or "fp32" (FP32 storage and field/LLG
-    arithmetic with FP64 thermal transform and FP64 reductions).
+    arithmetic with FP64 thermal transform; record sums in float pairs per thread, FP64 beyond).
     ``slab=(nslabs, index)`` makes the handle of one slab of a single lattice (the owned
     global range plus halo copies, advanced by ``heun_pass``; see ``paper_1310_6143_gb300.slab``).
     """
