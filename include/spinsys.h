@@ -210,10 +210,10 @@ ss_status set_temperature_schedule(ss_system *h, const double *T_per_step, int64
  * Each step records the moment and energy of the state at its start (Eq. spinhamiltonian)
  * into the per-step record ring.  SS_ERR_INVALID_ARG for n < 0; a non-finite spin raised
  * on the device is reported as SS_ERR_NONFINITE by the next synchronising call.
- * The first FP32-mixed run by kernels or graphs that is long enough to gain from it (4 to 32
- * steps, by size; rows with row forms or packed slices) allocates 56 bytes per spin to work in.
- * Without that memory the run gives the same results, slower; a later call on the handle that
- * needs the memory takes it back. */
+ * FP32-mixed runs by kernels or graphs that are long enough to gain from it (4 to 32 steps, by
+ * size; rows with row forms or packed slices) work in 56 bytes per spin, allocated by the first
+ * such run (with the handle up to 64 MiB).  Without that memory the run gives the same results,
+ * slower; a later call on the handle that needs the memory takes it back. */
 ss_status llg_heun_step(ss_system *h, int64_t n);
 
 /* Advance every system by n >= 0 Monte Carlo steps (asynchronous; Section "Monte Carlo

@@ -747,10 +747,13 @@ bool packed_run(const ss_system *h, int64_t n) { return h->packed && wants_packe
 
 size_t packed_bytes(const ss_system *h) { return (size_t)packed_spins(h) * (3 * sizeof(float4) + sizeof(float2)); }
 
-// The float4 spins, allocated by the first run that takes them (handles that only do Monte Carlo,
-// alternative integrators, short runs or the cluster, persistent and system-block steps never hold
-// their 56 bytes per spin; allocating them takes 0.2 ms).  Without the memory the steps work on the
-// arrays.  Allowed while a stream is captured: nothing is enqueued on it here.
+// The float4 spins, allocated with the handle up to kPackedSmall bytes, else by the first run that takes
+// them: large handles that only do Monte Carlo, alternative integrators, short runs or the persistent
+// step, and small ones that the cluster steps, never hold their 56 bytes per spin.  Allocating takes 0.1 to
+// 0.2 ms whatever the size: of a small handle's first run that is a fifth (eight steps of 242 lattices of
+// 7 x 12 x 7 spins 351 us, 456 with it), of the 1024 x 1024 x 16 film's 2 %.  Without the memory the steps
+// work on the arrays.  Allowed while a stream is captured: nothing is enqueued on it here.
+constexpr size_t kPackedSmall = size_t(64) << 20;
 void ensure_packed(ss_system *h) {
     if (h->packed || h->packed_off) return;
     cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
@@ -1620,6 +1623,9 @@ ss_status create_impl(const ss_params *systems, int32_t count, ss_system **out, 
         cudaGetLastError();  // the control words and records are copied to pageable memory
         h->report = nullptr;
     }
+    // (last: it is done without where the handle's other memory leaves none)
+    if (packed_min(h) != kPackedNever && packed_bytes(h) <= kPackedSmall && (count > 1 || n > kClusterAutoMax))
+        ensure_packed(h);
     owner.h = nullptr;
     *out = h;
     return SS_OK;

@@ -47,7 +47,7 @@ def test_trials_launch_what_runs_launch():
     # however few steps are asked for: the trials run over the float4 spins that runs take
     from paper_1310_6143_gb300.system import SpinSystem
 
-    with SpinSystem(L.film(24, 20, 17), **KW) as s:
+    with SpinSystem(L.film(300, 300, 15), **KW) as s:
         held, ref = s.info()["device_bytes"], s.spins()
         s.autotune(1)
         assert (s.spins() == ref).all() and s.step_index == 0
@@ -55,5 +55,5 @@ def test_trials_launch_what_runs_launch():
         s.set_launch(256, 256)
         now = s.info()["device_bytes"]
         s.set_exec("kernels")
-        s.step(12)
+        s.step(8)
         assert s.info()["device_bytes"] == now > held + 56 * s.n

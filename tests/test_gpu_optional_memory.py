@@ -22,7 +22,7 @@ def env():
 
 
 def _film():
-    return L.film(24, 20, 17)
+    return L.film(300, 300, 15)  # 1.35 M spins: 76 MB of float4 spins, allocated by the first run of 8 steps
 
 
 def _sphere():
@@ -38,19 +38,50 @@ def test_held_by_runs_only(env):
         s.mc_step(2)
         s.semi_implicit_step(5)
         s.midpoint_step(4)
-        s.step(11)  # 8,160 spins with row forms: runs of 12 steps and more
-        s.set_exec("system_blocks")
-        s.step(12)
+        s.step(7)
         s.set_exec("persistent")
-        s.step(12)
+        s.step(8)
         s.set_exec("kernels")
         s.set_row_patterns(False)
-        s.step(12)
+        s.step(8)
         s.set_row_patterns(True)
         assert s.info()["device_bytes"] == held
-        s.step(12)
+        s.step(8)
         assert s.info()["device_bytes"] == held + 56 * s.n
         s.step(8)
+        assert s.info()["device_bytes"] == held + 56 * s.n
+
+
+def test_small_handles_hold_it_from_the_start(env):
+    lib, SS = env
+    out, whole = [], 0
+    base = lib.ss_debug_live_bytes()
+    for short in (False, True):
+        if short:
+            lib.ss_debug_limit_bytes(base + whole - 16)  # done without
+        with SS(L.film(24, 20, 17), **KW) as s:
+            lib.ss_debug_limit_bytes(-1)
+            held = lib.ss_debug_live_bytes() - base
+            whole = whole or held
+            assert (held <= whole - 56 * s.n) == short
+            s.set_exec("kernels")
+            s.step(12)
+            assert lib.ss_debug_live_bytes() - base == held
+            s.set_exec("graph")
+            s.step(130)
+            out.append((s.spins(), s.record(0, 142)))
+    for x, y in zip(*out):
+        np.testing.assert_array_equal(x, y)
+
+
+def test_small_handles_of_the_cluster_do_not(env):
+    lib, SS = env
+    with SS(L.film(13, 10, 12), **KW) as s:  # 1,560 spins
+        s.step(40)
+        s.set_exec("kernels")
+        s.step(11)
+        held = s.info()["device_bytes"]
+        s.step(12)
         assert s.info()["device_bytes"] == held + 56 * s.n
 
 
@@ -156,10 +187,8 @@ def test_longer_runs_equal_single_steps(env, lats):
         with SS(systems, **KW) as s:
             s.set_exec("kernels")
             s.set_launch(block, block * slots)
-            held = s.info()["device_bytes"]
             for k in runs:
                 s.step(k)
-            assert s.info()["device_bytes"] - held == (56 * s.n if len(runs) < steps else 0)
             out = [s.spins()] + [v.cpu().numpy() for v in s.state_device(1)]
         ref = ref or out
         for x, y in zip(out, ref):
